@@ -19,6 +19,7 @@
 #include <thread>
 #include <vector>
 
+#include "band.cuh"
 #include "gsofa.h"
 #include "internal.cuh"
 
@@ -542,6 +543,413 @@ int check_options(const gsofa_options* in, gsofa_options* o) {
   o->collect_stats = in->collect_stats;
   o->validate = in->validate;
   if (o->chunk_size > 1024) return GSOFA_E_INVAL;
+  return GSOFA_OK;
+}
+
+// Pinned host scratch of the calling thread (descriptor uploads, size read-backs
+// of transient batches); reused once the previous call on this thread waited.
+void* thread_pinned(size_t bytes, int slot) {
+  thread_local void* buf[2] = {nullptr, nullptr};
+  thread_local size_t cap[2] = {0, 0};
+  if (cap[slot] < bytes) {
+    if (buf[slot]) cudaFreeHost(buf[slot]);
+    buf[slot] = nullptr;
+    cap[slot] = 0;
+    const size_t want = bytes + (bytes >> 1) + 4096;
+    if (cudaMallocHost(&buf[slot], want) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    cap[slot] = want;
+  }
+  return buf[slot];
+}
+
+// ---------------------------------------------------------------- banded matrices
+// Options that leave the choice of kernel to the library; anything that picks or tunes a
+// traversal kernel, or asks for its work counters, runs the traversal.
+bool band_allowed(const gsofa_options& o) {
+  return o.frontier_order == 0 && o.smem_max_source == 0 && o.threads_per_source == 0 && o.list_capacity == 0 &&
+         o.work_chunk == 0 && o.fill_first == 0 && o.collect_stats != 1 && o.validate != 2 && o.label_bits == 0 &&
+         o.expand_mode == 0 && o.schedule == 0 && o.team_sources == 0 && o.warps_per_sm == 0 && o.host_spill == 0 &&
+         o.clean_heads == 0;
+}
+
+struct BandShape {
+  int C = 0;        // CTAs per matrix (0: the band does not fit on chip)
+  int threads = 0;
+  size_t smem = 0;
+};
+
+// Launch shape for a band of LB words left and UB words right of a row's own.  One matrix
+// (alone) is spread over a cluster once its window is wide enough for the split to pay for
+// the cluster's barriers (us per 32 rows with 1 / 4 / 8 CTAs: LB 3: 1.6 / 2.3 / 2.4, LB 7:
+// 2.3 / 2.2 / 2.4, LB 10: 3.1 / 2.5 / 2.7, LB 33: - / 5.0 / 4.4).  Batches have other
+// matrices to fill the chip with and take the smallest cluster that holds the window.
+BandShape band_shape(int LB, int UB, bool alone) {
+  BandShape s;
+  for (int C = !alone || LB <= 8 ? 1 : (LB <= 16 ? 4 : 8); C <= 8; C *= 2) {
+    const size_t b = band_smem_bytes(LB, UB, C);
+    if (b > BAND_SMEM_MAX - 1024) continue;
+    s.C = C;
+    s.smem = b;
+    break;
+  }
+  if (!s.C) return s;
+  // 14 worker warps: a batch's longest matrix sets its time (512 matrices: 1.28 ms; with 256
+  // threads 1.90, with 128 3.99)
+  s.threads = 512;
+  return s;
+}
+
+// Device memory and results of one banded call (one matrix or a batch).
+struct BandRun {
+  Ctx* c = nullptr;
+  cudaStream_t st = nullptr;
+  BandArgs a;
+  std::vector<BandMat> mats;
+  unsigned char* ctr = nullptr;   // BandCounters | band | mat_tot | nsuper | cross: zeroed together
+  unsigned char* hctr = nullptr;  // pinned copy (all but cross)
+  size_t ctr_bytes = 0, host_bytes = 0;
+  BandMat* d_mats = nullptr;
+  int32_t *nL = nullptr, *nU = nullptr, *flags = nullptr, *fill = nullptr;
+  long long* part = nullptr;
+  uint32_t* bits = nullptr;
+  int64_t *Lrp = nullptr, *Urp = nullptr;
+  int32_t *Lci = nullptr, *Uci = nullptr, *sup = nullptr;
+  int launches = 0;
+
+  const BandCounters* counters() const { return (const BandCounters*)hctr; }
+  int32_t* h_band() const { return (int32_t*)(hctr + 64); }
+  unsigned long long* h_tot() const { return (unsigned long long*)(hctr + 64 + 8 * mats.size()); }
+  int32_t* h_nsuper() const { return (int32_t*)(hctr + 64 + 24 * mats.size()); }
+  void free_scratch() {
+    pfree(ctr, st); pfree(d_mats, st); pfree(nL, st); pfree(nU, st); pfree(flags, st);
+    pfree(part, st); pfree(bits, st);
+  }
+  void free_results() {
+    pfree(fill, st); pfree(Lrp, st); pfree(Urp, st); pfree(Lci, st); pfree(Uci, st); pfree(sup, st);
+  }
+};
+
+// Lay out the matrices, check them and measure their bands (one wait).
+int band_measure(BandRun& b, const gsofa_options& o) {
+  Ctx* c = b.c;
+  cudaStream_t st = b.st;
+  const size_t B = b.mats.size();
+  BandArgs& a = b.a;
+  std::memset(&a, 0, sizeof(a));
+  a.chunk = o.chunk_size;
+  a.group_rows = o.chunk_size * ((127 + o.chunk_size) / o.chunk_size);
+  int64_t rows = 0, groups = 0;
+  for (BandMat& m : b.mats) {
+    m.row_base = rows;
+    m.group_base = groups;
+    rows += m.n;
+    groups += ((int64_t)m.n + a.group_rows - 1) / a.group_rows;
+  }
+  if (rows > INT32_MAX - 1024) return GSOFA_E_NOMEM;
+  a.nmats = (int32_t)B;
+  a.one = b.mats[0];
+  a.rows = rows;
+  a.groups = groups;
+  const size_t cross_words = B == 1 ? (size_t)rows / 1024 + 2 : 0;
+  b.host_bytes = 64 + 28 * B;
+  b.ctr_bytes = ((b.host_bytes + 15) & ~(size_t)15) + 4 * cross_words;
+  b.hctr = (unsigned char*)thread_pinned(b.host_bytes, 1);
+  if (!b.hctr) return GSOFA_E_NOMEM;
+  if (palloc(c, &b.ctr, b.ctr_bytes, st) != cudaSuccess || palloc(c, &b.fill, (size_t)rows, st) != cudaSuccess ||
+      (B > 1 && palloc(c, &b.d_mats, B, st) != cudaSuccess)) {
+    cudaGetLastError();
+    return GSOFA_E_NOMEM;
+  }
+  if (cudaMemsetAsync(b.ctr, 0, b.ctr_bytes, st) != cudaSuccess) return GSOFA_E_CUDA;
+  if (B > 1) {
+    void* stage = thread_pinned(sizeof(BandMat) * B, 0);
+    if (!stage) return GSOFA_E_NOMEM;
+    std::memcpy(stage, b.mats.data(), sizeof(BandMat) * B);
+    if (cudaMemcpyAsync(b.d_mats, stage, sizeof(BandMat) * B, cudaMemcpyHostToDevice, st) != cudaSuccess)
+      return GSOFA_E_CUDA;
+    a.mats = b.d_mats;
+  }
+  a.ctr = (BandCounters*)b.ctr;
+  a.band = (int32_t*)(b.ctr + 64);
+  a.mat_tot = B > 1 ? (unsigned long long*)(b.ctr + 64 + 8 * B) : nullptr;
+  a.mat_nsuper = (int32_t*)(b.ctr + 64 + 24 * B);
+  a.cross = cross_words ? (uint32_t*)(b.ctr + ((b.host_bytes + 15) & ~(size_t)15)) : nullptr;
+  a.fill = b.fill;
+  if (launch_band_scan(a, st) != cudaSuccess) return GSOFA_E_CUDA;
+  b.launches++;
+  if (cudaMemcpyAsync(b.hctr, b.ctr, 64 + 8 * B, cudaMemcpyDeviceToHost, st) != cudaSuccess) return GSOFA_E_CUDA;
+  return wait_stream(st);
+}
+
+// Bitmap words of all matrices once their bands are known; -1 where one does not fit on chip.
+int64_t band_layout(BandRun& b) {
+  int64_t words = 0;
+  for (size_t m = 0; m < b.mats.size(); m++) {
+    BandMat& d = b.mats[m];
+    d.LB = (b.h_band()[2 * m] + 31) / 32;
+    d.UB = (b.h_band()[2 * m + 1] + 31) / 32;
+    if (!band_shape(d.LB, d.UB, false).C) return -1;
+    d.bits_base = words;
+    words += (int64_t)d.n * (d.LB + d.UB + 1);
+  }
+  return words;
+}
+
+// Elimination, counts, and (after one wait) the results.  Consumes a measured and laid out run.
+int band_run(BandRun& b, int64_t words, Events& ev) {
+  Ctx* c = b.c;
+  cudaStream_t st = b.st;
+  BandArgs& a = b.a;
+  const size_t B = b.mats.size(), N = (size_t)a.rows;
+  if (palloc(c, &b.bits, (size_t)words, st) != cudaSuccess || palloc(c, &b.nL, N, st) != cudaSuccess ||
+      palloc(c, &b.nU, N, st) != cudaSuccess || palloc(c, &b.flags, N, st) != cudaSuccess ||
+      palloc(c, &b.part, 3 * (size_t)a.groups, st) != cudaSuccess) {
+    cudaGetLastError();
+    return GSOFA_E_NOMEM;
+  }
+  a.bits = b.bits;
+  a.row_nL = b.nL;
+  a.row_nU = b.nU;
+  a.flags = b.flags;
+  a.part = b.part;
+  a.one = b.mats[0];
+  cudaError_t e = cudaSuccess;
+  if (B > 1) {
+    void* stage = thread_pinned(sizeof(BandMat) * B, 0);
+    std::memcpy(stage, b.mats.data(), sizeof(BandMat) * B);
+    e = cudaMemcpyAsync(b.d_mats, stage, sizeof(BandMat) * B, cudaMemcpyHostToDevice, st);
+  }
+  ev.rec(2, st);
+  if (B == 1) {
+    const BandShape s = band_shape(a.one.LB, a.one.UB, true);
+    const int panels = (a.one.n + 31) / 32;
+    const int parts = std::max(1, std::min(panels, c->sms / s.C));
+    if (e == cudaSuccess) e = launch_band_elim(a, parts, s.C, s.threads, s.smem, st);
+    b.launches++;
+  } else {
+    // matrices are sorted by shape: one launch per cluster size
+    for (size_t m = 0; m < B && e == cudaSuccess;) {
+      const int C = band_shape(b.mats[m].LB, b.mats[m].UB, false).C;
+      int threads = 0;
+      size_t smem = 0, k = m;
+      for (; k < B; k++) {
+        const BandShape s = band_shape(b.mats[k].LB, b.mats[k].UB, false);
+        if (s.C != C) break;
+        threads = std::max(threads, s.threads);
+        smem = std::max(smem, s.smem);
+      }
+      a.first = (int32_t)m;
+      e = launch_band_elim(a, (int)(k - m), C, threads, smem, st);
+      b.launches++;
+      m = k;
+    }
+  }
+  ev.rec(3, st);
+  if (e == cudaSuccess) e = launch_band_count(a, st);
+  b.launches++;
+  ev.rec(4, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(b.hctr, b.ctr, b.host_bytes, cudaMemcpyDeviceToHost, st);
+  if (e != cudaSuccess) return GSOFA_E_CUDA;
+  const int rc = wait_stream(st);
+  if (rc) return rc;
+  const BandCounters& h = *b.counters();
+  if (palloc(c, &b.Lrp, N + B, st) != cudaSuccess || palloc(c, &b.Urp, N + B, st) != cudaSuccess ||
+      palloc(c, &b.Lci, (size_t)h.total_L, st) != cudaSuccess || palloc(c, &b.Uci, (size_t)h.total_U, st) != cudaSuccess ||
+      palloc(c, &b.sup, (size_t)h.n_super + B, st) != cudaSuccess) {
+    cudaGetLastError();
+    return GSOFA_E_NOMEM;
+  }
+  a.L_rowptr = b.Lrp;
+  a.U_rowptr = b.Urp;
+  a.L_colidx = b.Lci;
+  a.U_colidx = b.Uci;
+  a.super_start = b.sup;
+  if (launch_band_expand(a, st) != cudaSuccess) return GSOFA_E_CUDA;
+  b.launches++;
+  ev.rec(5, st);
+  return GSOFA_OK;
+}
+
+void band_times(Events& ev, gsofa_stats* s) {
+  s->ms_validate = ev.ms(0, 1);
+  s->ms_traverse = s->ms_traverse_global = ev.ms(2, 3);
+  s->ms_supernode = ev.ms(3, 4);
+  s->ms_emit = ev.ms(4, 5);
+  s->ms_total = ev.ms(0, 5);
+}
+
+// One matrix by band elimination.  *taken: the band fits on chip and the call is done
+// (whatever it returns); otherwise nothing is left behind and the traversal runs.
+int run_band_single(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gsofa_options& o, cudaStream_t st,
+                    gsofa_result* out, bool* taken) {
+  *taken = false;
+  zero_result(out);
+  out->err_detail = -1;
+  Events ev;
+  ev.create(o.collect_stats != 0);
+  ev.rec(0, st);
+  BandRun b;
+  b.c = c;
+  b.st = st;
+  BandMat m;
+  std::memset(&m, 0, sizeof(m));
+  m.rowptr = rp;
+  m.colidx = ci;
+  m.n = n;
+  b.mats.push_back(m);
+  int rc = band_measure(b, o);
+  ev.rec(1, st);
+  int64_t words = -1;
+  if (rc == GSOFA_OK) {
+    if (b.counters()->err) {
+      rc = GSOFA_E_INVAL;
+      out->err_detail = b.counters()->bad_row ? INT_MAX - b.counters()->bad_row : -1;
+    } else {
+      words = band_layout(b);
+      if (words >= 0) rc = band_run(b, words, ev);
+    }
+  }
+  b.free_scratch();
+  if (rc != GSOFA_OK || words < 0) {
+    if (rc == GSOFA_E_TIMEOUT || rc == GSOFA_E_CUDA) wait_stream(st);
+    cudaGetLastError();
+    b.free_results();
+    *taken = rc != GSOFA_OK;
+    return rc;
+  }
+  *taken = true;
+  const BandCounters h = *b.counters();
+  Priv* pv = new Priv();
+  pv->stream = st;
+  pv->device = c->device;
+  pv->mpool = c->mpool;
+  out->_priv = pv;
+  out->n = n;
+  out->on_device = 1;
+  out->nnz_L = (int64_t)h.total_L;
+  out->nnz_U = (int64_t)h.total_U;
+  out->n_super = h.n_super;
+  out->L_rowptr = b.Lrp;
+  out->U_rowptr = b.Urp;
+  out->L_colidx = b.Lci;
+  out->U_colidx = b.Uci;
+  out->fill_count = b.fill;
+  out->super_start = b.sup;
+  out->stats.kernel_launches = b.launches;
+  out->stats.traverse_launches = 1;
+  out->stats.levels = (n + 31) / 32;
+  if (o.collect_stats) {
+    rc = wait_stream(st);
+    if (rc) {
+      gsofa_free(out);
+      return rc;
+    }
+    band_times(ev, &out->stats);
+  }
+  return GSOFA_OK;
+}
+
+// The matrices idx of a batch (all of order > 0) by band elimination; `rest` receives those
+// whose band does not fit on chip.  Results share one block.
+int run_band_batch(Ctx* c, const std::vector<int32_t>& idx, const int32_t* n, const int32_t* const* rp,
+                   const int32_t* const* ci, const gsofa_options& o, cudaStream_t st, gsofa_result* outs,
+                   int* launches, std::vector<int32_t>* rest) {
+  rest->clear();
+  std::vector<int32_t> order(idx);
+  // largest first: the last CTAs to start are the shortest
+  std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) { return n[x] > n[y]; });
+  Events ev;
+  ev.create(o.collect_stats != 0);
+  for (int pass = 0; pass < 3 && !order.empty(); pass++) {
+    BandRun b;
+    b.c = c;
+    b.st = st;
+    for (int32_t k : order) {
+      BandMat m;
+      std::memset(&m, 0, sizeof(m));
+      m.rowptr = rp[k];
+      m.colidx = ci[k];
+      m.n = n[k];
+      b.mats.push_back(m);
+    }
+    ev.rec(0, st);
+    int rc = band_measure(b, o);
+    ev.rec(1, st);
+    int64_t words = -1;
+    if (rc == GSOFA_OK && b.counters()->err) rc = GSOFA_E_INVAL;
+    if (rc == GSOFA_OK) {
+      // by cluster size, those that do not fit apart
+      std::vector<int32_t> next;
+      std::vector<int> size(order.size());
+      bool sorted = true;
+      for (size_t m = 0; m < order.size(); m++) {
+        size[m] = band_shape((b.h_band()[2 * m] + 31) / 32, (b.h_band()[2 * m + 1] + 31) / 32, false).C;
+        if (size[m] == 0) rest->push_back(order[m]);
+        if (size[m] == 0 || (m && size[m] < size[m - 1])) sorted = false;
+      }
+      for (int C = 1; C <= 8; C *= 2)
+        for (size_t m = 0; m < order.size(); m++)
+          if (size[m] == C) next.push_back(order[m]);
+      if (!sorted) {  // lay the batch out again without them, in launch order
+        b.free_scratch();
+        b.free_results();
+        *launches += b.launches;
+        order.swap(next);
+        continue;
+      }
+      words = band_layout(b);
+      rc = words < 0 ? GSOFA_E_CUDA : band_run(b, words, ev);
+    }
+    b.free_scratch();
+    *launches += b.launches;
+    if (rc != GSOFA_OK) {
+      if (rc != GSOFA_E_INVAL) wait_stream(st);
+      cudaGetLastError();
+      b.free_results();
+      return rc;
+    }
+    SharedBlock* blk = new SharedBlock();
+    blk->stream = st;
+    blk->device = c->device;
+    for (void* q : {(void*)b.Lrp, (void*)b.Urp, (void*)b.Lci, (void*)b.Uci, (void*)b.sup, (void*)b.fill})
+      blk->ptrs.push_back(q);
+    blk->refs.store((int)order.size());
+    int64_t offL = 0, offU = 0, offS = 0;
+    for (size_t k = 0; k < order.size(); k++) {
+      gsofa_result* r = &outs[order[k]];
+      zero_result(r);
+      Priv* pv = new Priv();
+      pv->stream = st;
+      pv->device = c->device;
+      pv->shared = blk;
+      r->_priv = pv;
+      r->n = n[order[k]];
+      r->on_device = 1;
+      r->err_detail = -1;
+      const bool alone = order.size() == 1;
+      r->nnz_L = alone ? (int64_t)b.counters()->total_L : (int64_t)b.h_tot()[2 * k];
+      r->nnz_U = alone ? (int64_t)b.counters()->total_U : (int64_t)b.h_tot()[2 * k + 1];
+      r->n_super = alone ? b.counters()->n_super : b.h_nsuper()[k];
+      r->L_rowptr = b.Lrp + b.mats[k].row_base + k;
+      r->U_rowptr = b.Urp + b.mats[k].row_base + k;
+      r->L_colidx = b.Lci + offL;
+      r->U_colidx = b.Uci + offU;
+      r->fill_count = b.fill + b.mats[k].row_base;
+      r->super_start = b.sup + offS;
+      offL += r->nnz_L;
+      offU += r->nnz_U;
+      offS += r->n_super + 1;
+    }
+    if (o.collect_stats) {
+      rc = wait_stream(st);
+      if (rc) return rc;
+      band_times(ev, &outs[order[0]].stats);
+    }
+    return GSOFA_OK;
+  }
   return GSOFA_OK;
 }
 
@@ -1136,25 +1544,6 @@ int set_shape(Ctx* c, BatchPlan* p, const LaunchShape& sh) {
   return GSOFA_OK;
 }
 
-// Pinned host scratch of the calling thread (descriptor uploads, size read-backs
-// of transient batches); reused once the previous call on this thread waited.
-void* thread_pinned(size_t bytes, int slot) {
-  thread_local void* buf[2] = {nullptr, nullptr};
-  thread_local size_t cap[2] = {0, 0};
-  if (cap[slot] < bytes) {
-    if (buf[slot]) cudaFreeHost(buf[slot]);
-    buf[slot] = nullptr;
-    cap[slot] = 0;
-    const size_t want = bytes + (bytes >> 1) + 4096;
-    if (cudaMallocHost(&buf[slot], want) != cudaSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    cap[slot] = want;
-  }
-  return buf[slot];
-}
-
 int build_plan(Ctx* c, const std::vector<int32_t>& members, const int32_t* n, const int32_t* const* rp,
                const int32_t* const* ci, const gsofa_options& o, uint64_t sig, BatchPlan** out,
                bool transient, cudaStream_t st, int64_t pool_entries = 0) {
@@ -1579,16 +1968,28 @@ int run_batch(Ctx* c, int32_t count, const int32_t* n, const int32_t* const* rp,
     idx[k] = k;
   }
   std::vector<int32_t> members, singles;
-  for (int32_t k = 0; k < count; k++) {
+  int launches = 0;
+  int rc = GSOFA_OK;
+  std::vector<char> done(count, 0);
+  if (band_allowed(o)) {
+    std::vector<int32_t> some, rest;
+    for (int32_t k = 0; k < count; k++)
+      if (n[k] > 0) some.push_back(k);
+    rc = run_band_batch(c, some, n, rp, ci, o, st, outs, &launches, &rest);
+    if (rc == GSOFA_OK) {
+      for (int32_t k : some) done[k] = 1;
+      for (int32_t k : rest) done[k] = 0;
+    }
+  }
+  for (int32_t k = 0; rc == GSOFA_OK && k < count; k++) {
+    if (done[k]) continue;
     const int32_t nk = n[k];
     if (nk == 0) { singles.push_back(k); continue; }
     const int l16 = nk <= 65533 ? 1 : 0;
     if (o.smem_max_source == 0 && trav_smem_max_S(nk, limit, l16) >= nk) members.push_back(k);
     else singles.push_back(k);
   }
-  int launches = 0;
-  int rc = GSOFA_OK;
-  if (!members.empty())
+  if (rc == GSOFA_OK && !members.empty())
     rc = run_batch_members(c, members, n, rp, ci, o, st, outs, &launches, transient, pool_entries);
   for (size_t j = 0; rc == GSOFA_OK && j < singles.size(); j++) {
     const int32_t k = singles[j];
@@ -1764,6 +2165,12 @@ namespace {
 // Autotune reads nnz (device input: one read) and keeps its choice per (n, nnz).
 int run_single(Ctx* c, int32_t n, const int32_t* d_rowptr, const int32_t* d_colidx, gsofa_options o,
                cudaStream_t st, gsofa_result* out, int64_t nnz_known) {
+  if (n > 0 && band_allowed(o)) {
+    bool taken = false;
+    const int rc = run_band_single(c, n, d_rowptr, d_colidx, o, st, out, &taken);
+    if (taken) return rc;
+    o.validate = 2;  // checked above
+  }
   const bool tune = o.autotune && o.frontier_order == 0 && n > 0;
   if (o.frontier_order == 0 && !tune) {
     // class order for every source (the fewest expansions and the fastest on

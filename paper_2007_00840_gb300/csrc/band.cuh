@@ -1,0 +1,58 @@
+// Banded path (band.cu): descriptors and launchers.
+#pragma once
+
+#include "internal.cuh"
+
+namespace gsofa {
+
+constexpr int BAND_SMEM_MAX = 227 * 1024;
+constexpr int BAND_REACH_MAX = 8192;  // above the widest band that eight CTAs hold
+
+// Counters of one call.
+struct BandCounters {
+  unsigned long long total_L, total_U;
+  int32_t err;          // ERR_* bits
+  int32_t bad_row;      // INT_MAX - first offending row (0: none)
+  int32_t n_super;
+  int32_t groups_done;
+};
+
+// One matrix.  LB, UB: words of columns left and right of a row's own word that the band reaches.
+struct BandMat {
+  const int32_t* rowptr;
+  const int32_t* colidx;
+  int64_t row_base;    // first row in the concatenated per-row arrays
+  int64_t group_base;  // first row group
+  int64_t bits_base;   // first word of its bitmap rows (LB + UB + 1 words each)
+  int32_t n, LB, UB, pad;
+};
+
+struct BandArgs {
+  const BandMat* mats;  // null: one matrix, `one`
+  BandMat one;
+  int32_t nmats;
+  int32_t first;        // elimination: first matrix of this launch
+  int64_t rows;         // rows of all matrices
+  int64_t groups;       // row groups of all matrices
+  int32_t chunk;        // rows per supernode chunk
+  int32_t group_rows;   // rows per group: a multiple of chunk
+  BandCounters* ctr;
+  int32_t* band;        // per matrix: largest i - j, largest j - i
+  uint32_t* cross;      // one matrix: bit q set where an entry below the diagonal crosses row 32q (null: batch)
+  uint32_t* bits;
+  int32_t *row_nL, *row_nU, *fill, *flags;
+  long long* part;      // per group: [nnz(L), nnz(U), supernodes], then exclusive sums
+  unsigned long long* mat_tot;  // per matrix [nnz(L), nnz(U)] (null: one matrix)
+  int32_t* mat_nsuper;
+  int64_t *L_rowptr, *U_rowptr;
+  int32_t *L_colidx, *U_colidx, *super_start;
+};
+
+size_t band_smem_bytes(int LB, int UB, int C);
+cudaError_t launch_band_scan(const BandArgs& a, cudaStream_t st);
+// `count` matrices from a.first on, or the parts one matrix's panels are dealt to: C CTAs (a cluster) each.
+cudaError_t launch_band_elim(const BandArgs& a, int count, int C, int threads, size_t smem, cudaStream_t st);
+cudaError_t launch_band_count(const BandArgs& a, cudaStream_t st);
+cudaError_t launch_band_expand(const BandArgs& a, cudaStream_t st);
+
+}  // namespace gsofa
