@@ -575,33 +575,6 @@ bool band_allowed(const gsofa_options& o) {
          o.clean_heads == 0;
 }
 
-struct BandShape {
-  int C = 0;        // CTAs per matrix (0: the band does not fit on chip)
-  int threads = 0;
-  size_t smem = 0;
-};
-
-// Launch shape for a band of LB words left and UB words right of a row's own.  One matrix
-// (alone) is spread over a cluster once its window is wide enough for the split to pay for
-// the cluster's barriers (us per 32 rows with 1 / 4 / 8 CTAs: LB 3: 1.6 / 2.3 / 2.4, LB 7:
-// 2.3 / 2.2 / 2.4, LB 10: 3.1 / 2.5 / 2.7, LB 33: - / 5.0 / 4.4).  Batches have other
-// matrices to fill the chip with and take the smallest cluster that holds the window.
-BandShape band_shape(int LB, int UB, bool alone) {
-  BandShape s;
-  for (int C = !alone || LB <= 8 ? 1 : (LB <= 16 ? 4 : 8); C <= 8; C *= 2) {
-    const size_t b = band_smem_bytes(LB, UB, C);
-    if (b > BAND_SMEM_MAX - 1024) continue;
-    s.C = C;
-    s.smem = b;
-    break;
-  }
-  if (!s.C) return s;
-  // 14 worker warps: a batch's longest matrix sets its time (512 matrices: 1.28 ms; with 256
-  // threads 1.90, with 128 3.99)
-  s.threads = 512;
-  return s;
-}
-
 // Device memory and results of one banded call (one matrix or a batch).
 struct BandRun {
   Ctx* c = nullptr;

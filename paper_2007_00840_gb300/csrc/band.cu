@@ -617,7 +617,7 @@ __global__ void __launch_bounds__(512, 1) band_elim_kernel(BandArgs a) {
         }
         {
           // finished rows out; their slot is zeroed for the panel that takes it
-          if (P % C == rank) {
+          if (P % C == rank && a.bits) {
             const int rows = min(32, B.n - 32 * P);
             uint32_t* x = panel_rows<C>(B, P);
             uint32_t* o = out + (size_t)32 * P * wx;
@@ -632,6 +632,25 @@ __global__ void __launch_bounds__(512, 1) band_elim_kernel(BandArgs a) {
               if (c2 >= wx) {
                 c2 -= wx;
                 r2++;
+              }
+            }
+          } else if (P % C == rank) {  // sizes alone
+            for (int r2 = warp - 1; r2 < 32; r2 += nwk) {
+              uint32_t* row = panel_rows<C>(B, P) + r2 * B.xs;
+              const int i = 32 * P + r2;
+              int l = 0, u = 0;
+              for (int c2 = lane; c2 < wx; c2 += 32) {
+                if (c2 < B.LB) l += __popc(row[c2]);
+                else if (c2 > B.LB) u += __popc(pu[r2 * B.us + c2 - B.LB - 1]);
+                row[c2] = 0u;
+              }
+              const uint32_t w = S.pw[32 * (P & 1) + r2];
+              l = __reduce_add_sync(FULL, l) + __popc(w & lt_mask(r2));
+              u = __reduce_add_sync(FULL, u) + __popc(w & gt_mask(r2)) + 1;
+              if (lane == 0 && i < B.n) {
+                a.row_nL[i] = l;
+                a.row_nU[i] = u;
+                a.fill[i] = l + u - a.fill[i];
               }
             }
           }
@@ -866,6 +885,27 @@ size_t band_smem_bytes(int LB, int UB, int C) {
   const int wx = LB + UB + 1;
   const size_t slots = (size_t)(LB + 2 + C - 1) / C;
   return 4 * (128 + 64 + 68 + 192 * (size_t)(UB | 1) + 4 * BAND_STAGE + slots * 32 * (size_t)((wx | 1) + 1));
+}
+
+// Launch shape for a band of LB words left and UB words right of a row's own.  One matrix
+// (alone) is spread over a cluster once its window is wide enough for the split to pay for
+// the cluster's barriers (us per 32 rows with 1 / 4 / 8 CTAs: LB 3: 1.6 / 2.3 / 2.4, LB 7:
+// 2.3 / 2.2 / 2.4, LB 10: 3.1 / 2.5 / 2.7, LB 33: - / 5.0 / 4.4).  Batches have other
+// matrices to fill the chip with and take the smallest cluster that holds the window.
+BandShape band_shape(int LB, int UB, bool alone) {
+  BandShape s;
+  for (int C = !alone || LB <= 8 ? 1 : (LB <= 16 ? 4 : 8); C <= 8; C *= 2) {
+    const size_t b = band_smem_bytes(LB, UB, C);
+    if (b > BAND_SMEM_MAX - 1024) continue;
+    s.C = C;
+    s.smem = b;
+    break;
+  }
+  if (!s.C) return s;
+  // 14 worker warps: a batch's longest matrix sets its time (512 matrices: 1.28 ms; with 256
+  // threads 1.90, with 128 3.99)
+  s.threads = 512;
+  return s;
 }
 
 cudaError_t launch_band_scan(const BandArgs& a, cudaStream_t st) {

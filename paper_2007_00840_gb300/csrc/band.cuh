@@ -39,7 +39,7 @@ struct BandArgs {
   BandCounters* ctr;
   int32_t* band;        // per matrix: largest i - j, largest j - i
   uint32_t* cross;      // one matrix: bit q set where an entry below the diagonal crosses row 32q (null: batch)
-  uint32_t* bits;
+  uint32_t* bits;       // null (one matrix): per-row sizes and fill counts only
   int32_t *row_nL, *row_nU, *fill, *flags;
   long long* part;      // per group: [nnz(L), nnz(U), supernodes], then exclusive sums
   unsigned long long* mat_tot;  // per matrix [nnz(L), nnz(U)] (null: one matrix)
@@ -49,6 +49,14 @@ struct BandArgs {
 };
 
 size_t band_smem_bytes(int LB, int UB, int C);
+struct BandShape {
+  int C = 0;  // CTAs per matrix (0: the band does not fit on chip)
+  int threads = 0;
+  size_t smem = 0;
+};
+// Launch shape for a band of LB words left and UB words right of a row's own; alone: one
+// matrix has the device.
+BandShape band_shape(int LB, int UB, bool alone);
 cudaError_t launch_band_scan(const BandArgs& a, cudaStream_t st);
 // `count` matrices from a.first on, or the parts one matrix's panels are dealt to: C CTAs (a cluster) each.
 cudaError_t launch_band_elim(const BandArgs& a, int count, int C, int threads, size_t smem, cudaStream_t st);

@@ -12,6 +12,7 @@
 #include <cstring>
 #include <mutex>
 
+#include "band.cuh"
 #include "gsofa.h"
 #include "internal.cuh"
 
@@ -19,6 +20,7 @@ namespace gsofa {
 namespace {
 
 static_assert(GSOFA_NOALLOC_SCRATCH_BYTES >= 4096, "scratch too small");
+static_assert(sizeof(BandCounters) <= 64, "counters of the banded path");
 static_assert(sizeof(DevCounters) <= 256, "the counters block must fit ahead of the overflow lists");
 
 // Scratch of this entry point: [0, 256) counters, then frontier overflow lists.
@@ -71,6 +73,42 @@ extern "C" int gsofa_row_counts_noalloc(int32_t n, const int32_t* d_rowptr, cons
   DevCounters* ctr = (DevCounters*)base;
   int32_t* spill = (int32_t*)((unsigned char*)base + 256);
   const size_t spill_bytes = GSOFA_NOALLOC_SCRATCH_BYTES - 256;
+
+  // a band that fits on chip: its sizes come from the elimination (27x25x29 grid: 27.1 ms
+  // by the traversal below), whose scratch is the counters and one bit per 32 rows
+  if (n > 0) {
+    BandArgs b;
+    memset(&b, 0, sizeof(b));
+    unsigned char* p = (unsigned char*)base;
+    const size_t cross_bytes = 4 * ((size_t)n / 1024 + 2);
+    b.ctr = (BandCounters*)p;
+    b.band = (int32_t*)(p + 64);
+    b.cross = (uint32_t*)(p + 128);
+    b.nmats = 1;
+    b.one.rowptr = d_rowptr;
+    b.one.colidx = d_colidx;
+    b.one.n = n;
+    b.rows = n;
+    b.fill = d_fill_count;
+    b.row_nL = d_nnzL;
+    b.row_nU = d_nnzU;
+    if (cudaMemsetAsync(p, 0, 128 + cross_bytes, st) != cudaSuccess) return GSOFA_E_CUDA;
+    if (launch_band_scan(b, st) != cudaSuccess) return GSOFA_E_CUDA;
+    struct { BandCounters c; unsigned char pad[64 - sizeof(BandCounters)]; int32_t band[2]; } m;
+    if (cudaMemcpyAsync(&m, p, sizeof(m), cudaMemcpyDeviceToHost, st) != cudaSuccess) return GSOFA_E_CUDA;
+    rc = wait_stream(st);
+    if (rc) return rc;
+    if (m.c.err) return GSOFA_E_INVAL;
+    b.one.LB = (m.band[0] + 31) / 32;
+    b.one.UB = (m.band[1] + 31) / 32;
+    const BandShape s = band_shape(b.one.LB, b.one.UB, true);
+    if (s.C) {
+      const int panels = (n + 31) / 32, most = sms / s.C;
+      if (launch_band_elim(b, panels < most ? panels : most, s.C, s.threads, s.smem, st) != cudaSuccess)
+        return GSOFA_E_CUDA;
+      return wait_stream(st);
+    }
+  }
 
   // every source in the shared-memory tier with 16-bit maxId labels
   const int label16 = 1;
