@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "band.cuh"
+#include "fronts.cuh"
 #include "gsofa.h"
 #include "internal.cuh"
 
@@ -754,8 +755,362 @@ void band_times(Events& ev, gsofa_stats* s) {
   s->ms_total = ev.ms(0, 5);
 }
 
-// One matrix by band elimination.  *taken: the band fits on chip and the call is done
-// (whatever it returns); otherwise nothing is left behind and the traversal runs.
+// ---------------------------------------------------------------- nested dissection
+// Orders from which the blocks of a dissection are looked for (below, the traversal takes
+// about as long as the search), and up to which what remains is one front.
+constexpr int32_t FRONT_MIN_ORDER = 16384;
+constexpr int32_t FRONT_LAST_ORDER = 2900;
+
+// Pool memory of one call, freed together.
+struct Held {
+  Ctx* c;
+  cudaStream_t st;
+  std::vector<void*> ptrs;
+  bool ok = true;
+  template <typename T>
+  T* get(size_t count) {
+    T* p = nullptr;
+    if (!ok || palloc(c, &p, count, st) != cudaSuccess) {
+      cudaGetLastError();
+      ok = false;
+      return nullptr;
+    }
+    ptrs.push_back(p);
+    return p;
+  }
+  void free_all() {
+    for (void* p : ptrs) cudaFreeAsync(p, st);
+    ptrs.clear();
+  }
+  ~Held() { free_all(); }
+};
+
+// One matrix by elimination of its dissection blocks (fronts.cu).  The CSR has been
+// checked; fill holds every row's entries of A (diagonal counted) and becomes the result's
+// fill counts.  *taken: done (whatever it returns); otherwise the pattern is not ordered
+// for it, or memory ran out, and nothing is left behind but fill as it was.
+int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gsofa_options& o, cudaStream_t st,
+               int32_t* fill, gsofa_result* out, Events& ev, int* launches, bool* taken) {
+  *taken = false;
+  Held keep{c, st}, level_mem{c, st}, next_mem{c, st};
+  const int32_t pcap = n > (1 << 27) ? 0 : 4 * n + 1024;
+  if (!pcap) return GSOFA_OK;
+  FrontLevel l;
+  std::memset(&l, 0, sizeof(l));
+  l.own = keep.get<int32_t>(n);
+  l.own_row = keep.get<int32_t>(n);
+  l.head = keep.get<int32_t>(n);
+  l.npieces = keep.get<int32_t>(n);
+  l.piece_next = keep.get<int32_t>(pcap);
+  l.piece_blk = keep.get<int32_t>(pcap);
+  l.piece_row = keep.get<int32_t>(pcap);
+  l.piece_cap = pcap;
+  int32_t* gid0 = keep.get<int32_t>(n);
+  if (!keep.ok) return GSOFA_OK;
+#define FK(x)                                    \
+  do {                                           \
+    if ((x) != cudaSuccess) return GSOFA_E_CUDA; \
+  } while (0)
+  FK(cudaMemsetAsync(l.head, 0xFF, 4 * (size_t)n, st));
+  FK(cudaMemsetAsync(l.npieces, 0, 4 * (size_t)n, st));
+  FK(launch_front_iota(gid0, n, st));
+  l.n = n;
+  l.beg = rp;
+  l.end = rp + 1;
+  l.col = ci;
+  l.gid = gid0;
+  std::vector<FrontBlock> blocks;
+  ev.rec(2, st);
+  for (int level = 0; level < 16; level++) {
+    std::vector<FrontMat> fronts;
+    const bool whole = l.n <= FRONT_LAST_ORDER;
+    int32_t n1 = 0, br_total = 0;
+    int64_t room = 0;
+    int32_t* bcg = nullptr;
+    if (whole) {
+      const int rc = wait_stream(st);  // the staging buffers are free
+      if (rc) return rc;
+      FK(launch_front_whole(l, st));
+      *launches += 1;
+      FrontMat m;
+      std::memset(&m, 0, sizeof(m));
+      m.sz = l.n;
+      fronts.push_back(m);
+    } else {
+      const size_t nl = (size_t)l.n;
+      const int32_t cap = l.n / FRONT_BLOCK_MIN + 1;
+      l.cap = cap;
+      l.low = level_mem.get<int32_t>(nl);
+      l.best = level_mem.get<int32_t>(nl);
+      l.blk = level_mem.get<int32_t>(nl);
+      l.rem = level_mem.get<int32_t>(nl);
+      l.bound = level_mem.get<int32_t>(nl);
+      int64_t* rank = level_mem.get<int64_t>(nl + 1);
+      int64_t* rooms = level_mem.get<int64_t>(nl + 1);
+      void* tmp = level_mem.get<unsigned char>(scan_tmp_bytes(l.n));
+      // counters and block arrays in one piece: one copy brings back what the host needs
+      int32_t* blk7 = level_mem.get<int32_t>(16 + 7 * (size_t)cap);
+      l.br_cap = 2 * l.n + 1024;
+      l.br_row = level_mem.get<int32_t>(l.br_cap);
+      l.br_b = level_mem.get<int32_t>(l.br_cap);
+      l.br_e = level_mem.get<int32_t>(l.br_cap);
+      l.bc_cap = l.n + 1024;
+      l.bc = level_mem.get<int32_t>(l.bc_cap);
+      bcg = keep.get<int32_t>(l.bc_cap);
+      if (!level_mem.ok || !keep.ok) return GSOFA_OK;
+      l.ctr = (FrontCounters*)blk7;
+      int32_t* q = blk7 + 16;
+      l.b_first = q; l.b_size = q + cap; l.b_nr = q + 2 * (size_t)cap; l.b_nb = q + 3 * (size_t)cap;
+      l.b_br = q + 4 * (size_t)cap; l.b_bc = q + 5 * (size_t)cap; l.b_fill = q + 6 * (size_t)cap;
+      FK(cudaMemsetAsync(blk7, 0, 4 * (16 + 7 * (size_t)cap), st));
+      FK(cudaMemsetAsync(l.low, 0x7F, 4 * nl, st));
+      FK(cudaMemsetAsync(l.best, 0xFF, 4 * nl, st));
+      FK(cudaMemsetAsync(l.blk, 0xFF, 4 * nl, st));
+      FK(cudaMemsetAsync(l.bound, 0, 4 * nl, st));
+      FK(launch_fill_i32(l.rem, l.n, 1, st));
+      FK(launch_front_blocks(l, st));
+      FK(launch_scan_i32_i64(l.rem, rank, l.n, tmp, st));
+      FK(launch_front_above(l, st));
+      FK(launch_scan_i32_i64(l.bound, rooms, l.n, tmp, st));
+      *launches += 16;
+      l.rank = rank;
+      l.room = rooms;
+      const size_t hb = 4 * (16 + 6 * (size_t)cap);
+      unsigned char* h = (unsigned char*)thread_pinned(hb + 16, 1);
+      if (!h) return GSOFA_OK;
+      FK(cudaMemcpyAsync(h, rank + nl, 8, cudaMemcpyDeviceToHost, st));
+      FK(cudaMemcpyAsync(h + 8, rooms + nl, 8, cudaMemcpyDeviceToHost, st));
+      FK(cudaMemcpyAsync(h + 16, blk7, hb, cudaMemcpyDeviceToHost, st));
+      int rc = wait_stream(st);
+      if (rc) return rc;
+      const FrontCounters* fc = (const FrontCounters*)(h + 16);
+      n1 = (int32_t)((const int64_t*)h)[0];
+      room = ((const int64_t*)h)[1];
+      br_total = fc->br_total;
+      // give up where this level does not get far: the traversal runs instead
+      if (fc->overflow || fc->max_pieces > FRONT_PIECES || n1 > l.n - l.n / 4 || n1 > FRONT_REDUCED_MAX ||
+          room > (int64_t)1 << 30)
+        return GSOFA_OK;
+      const int32_t* hq = (const int32_t*)(h + 16) + 16;
+      for (int32_t b = 0; b < fc->nblocks; b++) {
+        FrontMat m;
+        std::memset(&m, 0, sizeof(m));
+        m.first_vertex = hq[b];
+        m.sz = hq[cap + b];
+        m.nr = hq[2 * (size_t)cap + b];
+        m.nb = hq[3 * (size_t)cap + b];
+        m.br_base = hq[4 * (size_t)cap + b];
+        m.bc_base = hq[5 * (size_t)cap + b];
+        fronts.push_back(m);
+      }
+      if (fc->bc_total > 0) FK(launch_front_gids(l, l.bc, fc->bc_total, bcg, st));
+    }
+    // launch shapes; bitmap rows one front after the other
+    const size_t B = fronts.size();
+    std::vector<int> cs(B);
+    std::vector<size_t> smem(B);
+    int64_t words = 0;
+    for (size_t b = 0; b < B; b++) {
+      FrontMat& m = fronts[b];
+      const int pivots = (m.sz + 31) / 32;
+      cs[b] = 0;
+      for (int C = 1; C <= 8 && !cs[b]; C *= 2) {
+        smem[b] = front_smem_bytes(m.sz, m.nr, m.nb, C);
+        if (smem[b] <= BAND_SMEM_MAX - 1024) cs[b] = C;
+      }
+      if (!cs[b]) return GSOFA_OK;
+      // few fronts: more CTAs each
+      while (cs[b] < 8 && B * 2 * cs[b] <= (size_t)c->sms / 2 && pivots > 8 * cs[b]) {
+        cs[b] *= 2;
+        smem[b] = front_smem_bytes(m.sz, m.nr, m.nb, cs[b]);
+      }
+      m.bits_base = words;
+      words += (int64_t)(32 * pivots + m.nr) * (pivots + (m.nb + 31) / 32);
+    }
+    std::vector<int32_t> order(B);
+    for (size_t b = 0; b < B; b++) order[b] = (int32_t)b;
+    std::stable_sort(order.begin(), order.end(), [&](int32_t x, int32_t y) {
+      return cs[x] != cs[y] ? cs[x] < cs[y] : fronts[x].sz + fronts[x].nr > fronts[y].sz + fronts[y].nr;
+    });
+    uint32_t* bits = keep.get<uint32_t>((size_t)words);
+    FrontMat* d_fronts = level_mem.get<FrontMat>(2 * B);  // by block number, then in launch order
+    FrontMat* stage = (FrontMat*)thread_pinned(sizeof(FrontMat) * 2 * B, 0);
+    if (!keep.ok || !level_mem.ok || !stage) return GSOFA_OK;
+    for (size_t b = 0; b < B; b++) {
+      stage[b] = fronts[b];
+      stage[B + b] = fronts[order[b]];
+    }
+    FK(cudaMemcpyAsync(d_fronts, stage, sizeof(FrontMat) * 2 * B, cudaMemcpyHostToDevice, st));
+    FrontArgs f;
+    std::memset(&f, 0, sizeof(f));
+    f.fronts = d_fronts + B;
+    f.beg = l.beg;
+    f.end = l.end;
+    f.col = l.col;
+    f.br_b = l.br_b;
+    f.br_e = l.br_e;
+    f.bc = l.bc;
+    f.bits = bits;
+    for (size_t b = 0; b < B;) {
+      size_t k = b, most = 0;
+      for (; k < B && cs[order[k]] == cs[order[b]]; k++) most = std::max(most, smem[order[k]]);
+      f.first = (int32_t)b;
+      FK(launch_front_elim(f, (int)(k - b), cs[order[b]], most, st));
+      *launches += 1;
+      b = k;
+    }
+    const size_t b0 = blocks.size();
+    if (n1 > 0 && !whole) {
+      int32_t* beg1 = next_mem.get<int32_t>(n1);
+      int32_t* end1 = next_mem.get<int32_t>(n1);
+      int32_t* col1 = next_mem.get<int32_t>((size_t)(room > 0 ? room : 1));
+      int32_t* gid1 = keep.get<int32_t>(n1);
+      if (!next_mem.ok || !keep.ok) return GSOFA_OK;
+      FK(launch_front_reduce(l, n1, d_fronts, bits, beg1, end1, col1, gid1, st));
+      *launches += 2;
+      for (size_t b = 0; b < B; b++) {
+        FrontBlock q;
+        std::memset(&q, 0, sizeof(q));
+        const FrontMat& m = fronts[b];
+        q.bits = bits + m.bits_base;
+        q.cols = l.gid + m.first_vertex;
+        q.bcols = bcg + m.bc_base;
+        q.level = level;
+        q.sz = m.sz;
+        q.nb = m.nb;
+        q.pivots = (m.sz + 31) / 32;
+        q.W = q.pivots + (m.nb + 31) / 32;
+        blocks.push_back(q);
+      }
+      level_mem.free_all();
+      std::swap(level_mem.ptrs, next_mem.ptrs);
+      l.blocks_before = (int32_t)(b0 + B);
+      l.pieces_before += br_total;
+      l.n = n1;
+      l.beg = beg1;
+      l.end = end1;
+      l.col = col1;
+      l.gid = gid1;
+      continue;
+    }
+    for (size_t b = 0; b < B; b++) {
+      FrontBlock q;
+      std::memset(&q, 0, sizeof(q));
+      const FrontMat& m = fronts[b];
+      q.bits = bits + m.bits_base;
+      q.cols = l.gid + m.first_vertex;
+      q.bcols = bcg ? bcg + m.bc_base : nullptr;
+      q.level = level;
+      q.sz = m.sz;
+      q.nb = m.nb;
+      q.pivots = (m.sz + 31) / 32;
+      q.W = q.pivots + (m.nb + 31) / 32;
+      blocks.push_back(q);
+    }
+    n1 = -1;
+    level_mem.free_all();
+    l.n = 0;
+    break;
+  }
+  if (l.n != 0) return GSOFA_OK;  // too many levels
+
+  ev.rec(3, st);
+  int rc = wait_stream(st);  // the staging buffers are free
+  if (rc) return rc;
+  // sizes, then columns and supernodes
+  FrontBlock* d_blocks = keep.get<FrontBlock>(blocks.size());
+  FrontBlock* stage = (FrontBlock*)thread_pinned(sizeof(FrontBlock) * blocks.size(), 0);
+  int32_t* nL = keep.get<int32_t>(n);
+  int32_t* nU = keep.get<int32_t>(n);
+  int32_t* flags = keep.get<int32_t>(n);
+  int64_t* pos = keep.get<int64_t>((size_t)n + 1);
+  void* tmp = keep.get<unsigned char>(scan_tmp_bytes(n));
+  DevCounters* ctr = keep.get<DevCounters>(1);
+  unsigned char* h = (unsigned char*)thread_pinned(16 + sizeof(DevCounters), 1);
+  if (!keep.ok || !stage || !h) return GSOFA_OK;
+  *taken = true;
+  BandRun res;
+  res.c = c;
+  res.st = st;
+  res.fill = nullptr;
+  auto fail = [&](int rc) {
+    wait_stream(st);
+    cudaGetLastError();
+    res.free_results();
+    return rc;
+  };
+#define RK(x)                                          \
+  do {                                                 \
+    if ((x) != cudaSuccess) return fail(GSOFA_E_CUDA); \
+  } while (0)
+  std::memcpy(stage, blocks.data(), sizeof(FrontBlock) * blocks.size());
+  RK(cudaMemcpyAsync(d_blocks, stage, sizeof(FrontBlock) * blocks.size(), cudaMemcpyHostToDevice, st));
+  FrontEmit e;
+  std::memset(&e, 0, sizeof(e));
+  e.n = n;
+  e.blocks = d_blocks;
+  e.own = l.own;
+  e.own_row = l.own_row;
+  e.head = l.head;
+  e.piece_next = l.piece_next;
+  e.piece_blk = l.piece_blk;
+  e.piece_row = l.piece_row;
+  e.row_nL = nL;
+  e.row_nU = nU;
+  e.fill = fill;
+  RK(launch_init_counters(ctr, st));
+  RK(launch_front_count(e, st));
+  if (palloc(c, &res.Lrp, (size_t)n + 1, st) != cudaSuccess || palloc(c, &res.Urp, (size_t)n + 1, st) != cudaSuccess)
+    return fail(GSOFA_E_NOMEM);
+  RK(launch_scan_i32_i64(nL, res.Lrp, n, tmp, st));
+  RK(launch_scan_i32_i64(nU, res.Urp, n, tmp, st));
+  RK(cudaMemcpyAsync(h, res.Lrp + n, 8, cudaMemcpyDeviceToHost, st));
+  RK(cudaMemcpyAsync(h + 8, res.Urp + n, 8, cudaMemcpyDeviceToHost, st));
+  rc = wait_stream(st);
+  if (rc) return fail(rc);
+  out->nnz_L = ((const int64_t*)h)[0];
+  out->nnz_U = ((const int64_t*)h)[1];
+  if (palloc(c, &res.Lci, (size_t)out->nnz_L, st) != cudaSuccess || palloc(c, &res.Uci, (size_t)out->nnz_U, st) != cudaSuccess)
+    return fail(GSOFA_E_NOMEM);
+  e.L_rowptr = res.Lrp;
+  e.U_rowptr = res.Urp;
+  e.L_colidx = res.Lci;
+  e.U_colidx = res.Uci;
+  RK(launch_front_expand(e, st));
+  ev.rec(4, st);
+  RK(launch_supernode_flags(n, o.chunk_size, (const uint32_t*)res.Lci, res.Lrp, nL, nU, flags, ctr, st));
+  RK(launch_scan_i32_i64(flags, pos, n, tmp, st));
+  RK(cudaMemcpyAsync(h + 16, ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, st));
+  rc = wait_stream(st);
+  if (rc) return fail(rc);
+  out->n_super = ((const DevCounters*)(h + 16))->n_super;
+  if (palloc(c, &res.sup, (size_t)out->n_super + 1, st) != cudaSuccess) return fail(GSOFA_E_NOMEM);
+  RK(launch_scatter_starts(n, flags, pos, res.sup, st));
+  ev.rec(5, st);
+  *launches += 14;
+#undef FK
+#undef RK
+  Priv* pv = new Priv();
+  pv->stream = st;
+  pv->device = c->device;
+  pv->mpool = c->mpool;
+  out->_priv = pv;
+  out->n = n;
+  out->on_device = 1;
+  out->L_rowptr = res.Lrp;
+  out->U_rowptr = res.Urp;
+  out->L_colidx = res.Lci;
+  out->U_colidx = res.Uci;
+  out->fill_count = fill;
+  out->super_start = res.sup;
+  out->stats.traverse_launches = 1;
+  out->stats.levels = (int64_t)blocks.size();
+  return GSOFA_OK;
+}
+
+// One matrix by elimination on chip: as a band, or (larger ones) block by block of a
+// nested dissection.  *taken: the call is done (whatever it returns); otherwise nothing is
+// left behind and the traversal runs.
 int run_band_single(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gsofa_options& o, cudaStream_t st,
                     gsofa_result* out, bool* taken) {
   *taken = false;
@@ -784,6 +1139,29 @@ int run_band_single(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, con
       words = band_layout(b);
       if (words >= 0) rc = band_run(b, words, ev);
     }
+  }
+  if (rc == GSOFA_OK && words < 0 && n >= FRONT_MIN_ORDER) {
+    bool fronts = false;
+    int launches = b.launches;
+    rc = run_fronts(c, n, rp, ci, o, st, b.fill, out, ev, &launches, &fronts);
+    if (rc == GSOFA_OK && fronts) {
+      *taken = true;
+      b.fill = nullptr;  // the result's
+      b.free_scratch();
+      out->stats.kernel_launches = launches;
+      if (o.collect_stats) {
+        rc = wait_stream(st);
+        if (rc) {
+          gsofa_free(out);
+          return rc;
+        }
+        band_times(ev, &out->stats);
+      }
+      return GSOFA_OK;
+    }
+    const int32_t det = out->err_detail;
+    zero_result(out);
+    out->err_detail = det;
   }
   b.free_scratch();
   if (rc != GSOFA_OK || words < 0) {
@@ -1966,6 +2344,14 @@ int run_batch(Ctx* c, int32_t count, const int32_t* n, const int32_t* const* rp,
     rc = run_batch_members(c, members, n, rp, ci, o, st, outs, &launches, transient, pool_entries);
   for (size_t j = 0; rc == GSOFA_OK && j < singles.size(); j++) {
     const int32_t k = singles[j];
+    if (n[k] >= FRONT_MIN_ORDER && band_allowed(o)) {
+      bool taken = false;
+      rc = run_band_single(c, n[k], rp[k], ci[k], o, st, &outs[k], &taken);
+      if (taken) {
+        if (rc == GSOFA_OK) launches += outs[k].stats.kernel_launches;
+        continue;
+      }
+    }
     rc = run_device(c, n[k], rp[k], ci[k], o, st, &outs[k], pool_entries ? pool_entries[k] : 0);
     if (rc == GSOFA_OK) launches += outs[k].stats.kernel_launches;
   }

@@ -151,11 +151,13 @@ __global__ void band_scan_kernel(BandArgs a) {
 namespace {
 
 // One CTA's view of its matrix.  Panel q (rows 32q .. 32q+31) lives in CTA q % C at slot
-// (q / C) % slots; word c of a row of panel q is at index c - q + LB.
+// (q / C) % slots.  Band: word c of a row of panel q is at index c - q + LB, and a panel
+// reaches UB words right of its own.  Front (a dense block of W words per row, all of its
+// rows on chip): word c is at index c.
 struct Band {
   const int32_t* rowptr;
   const int32_t* colidx;
-  int n, LB, UB;
+  int n, LB, UB, W;
   int xs;          // words per row in shared memory (odd: lane-per-row accesses spread over the banks)
   int us;          // words per panel row in the panel buffers (odd)
   int slots;
@@ -166,6 +168,12 @@ template <int C>
 __device__ __forceinline__ uint32_t* panel_rows(const Band& B, int q) {
   return B.x + (size_t)((q / C) % B.slots) * 32 * B.xs;
 }
+
+// Word 0 of the columns in a row of panel q, and the words right of panel P's own.
+template <bool FRONT>
+__device__ __forceinline__ int word0(const Band& B, int q) { return FRONT ? 0 : B.LB - q; }
+template <bool FRONT>
+__device__ __forceinline__ int words_right(const Band& B, int P) { return FRONT ? B.W - 1 - P : B.UB; }
 
 // The entries of rows 32q .. 32q+31 into their zeroed slot (one warp), from the staged
 // copy of the panel's columns or in place.
@@ -324,21 +332,22 @@ __device__ __forceinline__ uint32_t close_word(uint32_t m, const uint32_t* g) {
 // The chain: panel P applied to the block of panel P + 1, then its factor.  With one CTA
 // the panel's rows right of the block are not ready yet (B runs beside this): their first
 // word is found here too.  Barrier 1 tells the workers that this warp's inputs are read.
-template <int C>
+template <int C, bool FRONT>
 __device__ __forceinline__ void step_chain(const Band& B, const PanelBufs& S, int P, int sync_threads) {
   const int lane = threadIdx.x & 31, at = 32 * (P & 1) + lane;
-  const uint32_t* x1 = panel_rows<C>(B, P + 1) + lane * B.xs + B.LB;
-  uint32_t m = B.LB > 0 ? x1[-1] : 0u, y = x1[0];
+  const uint32_t* x1 = panel_rows<C>(B, P + 1) + lane * B.xs + word0<FRONT>(B, P + 1) + P;
+  uint32_t m = FRONT || B.LB > 0 ? x1[0] : 0u, y = x1[1];
   uint32_t first = 0u;
+  const bool right = words_right<FRONT>(B, P) > 0;
   if constexpr (C == 1) {
-    const uint32_t v = B.UB > 0 ? panel_rows<C>(B, P)[lane * B.xs + B.LB + 1] : 0u;
+    const uint32_t v = right ? panel_rows<C>(B, P)[lane * B.xs + word0<FRONT>(B, P) + P + 1] : 0u;
     const uint32_t dip = S.dip[at];
     group_arrive(1, sync_threads);
     first = v;
 #pragma unroll
     for (int k = 0; k < 31; k++) first |= __shfl_sync(FULL, v, k) & spread(dip, k);
   } else {
-    if (B.UB > 0) first = S.pu[(size_t)32 * B.us * (P & 1) + lane * B.us];
+    if (right) first = S.pu[(size_t)32 * B.us * (P & 1) + lane * B.us];
     group_arrive(1, sync_threads);
   }
   if (__any_sync(FULL, m != 0u)) {
@@ -359,16 +368,17 @@ __device__ __forceinline__ void step_chain(const Band& B, const PanelBufs& S, in
 }
 
 // B: the rows of panel P right of the block; a row takes rows of the block as they came
-// in.  Items [i0, i0 + 32) of 16 * UB, one lane each: one word of two rows (one load of a
-// block row serves both).
-template <int C>
+// in.  Items [i0, i0 + 32) of 16 * ub (ub words right of the block), one lane each: one
+// word of two rows (one load of a block row serves both).
+template <int C, bool FRONT>
 __device__ __forceinline__ void step_rows(const Band& B, const PanelBufs& S, int P, int i0) {
   const int i = i0 + (threadIdx.x & 31);
-  if (i >= 16 * B.UB) return;
+  const int ub = words_right<FRONT>(B, P);
+  if (i >= 16 * ub) return;
   uint32_t* pu = S.pu + (size_t)32 * B.us * (P & 1);
   const uint32_t* dip = S.dip + 32 * (P & 1);
-  const int r0 = i / B.UB * 2, c = i - (r0 >> 1) * B.UB;
-  const uint32_t* col = panel_rows<C>(B, P) + B.LB + 1 + c;
+  const int r0 = i / ub * 2, c = i - (r0 >> 1) * ub;
+  const uint32_t* col = panel_rows<C>(B, P) + word0<FRONT>(B, P) + P + 1 + c;
   uint32_t m0 = dip[r0], m1 = dip[r0 + 1];
   uint32_t v0 = col[r0 * B.xs], v1 = col[(r0 + 1) * B.xs];
 #pragma unroll 1
@@ -416,6 +426,94 @@ __device__ __forceinline__ void step_tops(const PanelBufs& S, int P) {
   }
 }
 
+// The workers' part of the step of panel P: B (one CTA), then C for this CTA's panels
+// P + 1 .. hi.  nwk worker warps, warp 1 the first; `next`: the chain runs beside this.
+template <int C, bool FRONT>
+__device__ __forceinline__ void step_below(const Band& B, const PanelBufs& S, int P, int hi, bool next, int rank,
+                                           int nwk) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int wk = 32 * nwk, me = (int)threadIdx.x - 32;
+  const int ub = words_right<FRONT>(B, P);
+  // first: B, and the rows that the panel reaches, their words closed
+  const int lo = P + 1 + (C > 1 ? (rank - (P + 1) % C + C) % C : 0);  // this CTA's first panel from P + 1 on
+  const int cnt = hi >= lo ? (hi - lo) / C + 1 : 0;
+  const int nb = C == 1 ? (16 * ub + 31) / 32 : 0;
+  for (int u = warp - 1; u < nb + cnt; u += nwk) {
+    if (u < nb) {
+      step_rows<C, FRONT>(B, S, P, 32 * u);
+    } else {
+      const int q = lo + C * (u - nb);
+      const uint32_t m = panel_rows<C>(B, q)[lane * B.xs + word0<FRONT>(B, q) + P];
+      S.cl[32 * (u - nb) + lane] = __any_sync(FULL, m != 0u) ? close_word(m, S.pg + 32 * (P & 1)) : 0u;
+    }
+  }
+  if (next) group_sync(1, 32 * (C == 1 ? nwk + 2 : nwk + 1));
+  else group_sync(2, 32 * nwk);
+  if (cnt == 0) return;
+  const uint32_t* pu = S.pu + (size_t)32 * B.us * (P & 1);
+  const int slot0 = (lo / C) % B.slots;  // this CTA's panels from lo on have the slots from here on
+  // this thread's word of a row, and the stride of all workers
+  const int r_at = ub > 0 ? me / ub : 0, c_at = ub > 0 ? me - r_at * ub : 0;
+  const int dr = ub > 0 ? wk / ub : 0, dc = ub > 0 ? wk - dr * ub : 0;
+  // the closed words into place, and which partnerless rows they hold, numbered; the
+  // tables of those rows
+  const uint32_t* top = S.top + 33 * (P & 1);
+  const int nt = (int)top[0];
+  for (int u = warp - 1; u < cnt; u += nwk) {
+    int slot = slot0 + u;
+    if (slot >= B.slots) slot -= B.slots;
+    const uint32_t m = S.cl[32 * u + lane];
+    if (m) B.x[(slot * 32 + lane) * B.xs + word0<FRONT>(B, lo + C * u) + P] = m;
+    uint32_t has = 0u;
+#pragma unroll 4
+    for (int i = 0; i < nt; i++) has |= ((m >> top[1 + i]) & 1u) << i;
+    S.cl[32 * u + lane] = has;
+  }
+  if (ub > 0) {
+    const int ne = (nt + 3) / 4 * 16;
+    for (int e = r_at, c = c_at; e < ne;) {
+      uint32_t v = 0u;
+      const int g0 = e >> 4 << 2;
+#pragma unroll
+      for (int i = 0; i < 4; i++)
+        if (((e >> i) & 1) && g0 + i < nt) v |= pu[top[1 + g0 + i] * B.us + c];
+      S.tb[e * B.us + c] = v;
+      e += dr;
+      c += dc;
+      if (c >= ub) {
+        c -= ub;
+        e++;
+      }
+    }
+  }
+  group_sync(2, 32 * nwk);
+  if (ub == 0) return;
+  // then C, a word of a row per lane
+  for (int r = r_at, c = c_at; r < 32 * cnt;) {
+    uint32_t has = S.cl[r];
+    if (has) {
+      const int u = r >> 5;
+      int slot = slot0 + u;
+      if (slot >= B.slots) slot -= B.slots;
+      uint32_t* x = B.x + (slot * 32 + (r & 31)) * B.xs + word0<FRONT>(B, lo + C * u) + P + 1 + c;
+      uint32_t v = *x;
+      const uint32_t* tb = S.tb + c;
+      do {
+        v |= tb[(has & 15u) * B.us];
+        tb += 16 * B.us;
+        has >>= 4;
+      } while (has);
+      *x = v;
+    }
+    r += dr;
+    c += dc;
+    if (c >= ub) {
+      c -= ub;
+      r++;
+    }
+  }
+}
+
 }  // namespace
 
 // Warps of a CTA: 0 the chain, the last the loader (rows into the window), the others
@@ -438,10 +536,9 @@ __global__ void __launch_bounds__(512, 1) band_elim_kernel(BandArgs a) {
   B.xs = wx | 1;
   B.us = B.UB | 1;
   B.slots = (B.LB + 2 + C - 1) / C;
-  // the workers' strides over words of rows: UB words (C) and wx words (finished rows)
+  // the workers' stride over the words of finished rows
   const int wk = 32 * nwk, me = (int)threadIdx.x - 32;
-  const int ub_r = B.UB > 0 ? wk / B.UB : 0, ub_c = B.UB > 0 ? wk % B.UB : 0, wx_r = wk / wx, wx_c = wk % wx;
-  const int my_ub_r = B.UB > 0 ? me / B.UB : 0, my_ub_c = B.UB > 0 ? me % B.UB : 0;
+  const int wx_r = wk / wx, wx_c = wk % wx;
   PanelBufs S;
   S.pw = bsm;
   S.pg = S.pw + 64;
@@ -504,7 +601,7 @@ __global__ void __launch_bounds__(512, 1) band_elim_kernel(BandArgs a) {
       if constexpr (C > 1) {
         if (loader) step_tops<C>(S, q0);
         else
-          for (int i = 32 * warp; i < 16 * B.UB; i += 32 * (nw - 1)) step_rows<C>(B, S, q0, i);
+          for (int i = 32 * warp; i < 16 * B.UB; i += 32 * (nw - 1)) step_rows<C, false>(B, S, q0, i);
       }
     }
     sync_all();
@@ -515,7 +612,7 @@ __global__ void __launch_bounds__(512, 1) band_elim_kernel(BandArgs a) {
       // P + 1 into every CTA's buffers.
       const bool next = P + 1 < panels && (P + 1) % C == rank;
       if (chain) {
-        if (next) step_chain<C>(B, S, P, 32 * (C == 1 ? nwk + 2 : nwk + 1));
+        if (next) step_chain<C, false>(B, S, P, 32 * (C == 1 ? nwk + 2 : nwk + 1));
       } else if (loader) {
         if constexpr (C == 1) {
           step_tops<C>(S, P);
@@ -537,84 +634,9 @@ __global__ void __launch_bounds__(512, 1) band_elim_kernel(BandArgs a) {
         rb2 = rb3; re2 = re3;
         rb3 = rb4; re3 = re4;
       } else {
-        // first: B (one CTA), and the rows that the panel reaches, their words closed
-        const int lo = P + 1 + (C > 1 ? (rank - (P + 1) % C + C) % C : 0);  // this CTA's first panel from P + 1 on
         const int hi = min(P + B.LB, panels - 1);
-        const int cnt = hi >= lo ? (hi - lo) / C + 1 : 0;
-        const int nb = C == 1 ? (16 * B.UB + 31) / 32 : 0;
-        for (int u = warp - 1; u < nb + cnt; u += nwk) {
-          if (u < nb) {
-            step_rows<C>(B, S, P, 32 * u);
-          } else {
-            const int q = lo + C * (u - nb);
-            const uint32_t m = panel_rows<C>(B, q)[lane * B.xs + B.LB - (q - P)];
-            S.cl[32 * (u - nb) + lane] = __any_sync(FULL, m != 0u) ? close_word(m, S.pg + 32 * (P & 1)) : 0u;
-          }
-        }
-        if (next) group_sync(1, 32 * (C == 1 ? nwk + 2 : nwk + 1));
-        else group_sync(2, 32 * nwk);
+        step_below<C, false>(B, S, P, hi, next, rank, nwk);
         const uint32_t* pu = S.pu + (size_t)32 * B.us * (P & 1);
-        const int slot0 = (lo / C) % B.slots;  // this CTA's panels from lo on have the slots from here on
-        if (cnt > 0) {
-          // the closed words into place, and which partnerless rows they hold, numbered;
-          // the tables of those rows
-          const uint32_t* top = S.top + 33 * (P & 1);
-          const int nt = (int)top[0];
-          for (int u = warp - 1; u < cnt; u += nwk) {
-            int slot = slot0 + u;
-            if (slot >= B.slots) slot -= B.slots;
-            const uint32_t m = S.cl[32 * u + lane];
-            if (m) B.x[(slot * 32 + lane) * B.xs + B.LB - (lo - P) - C * u] = m;
-            uint32_t has = 0u;
-#pragma unroll 4
-            for (int i = 0; i < nt; i++) has |= ((m >> top[1 + i]) & 1u) << i;
-            S.cl[32 * u + lane] = has;
-          }
-          {
-            int e = my_ub_r, c = my_ub_c;
-            const int ne = (nt + 3) / 4 * 16;
-            while (e < ne && B.UB > 0) {
-              uint32_t v = 0u;
-              const int g0 = e >> 4 << 2;
-#pragma unroll
-              for (int i = 0; i < 4; i++)
-                if (((e >> i) & 1) && g0 + i < nt) v |= pu[top[1 + g0 + i] * B.us + c];
-              S.tb[e * B.us + c] = v;
-              e += ub_r;
-              c += ub_c;
-              if (c >= B.UB) {
-                c -= B.UB;
-                e++;
-              }
-            }
-          }
-          group_sync(2, 32 * nwk);
-          // then C, a word of a row per lane
-          int r = my_ub_r, c = my_ub_c;
-          while (r < 32 * cnt && B.UB > 0) {
-            uint32_t has = S.cl[r];
-            if (has) {
-              const int u = r >> 5;
-              int slot = slot0 + u;
-              if (slot >= B.slots) slot -= B.slots;
-              uint32_t* x = B.x + (slot * 32 + (r & 31)) * B.xs + B.LB - (lo - P) - C * u + 1 + c;
-              uint32_t v = *x;
-              const uint32_t* tb = S.tb + c;
-              do {
-                v |= tb[(has & 15u) * B.us];
-                tb += 16 * B.us;
-                has >>= 4;
-              } while (has);
-              *x = v;
-            }
-            r += ub_r;
-            c += ub_c;
-            if (c >= B.UB) {
-              c -= B.UB;
-              r++;
-            }
-          }
-        }
         {
           // finished rows out; their slot is zeroed for the panel that takes it
           if (P % C == rank && a.bits) {
@@ -661,7 +683,7 @@ __global__ void __launch_bounds__(512, 1) band_elim_kernel(BandArgs a) {
           __syncthreads();
           if (loader) step_tops<C>(S, P + 1);
           else
-            for (int i = 32 * warp; i < 16 * B.UB; i += 32 * (nw - 1)) step_rows<C>(B, S, P + 1, i);
+            for (int i = 32 * warp; i < 16 * B.UB; i += 32 * (nw - 1)) step_rows<C, false>(B, S, P + 1, i);
         }
       }
       sync_all();
@@ -669,6 +691,138 @@ __global__ void __launch_bounds__(512, 1) band_elim_kernel(BandArgs a) {
     if (loader) copy_async_wait<0>();
     __syncthreads();
     q0 = panels < last ? panels : last;
+  }
+}
+
+// ------------------------------------------------------------ fronts
+// Elimination of one block of a nested dissection (fronts.cu): rows 0 .. sz-1 are the
+// block's vertices (the pivots), then nr rows above the block that have entries in its
+// columns; columns are the block's, then the nb columns right of it that its rows reach.
+// The whole front is on chip; all of its rows come out: L and U of the block's vertices,
+// and for the rows above their L entries in the block and what they reach through it.
+template <int C>
+__global__ void __launch_bounds__(512, 1) front_elim_kernel(FrontArgs a) {
+  extern __shared__ __align__(16) uint32_t bsm[];
+  const int rank = C > 1 ? (int)(blockIdx.x % C) : 0;
+  const FrontMat d = a.fronts[a.first + blockIdx.x / C];
+  const int nw = blockDim.x >> 5, nwk = nw - 2;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool chain = warp == 0, loader = warp == nw - 1;
+  const int pivots = (d.sz + 31) >> 5, panels = pivots + ((d.nr + 31) >> 5);
+  Band B;
+  B.rowptr = nullptr;
+  B.colidx = a.col;
+  B.n = d.sz;
+  B.LB = 0;
+  B.W = pivots + ((d.nb + 31) >> 5);
+  B.UB = B.W - 1;
+  B.xs = B.W | 1;
+  B.us = B.UB | 1;
+  B.slots = (panels + C - 1) / C;
+  PanelBufs S;
+  S.pw = bsm;
+  S.pg = S.pw + 64;
+  S.dip = S.pg + 64;
+  S.top = S.dip + 64;
+  S.pu = S.top + 68;
+  S.cl = S.pu + 64 * B.us;
+  S.tb = S.cl + 32 * B.slots;
+  B.x = S.tb + 128 * B.us;
+  uint32_t* out = a.bits + d.bits_base;
+  const int32_t* bc = a.bc + d.bc_base;
+  auto sync_all = [&] {
+    if constexpr (C > 1) cg::this_cluster().sync();
+    else __syncthreads();
+  };
+
+  for (int i = threadIdx.x; i < B.slots * 32 * B.xs; i += blockDim.x) B.x[i] = 0u;
+  __syncthreads();
+  // the rows, one warp each: columns of the block are their offset, the others their place in bc
+  for (int i = warp; i < 32 * panels; i += nw) {
+    const int q = i >> 5;
+    if (q % C != rank) continue;
+    int b = 0, e = 0;
+    if (q < pivots) {
+      if (i < d.sz) {
+        b = a.beg[d.first_vertex + i];
+        e = a.end[d.first_vertex + i];
+      }
+    } else if (i - 32 * pivots < d.nr) {
+      b = a.br_b[d.br_base + i - 32 * pivots];
+      e = a.br_e[d.br_base + i - 32 * pivots];
+    }
+    uint32_t* row = panel_rows<C>(B, q) + (i & 31) * B.xs;
+    for (int k = b + lane; k < e; k += 32) {
+      const int c = a.col[k] - d.first_vertex;
+      int at = c;
+      if (c >= d.sz) {
+        int lo = 0, hi = d.nb - 1;
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (bc[mid] < c + d.first_vertex) lo = mid + 1; else hi = mid;
+        }
+        at = 32 * pivots + lo;
+      }
+      atomicOr(row + (at >> 5), 1u << (at & 31));
+    }
+  }
+  sync_all();
+  if (rank == 0) {
+    if (chain) step_factor<C>(S, 0, panel_rows<C>(B, 0)[lane * B.xs]);
+    __syncthreads();
+    if constexpr (C > 1) {
+      if (loader) step_tops<C>(S, 0);
+      else
+        for (int i = 32 * warp; i < 16 * B.UB; i += 32 * (nw - 1)) step_rows<C, true>(B, S, 0, i);
+    }
+  }
+  sync_all();
+  const int W = B.W;
+  for (int P = 0; P < pivots; P++) {
+    const bool next = P + 1 < pivots && (P + 1) % C == rank;
+    if (chain) {
+      if (next) step_chain<C, true>(B, S, P, 32 * (C == 1 ? nwk + 2 : nwk + 1));
+    } else if (loader) {
+      if constexpr (C == 1) {
+        // (without a chain beside them the workers wait for the partnerless rows by barrier 3)
+        step_tops<C>(S, P);
+        __syncwarp();
+        if (next) group_arrive(1, 32 * (nwk + 2));
+        else group_arrive(3, 32 * (nwk + 1));
+      }
+    } else {
+      if constexpr (C == 1) {
+        if (!next) group_sync(3, 32 * (nwk + 1));
+      }
+      step_below<C, true>(B, S, P, panels - 1, next, rank, nwk);
+      if (P % C == rank) {  // finished rows out
+        const int rows = min(32, d.sz - 32 * P);
+        const uint32_t* x = panel_rows<C>(B, P);
+        const uint32_t* pu = S.pu + (size_t)32 * B.us * (P & 1);
+        uint32_t* o = out + (size_t)32 * P * W;
+        for (int r = warp - 1; r < rows; r += nwk)
+          for (int c = lane; c < W; c += 32)
+            o[(size_t)r * W + c] = c < P ? x[r * B.xs + c] : (c == P ? S.pw[32 * (P & 1) + r] : pu[r * B.us + c - P - 1]);
+      }
+    }
+    if constexpr (C > 1) {
+      if (next) {
+        __syncthreads();
+        if (loader) step_tops<C>(S, P + 1);
+        else
+          for (int i = 32 * warp; i < 16 * words_right<true>(B, P + 1); i += 32 * (nw - 1))
+            step_rows<C, true>(B, S, P + 1, i);
+      }
+    }
+    sync_all();
+  }
+  // the rows above the block
+  for (int i = warp; i < d.nr; i += nw) {
+    const int q = pivots + (i >> 5);
+    if (q % C != rank) continue;
+    const uint32_t* row = panel_rows<C>(B, q) + (i & 31) * B.xs;
+    uint32_t* o = out + (size_t)(32 * pivots + i) * W;
+    for (int c = lane; c < W; c += 32) o[c] = row[c];
   }
 }
 
@@ -944,6 +1098,45 @@ cudaError_t launch_band_elim(const BandArgs& a, int count, int C, int threads, s
     case 2: return launch_elim<2>(a, count, threads, smem, st);
     case 4: return launch_elim<4>(a, count, threads, smem, st);
     default: return launch_elim<8>(a, count, threads, smem, st);
+  }
+}
+
+// Clusters of C CTAs for fronts [a.first, a.first + count).
+size_t front_smem_bytes(int sz, int nr, int nb, int C) {
+  const int pivots = (sz + 31) / 32, panels = pivots + (nr + 31) / 32, W = pivots + (nb + 31) / 32;
+  const size_t slots = (size_t)(panels + C - 1) / C;
+  return 4 * (128 + 64 + 68 + 192 * (size_t)((W - 1) | 1) + slots * 32 * (size_t)((W | 1) + 1));
+}
+
+namespace {
+template <int C>
+cudaError_t launch_front(const FrontArgs& a, int count, size_t smem, cudaStream_t st) {
+  cudaError_t e =
+      cudaFuncSetAttribute(front_elim_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, BAND_SMEM_MAX);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(count * C));
+  cfg.blockDim = dim3(512);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = C > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, front_elim_kernel<C>, a);
+}
+}  // namespace
+
+cudaError_t launch_front_elim(const FrontArgs& a, int count, int C, size_t smem, cudaStream_t st) {
+  if (count <= 0) return cudaSuccess;
+  switch (C) {
+    case 1: return launch_front<1>(a, count, smem, st);
+    case 2: return launch_front<2>(a, count, smem, st);
+    case 4: return launch_front<4>(a, count, smem, st);
+    default: return launch_front<8>(a, count, smem, st);
   }
 }
 

@@ -48,6 +48,26 @@ struct BandArgs {
   int32_t *L_colidx, *U_colidx, *super_start;
 };
 
+// A front: one block of a nested dissection (fronts.cu).
+struct FrontMat {
+  int64_t bits_base;     // first word of its rows: (sz rounded up to 32) + nr of them, W words each
+  int32_t first_vertex;  // the block is vertices [first_vertex, first_vertex + sz) of its level
+  int32_t sz, nr, nb;    // pivots, rows above the block, columns right of it
+  int32_t br_base, bc_base;
+};
+
+struct FrontArgs {
+  const FrontMat* fronts;
+  int32_t first;
+  const int32_t *beg, *end, *col;  // rows of the level: columns col[beg[i] .. end[i])
+  const int32_t *br_b, *br_e;      // rows above the blocks: their entries in the block's columns
+  const int32_t* bc;               // columns right of the blocks, increasing
+  uint32_t* bits;
+};
+
+size_t front_smem_bytes(int sz, int nr, int nb, int C);
+cudaError_t launch_front_elim(const FrontArgs& a, int count, int C, size_t smem, cudaStream_t st);
+
 size_t band_smem_bytes(int LB, int UB, int C);
 struct BandShape {
   int C = 0;  // CTAs per matrix (0: the band does not fit on chip)
