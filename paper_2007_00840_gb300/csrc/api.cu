@@ -760,6 +760,7 @@ void band_times(Events& ev, gsofa_stats* s) {
 // about as long as the search), and up to which what remains is one front.
 constexpr int32_t FRONT_MIN_ORDER = 16384;
 constexpr int32_t FRONT_LAST_ORDER = 2900;
+constexpr int32_t FRONT_FIRST_BLOCK = 512;
 
 // Pool memory of one call, freed together.
 struct Held {
@@ -840,6 +841,12 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
       const size_t nl = (size_t)l.n;
       const int32_t cap = l.n / FRONT_BLOCK_MIN + 1;
       l.cap = cap;
+      // blocks of A: 512 vertices (on a 1024 x 1024 grid 6.3 ms; 256: 7.3, 1,024: 6.6); of a
+      // reduced level, whose rows are long, as large as the kernels take
+      l.block_max = level == 0 ? FRONT_FIRST_BLOCK : FRONT_BLOCK_MAX;
+      const size_t right_words = (nl + 31) / 32;
+      l.wide = level > 0 && right_words * (size_t)cap * sizeof(uint2) <= ((size_t)256 << 20);
+      l.right = l.wide ? level_mem.get<uint2>(right_words * cap) : nullptr;
       l.low = level_mem.get<int32_t>(nl);
       l.best = level_mem.get<int32_t>(nl);
       l.blk = level_mem.get<int32_t>(nl);
@@ -867,6 +874,7 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
       FK(cudaMemsetAsync(l.best, 0xFF, 4 * nl, st));
       FK(cudaMemsetAsync(l.blk, 0xFF, 4 * nl, st));
       FK(cudaMemsetAsync(l.bound, 0, 4 * nl, st));
+      if (l.wide) FK(cudaMemsetAsync(l.right, 0, sizeof(uint2) * right_words * cap, st));
       FK(launch_fill_i32(l.rem, l.n, 1, st));
       FK(launch_front_blocks(l, st));
       FK(launch_scan_i32_i64(l.rem, rank, l.n, tmp, st));
@@ -901,6 +909,7 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
         m.nb = hq[3 * (size_t)cap + b];
         m.br_base = hq[4 * (size_t)cap + b];
         m.bc_base = hq[5 * (size_t)cap + b];
+        m.id = b;
         fronts.push_back(m);
       }
       if (fc->bc_total > 0) FK(launch_front_gids(l, l.bc, fc->bc_total, bcg, st));
@@ -920,7 +929,7 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
       }
       if (!cs[b]) return GSOFA_OK;
       // few fronts: more CTAs each
-      while (cs[b] < 8 && B * 2 * cs[b] <= (size_t)c->sms / 2 && pivots > 8 * cs[b]) {
+      while (cs[b] < 8 && B * 2 * cs[b] <= (size_t)c->sms && pivots + (m.nr + 31) / 32 > 4 * cs[b]) {
         cs[b] *= 2;
         smem[b] = front_smem_bytes(m.sz, m.nr, m.nb, cs[b]);
       }
@@ -950,6 +959,8 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
     f.br_b = l.br_b;
     f.br_e = l.br_e;
     f.bc = l.bc;
+    f.right = whole ? nullptr : l.right;
+    f.right_words = (l.n + 31) / 32;
     f.bits = bits;
     for (size_t b = 0; b < B;) {
       size_t k = b, most = 0;

@@ -54,6 +54,7 @@ struct FrontMat {
   int32_t first_vertex;  // the block is vertices [first_vertex, first_vertex + sz) of its level
   int32_t sz, nr, nb;    // pivots, rows above the block, columns right of it
   int32_t br_base, bc_base;
+  int32_t id, pad;       // the block's number on its level
 };
 
 struct FrontArgs {
@@ -62,6 +63,8 @@ struct FrontArgs {
   const int32_t *beg, *end, *col;  // rows of the level: columns col[beg[i] .. end[i])
   const int32_t *br_b, *br_e;      // rows above the blocks: their entries in the block's columns
   const int32_t* bc;               // columns right of the blocks, increasing
+  const uint2* right;              // their places (FrontLevel::right), or null: searched in bc
+  int32_t right_words;             // words of a block in right
   uint32_t* bits;
 };
 

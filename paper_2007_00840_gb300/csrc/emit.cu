@@ -246,14 +246,18 @@ __global__ void supernode_kernel(int32_t n, int32_t chunk, const uint32_t* __res
       const int64_t off = row_off[s];
       bool has = false;
       if (off >= 0) {
-        int lo = 0, hi = row_nL[s];
+        // L(s,:) has at most s - r entries from r on: r, if there, is among its last s - r
+        // (the first of them where the rows between are all there, which one load tells)
+        const int nl = row_nL[s];
+        int lo = max(0, nl - (s - r)), hi = nl;
         const uint32_t key = (uint32_t)r;
+        if (lo < hi && pool[off + lo] >= key) hi = lo;
         while (lo < hi) {
           const int mid = (lo + hi) >> 1;
           const uint32_t x = pool[off + mid];
           if (x < key) lo = mid + 1; else hi = mid;
         }
-        has = lo < row_nL[s] && pool[off + lo] == key;
+        has = lo < nl && pool[off + lo] == key;
       }
       if (has) {
         flags[s] = 0;
@@ -424,13 +428,15 @@ __global__ void supernode_batch_kernel(const MatDesc* __restrict__ mats, int32_t
       const int64_t off = row_off[g];
       bool has = false;
       if (off >= 0) {
-        int lo = 0, hi = row_nL[g];
+        const int nl = row_nL[g];
+        int lo = max(0, nl - (c0 + u - r)), hi = nl;  // as in supernode_kernel
         const uint32_t key = (uint32_t)r;
+        if (lo < hi && pool[off + lo] >= key) hi = lo;
         while (lo < hi) {
           const int mid = (lo + hi) >> 1;
           if (pool[off + mid] < key) lo = mid + 1; else hi = mid;
         }
-        has = lo < row_nL[g] && pool[off + lo] == key;
+        has = lo < nl && pool[off + lo] == key;
       }
       if (has) {
         flags[g] = 0;

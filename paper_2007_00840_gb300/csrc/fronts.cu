@@ -29,14 +29,18 @@ __device__ __forceinline__ uint32_t lt_bits(int k) { return (1u << k) - 1u; }
 
 constexpr int TILE = 1024;
 
-// smallest neighbour of every vertex, over its row and its column; eight lanes per row
+// smallest neighbour of every vertex, over its row and its column; LANES lanes per row
+// (eight for rows of A, 32 for the rows of a reduced level, which have hundreds of
+// entries: 167 -> 40 us on a level of 6,000 rows)
+template <int LANES>
 __global__ void front_low_kernel(FrontLevel l) {
-  const int sub = threadIdx.x & 7;
-  const int step = (gridDim.x * blockDim.x) >> 3;
-  for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 3; i < l.n; i += step) {
+  const int sub = threadIdx.x % LANES;
+  const int step = (gridDim.x * blockDim.x) / LANES;
+  for (int i = (blockIdx.x * blockDim.x + threadIdx.x) / LANES; i < l.n; i += step) {
     const int e = l.end[i];
     int lo = i;
-    for (int k = l.beg[i] + sub; k < e; k += 8) {
+#pragma unroll 4
+    for (int k = l.beg[i] + sub; k < e; k += LANES) {
       const int c = l.col[k];
       lo = min(lo, c);
       if (c > i && *(volatile int32_t*)(l.low + c) > i) atomicMin(l.low + c, i);
@@ -45,35 +49,53 @@ __global__ void front_low_kernel(FrontLevel l) {
   }
 }
 
-// Closed stretches: for every vertex i the start of the smallest closed stretch ending at
-// i, where that has at most FRONT_BLOCK_MAX vertices.  Stretches nest or are apart, so one
-// pass with a stack of starts finds them; a CTA does a tile of vertices after a pass over
-// the FRONT_BLOCK_MAX before it (a start further left is too far anyway).
-__global__ void front_stretch_kernel(FrontLevel l) {
-  __shared__ int32_t low[TILE + FRONT_BLOCK_MAX];
-  __shared__ int32_t stack[TILE + FRONT_BLOCK_MAX + 1];
-  __shared__ int32_t start[TILE];
-  for (int t0 = blockIdx.x * TILE; t0 < l.n; t0 += gridDim.x * TILE) {
-    const int left = max(0, t0 - FRONT_BLOCK_MAX), right = min(l.n, t0 + TILE);
+// Closed stretches: for every vertex i the start R(i) of the smallest closed stretch that
+// ends at i, where it has at most block_max vertices: the least fixed point of
+// R(i) = min of R over [R(i), i], from the smallest neighbours.  A CTA does a tile of
+// vertices and looks at the FRONT_BLOCK_MAX before it (a start further left is too far
+// anyway).  Each round answers all range minima from windows of 1, 2, 4, .. vertices, and
+// since every vertex uses the others' current starts few rounds are needed (a pass with a
+// stack of starts by one thread took 186 us per level, this about 15).
+__global__ void __launch_bounds__(1024) front_stretch_kernel(FrontLevel l) {
+  constexpr int LEN = TILE + FRONT_BLOCK_MAX;
+  static_assert(LEN == 2048 && FRONT_BLOCK_MAX <= 1 << 10, "two vertices per thread, eleven windows");
+  __shared__ int16_t win[11][LEN];  // win[k][x]: smallest start over the 2^k vertices that end at x
+  const int t0 = blockIdx.x * TILE;
+  const int left = max(0, t0 - FRONT_BLOCK_MAX), len = min(l.n, t0 + TILE) - left;
+  int v[2];
+  for (int q = 0; q < 2; q++) {
+    const int x = threadIdx.x + 1024 * q;
+    const int lo = x < len ? min(l.low[left + x], left + x) - left : 0;
+    v[q] = lo < 0 || x - lo >= l.block_max ? -1 : lo;  // -1: too far left
+  }
+  for (;;) {
+    for (int q = 0; q < 2; q++) win[0][threadIdx.x + 1024 * q] = (int16_t)v[q];
     __syncthreads();
-    for (int i = left + threadIdx.x; i < right; i += blockDim.x) low[i - left] = min(l.low[i], i);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int sp = 0;
-      for (int i = left; i < right; i++) {
-        const int a = low[i - left];
-        int s = i;
-        while (s > a && sp > 0) s = stack[--sp];
-        if (s > a) s = -1;  // it starts left of what this tile looks at
-        stack[sp++] = s;
-        if (i >= t0) start[i - t0] = s;
+    for (int k = 1; k < 11; k++) {
+      for (int q = 0; q < 2; q++) {
+        const int x = threadIdx.x + 1024 * q, y = x - (1 << (k - 1));
+        const int16_t a = win[k - 1][x];
+        win[k][x] = y >= 0 ? min(a, win[k - 1][y]) : a;
+      }
+      __syncthreads();
+    }
+    int changed = 0;
+    for (int q = 0; q < 2; q++) {
+      const int x = threadIdx.x + 1024 * q;
+      if (x >= len || v[q] < 0 || v[q] == x) continue;
+      const int k = 31 - __clz(x - v[q] + 1);
+      int r = min((int)win[k][x], (int)win[k][v[q] + (1 << k) - 1]);
+      if (r < 0 || x - r >= l.block_max) r = -1;
+      if (r != v[q]) {
+        v[q] = r;
+        changed = 1;
       }
     }
-    __syncthreads();
-    for (int i = t0 + threadIdx.x; i < right; i += blockDim.x) {
-      const int s = start[i - t0];
-      if (s >= 0 && i - s < FRONT_BLOCK_MAX) atomicMax(l.best + s, i);
-    }
+    if (!__syncthreads_or(changed)) break;
+  }
+  for (int q = 0; q < 2; q++) {
+    const int x = threadIdx.x + 1024 * q;
+    if (x < len && left + x >= t0 && v[q] >= 0) atomicMax(l.best + left + v[q], left + x);
   }
 }
 
@@ -146,15 +168,16 @@ __device__ __forceinline__ int lower_entry(const int32_t* col, int k0, int k1, i
 // Rows of remaining vertices: their entries in one block are consecutive (blocks are
 // stretches).  FILL false: blocks' row counts, and the entries outside blocks; true: the
 // rows into their blocks' lists, and onto their vertices' piece lists.
-template <bool FILL>
+template <bool FILL, int LANES>
 __global__ void front_runs_kernel(FrontLevel l) {
-  const int sub = threadIdx.x & 7;
-  const int step = (gridDim.x * blockDim.x) >> 3;
-  for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 3; i < l.n; i += step) {
+  const int sub = threadIdx.x % LANES;
+  const int step = (gridDim.x * blockDim.x) / LANES;
+  for (int i = (blockIdx.x * blockDim.x + threadIdx.x) / LANES; i < l.n; i += step) {
     if (l.blk[i] >= 0) continue;
     const int b0 = l.beg[i], e0 = l.end[i];
     int outside = 0, runs = 0;
-    for (int k = b0 + sub; k < e0; k += 8) {
+#pragma unroll 2
+    for (int k = b0 + sub; k < e0; k += LANES) {
       const int c = l.col[k];
       const int b = l.blk[c];
       if (b < 0) {
@@ -303,6 +326,76 @@ __global__ void front_right_kernel(FrontLevel l) {
   }
 }
 
+// The same on a level of long rows: every block's bitmap over the level's vertices, a warp
+// per row of the block (one CTA per block hashing half a million entries took 1,356 us on
+// a level of 16 blocks) ...
+__global__ void front_right_set_kernel(FrontLevel l) {
+  const int lane = threadIdx.x & 31;
+  const int step = (gridDim.x * blockDim.x) >> 5;
+  const int words = (l.n + 31) >> 5;
+  for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < l.n; i += step) {
+    const int b = l.blk[i];
+    if (b < 0) continue;
+    uint2* right = l.right + (size_t)b * words;
+    const int e = l.end[i];
+    const int k0 = lower_entry(l.col, l.beg[i], e, l.b_first[b] + l.b_size[b]);
+#pragma unroll 4
+    for (int k = k0 + lane; k < e; k += 32) {
+      const int c = l.col[k];
+      const uint32_t bit = 1u << (c & 31);
+      if (!(*(volatile uint32_t*)&right[c >> 5].x & bit)) atomicOr(&right[c >> 5].x, bit);
+    }
+  }
+}
+
+// ... then the numbers before each word, and the columns.
+__global__ void front_right_list_kernel(FrontLevel l) {
+  __shared__ int32_t sh[32];
+  __shared__ int32_t s_carry, s_at;
+  const int nb = min(l.ctr->nblocks, l.cap);
+  const int words = (l.n + 31) >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int b = blockIdx.x; b < nb; b += gridDim.x) {
+    uint2* right = l.right + (size_t)b * words;
+    __syncthreads();
+    if (threadIdx.x == 0) s_carry = 0;
+    __syncthreads();
+    for (int w0 = 0; w0 < words; w0 += blockDim.x) {
+      const int w = w0 + threadIdx.x;
+      const int v = w < words ? __popc(right[w].x) : 0;
+      int s = v;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(FULL, s, o);
+        if (lane >= o) s += x;
+      }
+      if (lane == 31) sh[warp] = s;
+      __syncthreads();
+      int before = s_carry, all = 0;
+      for (int k = 0; k < nw; k++) {
+        if (k < warp) before += sh[k];
+        all += sh[k];
+      }
+      if (w < words) right[w].y = (uint32_t)(before + s - v);
+      __syncthreads();
+      if (threadIdx.x == 0) s_carry += all;
+      __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+      const int count = s_carry;
+      s_at = atomicAdd(&l.ctr->bc_total, count);
+      if (s_at + count > l.bc_cap) l.ctr->overflow = 1;
+      l.b_nb[b] = count;
+      l.b_bc[b] = s_at;
+    }
+    __syncthreads();
+    if (s_at + s_carry <= l.bc_cap)
+      for (int w = threadIdx.x; w < words; w += blockDim.x) {
+        int at = s_at + (int)right[w].y;
+        for (uint32_t m = right[w].x; m; m &= m - 1) l.bc[at++] = 32 * w + __ffs(m) - 1;
+      }
+  }
+}
+
 // Entries a reduced row may have: those outside blocks (counted) and all columns right of
 // the blocks below it.
 __global__ void front_bound_kernel(FrontLevel l) {
@@ -319,20 +412,23 @@ __global__ void front_reduce_kernel(FrontLevel l, int32_t n1, const FrontMat* fr
                                     int32_t* beg1, int32_t* end1, int32_t* col1, int32_t* gid1) {
   extern __shared__ uint32_t sm[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const int words = (n1 + 31) >> 5;
-  uint32_t* set = sm + (size_t)warp * words;
-  for (int w = lane; w < words; w += 32) set[w] = 0u;
+  const int words = (n1 + 31) >> 5, swords = (words + 31) >> 5;
+  uint32_t* set = sm + (size_t)warp * (words + swords);
+  uint32_t* sum = set + words;  // one bit per nonzero word
+  for (int w = lane; w < words + swords; w += 32) set[w] = 0u;
   __syncwarp();
+  auto put = [&](int x) {
+    const uint32_t bit = 1u << (x & 31);
+    const uint32_t old = atomicOr(set + (x >> 5), bit);
+    if (old == 0u) atomicOr(sum + (x >> 10), 1u << ((x >> 5) & 31));
+  };
   for (int i = blockIdx.x * nw + warp; i < l.n; i += gridDim.x * nw) {
     if (l.blk[i] >= 0) continue;
     const int v = l.gid ? l.gid[i] : i;
     const int e = l.end[i];
     for (int k = l.beg[i] + lane; k < e; k += 32) {
       const int c = l.col[k];
-      if (l.blk[c] < 0) {
-        const int x = (int)l.rank[c];
-        atomicOr(set + (x >> 5), 1u << (x & 31));
-      }
+      if (l.blk[c] < 0) put((int)l.rank[c]);
     }
     // this level's pieces are the newest on the vertex's list
     for (int p = l.head[v]; p >= l.pieces_before; p = l.piece_next[p]) {
@@ -341,8 +437,7 @@ __global__ void front_reduce_kernel(FrontLevel l, int32_t n1, const FrontMat* fr
       const uint32_t* row = bits + f.bits_base + (size_t)l.piece_row[p] * W + pivots;
       for (int w = lane; w < W - pivots; w += 32) {
         for (uint32_t m = row[w]; m; m &= m - 1) {
-          const int x = (int)l.rank[l.bc[f.bc_base + 32 * w + __ffs(m) - 1]];
-          atomicOr(set + (x >> 5), 1u << (x & 31));
+          put((int)l.rank[l.bc[f.bc_base + 32 * w + __ffs(m) - 1]]);
         }
       }
     }
@@ -353,10 +448,11 @@ __global__ void front_reduce_kernel(FrontLevel l, int32_t n1, const FrontMat* fr
       beg1[to] = at;
       gid1[to] = v;
     }
-    for (int w0 = 0; w0 < words; w0 += 32) {
-      const int w = w0 + lane;
-      uint32_t m = w < words ? set[w] : 0u;
-      if (!__any_sync(FULL, m != 0u)) continue;
+    for (int sw = 0; sw < swords; sw++) {
+      const uint32_t some = sum[sw];
+      if (!some) continue;
+      const int w = 32 * sw + lane;
+      uint32_t m = (some >> lane) & 1u ? set[w] : 0u;
       if (m) set[w] = 0u;
       const int cnt = __popc(m);
       int s = cnt;
@@ -369,6 +465,8 @@ __global__ void front_reduce_kernel(FrontLevel l, int32_t n1, const FrontMat* fr
       at += __shfl_sync(FULL, s, 31);
     }
     if (lane == 0) end1[to] = at;
+    __syncwarp();
+    for (int sw = lane; sw < swords; sw += 32) sum[sw] = 0u;
     __syncwarp();
   }
 }
@@ -447,13 +545,19 @@ __global__ void __launch_bounds__(256) front_expand_kernel(FrontEmit e) {
     int32_t* U = e.U_colidx + e.U_rowptr[v];
     if (lane == 0) U[0] = v;
     U++;
-    for (int w = r >> 5; w < b.W; w++) {
-      uint32_t m = row[w];
-      if (w == r >> 5) m &= gt_bits(r & 31);
-      if (!m) continue;
-      if ((m >> lane) & 1u)
-        U[__popc(m & lt_bits(lane))] = w < b.pivots ? b.cols[32 * w + lane] : b.bcols[32 * (w - b.pivots) + lane];
-      U += __popc(m);
+    for (int w0 = r >> 5; w0 < b.W; w0 += 32) {
+      uint32_t mine = w0 + lane < b.W ? row[w0 + lane] : 0u;
+      if (w0 + lane == r >> 5) mine &= gt_bits(r & 31);
+      unsigned any = __ballot_sync(FULL, mine != 0u);
+      while (any) {
+        const int k = __ffs(any) - 1;
+        any &= any - 1;
+        const uint32_t m = __shfl_sync(FULL, mine, k);
+        const int w = w0 + k;
+        if ((m >> lane) & 1u)
+          U[__popc(m & lt_bits(lane))] = w < b.pivots ? b.cols[32 * w + lane] : b.bcols[32 * (w - b.pivots) + lane];
+        U += __popc(m);
+      }
     }
     // the pieces of L
     int np = 0;
@@ -508,19 +612,24 @@ __global__ void __launch_bounds__(256) front_expand_kernel(FrontEmit e) {
           base += __reduce_add_sync(FULL, c);
         }
       }
-      for (int w = 0; w < me.words; w++) {
-        uint32_t m = me.row[w];
-        if (w == me.words - 1) m &= me.mask;
-        if (!m) continue;
-        if ((m >> lane) & 1u) {
-          const int c = me.cols[32 * w + lane];
-          int at = base + __popc(m & lt_bits(lane));
-          if (lower)
-            for (int q = 0; q < np; q++)
-              if (pc[q].level < me.level && pc[q].last < c) at += pc[q].count;
-          L[at] = c;
+      for (int w0 = 0; w0 < me.words; w0 += 32) {
+        uint32_t mine = w0 + lane < me.words ? me.row[w0 + lane] : 0u;
+        if (w0 + lane == me.words - 1) mine &= me.mask;
+        unsigned any = __ballot_sync(FULL, mine != 0u);
+        while (any) {
+          const int k = __ffs(any) - 1;
+          any &= any - 1;
+          const uint32_t m = __shfl_sync(FULL, mine, k);
+          if ((m >> lane) & 1u) {
+            const int c = me.cols[32 * (w0 + k) + lane];
+            int at = base + __popc(m & lt_bits(lane));
+            if (lower)
+              for (int q = 0; q < np; q++)
+                if (pc[q].level < me.level && pc[q].last < c) at += pc[q].count;
+            L[at] = c;
+          }
+          base += __popc(m);
         }
-        base += __popc(m);
       }
     }
     __syncwarp();
@@ -536,26 +645,35 @@ int grid_for(long long threads, int block, int most) {
 }  // namespace
 
 cudaError_t launch_front_blocks(const FrontLevel& l, cudaStream_t st) {
-  front_low_kernel<<<grid_for(8LL * l.n, 256, 8192), 256, 0, st>>>(l);
+  if (l.wide) front_low_kernel<32><<<grid_for(32LL * l.n, 256, 8192), 256, 0, st>>>(l);
+  else front_low_kernel<8><<<grid_for(8LL * l.n, 256, 8192), 256, 0, st>>>(l);
   const int tiles = (l.n + TILE - 1) / TILE;
-  front_stretch_kernel<<<tiles, 128, 0, st>>>(l);
+  front_stretch_kernel<<<tiles, 1024, 0, st>>>(l);
   front_pick_kernel<<<tiles, 1024, 0, st>>>(l);
   front_mark_kernel<<<grid_for(l.cap, 1, 4096), 256, 0, st>>>(l);
   return cudaGetLastError();
 }
 
 cudaError_t launch_front_above(const FrontLevel& l, cudaStream_t st) {
-  front_runs_kernel<false><<<grid_for(8LL * l.n, 256, 8192), 256, 0, st>>>(l);
+  const int g8 = grid_for(8LL * l.n, 256, 8192), g32 = grid_for(32LL * l.n, 256, 8192);
+  if (l.wide) front_runs_kernel<false, 32><<<g32, 256, 0, st>>>(l);
+  else front_runs_kernel<false, 8><<<g8, 256, 0, st>>>(l);
   front_offsets_kernel<<<1, 1024, 0, st>>>(l);
-  front_runs_kernel<true><<<grid_for(8LL * l.n, 256, 8192), 256, 0, st>>>(l);
-  front_right_kernel<<<grid_for(l.cap, 1, 2048), 512, 0, st>>>(l);
+  if (l.wide) front_runs_kernel<true, 32><<<g32, 256, 0, st>>>(l);
+  else front_runs_kernel<true, 8><<<g8, 256, 0, st>>>(l);
+  if (l.wide) {
+    front_right_set_kernel<<<g32, 256, 0, st>>>(l);
+    front_right_list_kernel<<<grid_for(l.cap, 1, 2048), 512, 0, st>>>(l);
+  } else {
+    front_right_kernel<<<grid_for(l.cap, 1, 2048), 512, 0, st>>>(l);
+  }
   front_bound_kernel<<<grid_for(l.n, 256, 1024), 256, 0, st>>>(l);
   return cudaGetLastError();
 }
 
 cudaError_t launch_front_reduce(const FrontLevel& l, int32_t n1, const FrontMat* fronts, const uint32_t* bits,
                                 int32_t* beg, int32_t* end, int32_t* col, int32_t* gid, cudaStream_t st) {
-  const size_t per = 4 * (size_t)((n1 + 31) / 32);
+  const size_t per = 4 * ((size_t)((n1 + 31) / 32) + (size_t)((n1 + 1023) / 1024));
   int nw = 16;
   while (nw > 1 && per * nw > 96 * 1024) nw >>= 1;
   const cudaError_t e =

@@ -5,7 +5,7 @@
 
 namespace gsofa {
 
-constexpr int FRONT_BLOCK_MAX = 1024;  // vertices of a block
+constexpr int FRONT_BLOCK_MAX = 1024;  // vertices of a block at most
 constexpr int FRONT_BLOCK_MIN = 64;    // smaller closed stretches are left to the next level
 constexpr int FRONT_PIECES = 64;       // blocks below one vertex at most
 constexpr int FRONT_BC_MAX = 4096;     // columns right of a block at most
@@ -23,9 +23,11 @@ struct FrontCounters {
 // col[beg[i] .. end[i]), increasing.
 struct FrontLevel {
   int32_t n;
+  int32_t block_max;   // vertices of a block at most on this level
+  int32_t wide;        // rows are long: a warp each, and columns right of blocks by bitmaps
   const int32_t *beg, *end, *col, *gid;
   int32_t* low;        // smallest neighbour in either direction (set to a large value before)
-  int32_t* best;       // per start: end of the largest closed stretch of at most FRONT_BLOCK_MAX (-1: none)
+  int32_t* best;       // per start: end of the largest closed stretch of at most block_max (-1: none)
   int32_t* blk;        // per vertex: its block or -1
   int32_t* rem;        // per vertex: 1 where it stays for the next level
   const int64_t* rank; // exclusive sums of rem
@@ -37,6 +39,7 @@ struct FrontLevel {
   int32_t *br_row, *br_b, *br_e;  // rows above blocks: vertex, entries in the block's columns
   int32_t* bc;         // columns right of blocks
   int32_t bc_cap;
+  uint2* right;        // wide: per block and 32 vertices, the columns right of it: bits, number before
   // per original vertex
   int32_t* own;        // block it is eliminated in (over all levels)
   int32_t* own_row;
