@@ -761,6 +761,9 @@ void band_times(Events& ev, gsofa_stats* s) {
 constexpr int32_t FRONT_MIN_ORDER = 16384;
 constexpr int32_t FRONT_LAST_ORDER = 2900;
 constexpr int32_t FRONT_FIRST_BLOCK = 512;
+// threads of a front where there are more fronts than SMs: two CTAs fit an SM (1024 x 1024
+// grid 5.56 -> 5.23 ms; 256 the same, 192 5.32, 128 5.82)
+constexpr int FRONT_MANY_THREADS = 384;
 
 // Pool memory of one call, freed together.
 struct Held {
@@ -805,6 +808,9 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
   l.piece_next = keep.get<int32_t>(pcap);
   l.piece_blk = keep.get<int32_t>(pcap);
   l.piece_row = keep.get<int32_t>(pcap);
+  l.piece_nL = keep.get<int32_t>(pcap);
+  int32_t* nL = keep.get<int32_t>(n);
+  int32_t* nU = keep.get<int32_t>(n);
   l.piece_cap = pcap;
   int32_t* gid0 = keep.get<int32_t>(n);
   if (!keep.ok) return GSOFA_OK;
@@ -821,6 +827,8 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
   l.col = ci;
   l.gid = gid0;
   std::vector<FrontBlock> blocks;
+  FrontEmit e;
+  std::memset(&e, 0, sizeof(e));
   ev.rec(2, st);
   for (int level = 0; level < 16; level++) {
     std::vector<FrontMat> fronts;
@@ -863,6 +871,7 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
       l.br_e = level_mem.get<int32_t>(l.br_cap);
       l.bc_cap = l.n + 1024;
       l.bc = level_mem.get<int32_t>(l.bc_cap);
+      l.bc_next = level_mem.get<int32_t>(l.bc_cap);
       bcg = keep.get<int32_t>(l.bc_cap);
       if (!level_mem.ok || !keep.ok) return GSOFA_OK;
       l.ctr = (FrontCounters*)blk7;
@@ -912,7 +921,7 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
         m.id = b;
         fronts.push_back(m);
       }
-      if (fc->bc_total > 0) FK(launch_front_gids(l, l.bc, fc->bc_total, bcg, st));
+      if (fc->bc_total > 0) FK(launch_front_gids(l, fc->bc_total, bcg, st));
     }
     // launch shapes; bitmap rows one front after the other
     const size_t B = fronts.size();
@@ -962,11 +971,15 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
     f.right = whole ? nullptr : l.right;
     f.right_words = (l.n + 31) / 32;
     f.bits = bits;
+    f.gid = l.gid;
+    f.row_nL = nL;
+    f.row_nU = nU;
+    f.piece_nL = l.piece_nL + l.pieces_before;
     for (size_t b = 0; b < B;) {
       size_t k = b, most = 0;
       for (; k < B && cs[order[k]] == cs[order[b]]; k++) most = std::max(most, smem[order[k]]);
       f.first = (int32_t)b;
-      FK(launch_front_elim(f, (int)(k - b), cs[order[b]], most, st));
+      FK(launch_front_elim(f, (int)(k - b), cs[order[b]], (int)(k - b) > c->sms ? FRONT_MANY_THREADS : 512, most, st));
       *launches += 1;
       b = k;
     }
@@ -991,7 +1004,12 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
         q.nb = m.nb;
         q.pivots = (m.sz + 31) / 32;
         q.W = q.pivots + (m.nb + 31) / 32;
+        q.first = level == 0 ? m.first_vertex : -1;
         blocks.push_back(q);
+      }
+      if (level == 0) {
+        e.left_gid = gid1;
+        e.left = n1;
       }
       level_mem.free_all();
       std::swap(level_mem.ptrs, next_mem.ptrs);
@@ -1016,6 +1034,7 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
       q.nb = m.nb;
       q.pivots = (m.sz + 31) / 32;
       q.W = q.pivots + (m.nb + 31) / 32;
+      q.first = level == 0 ? m.first_vertex : -1;
       blocks.push_back(q);
     }
     n1 = -1;
@@ -1031,8 +1050,6 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
   // sizes, then columns and supernodes
   FrontBlock* d_blocks = keep.get<FrontBlock>(blocks.size());
   FrontBlock* stage = (FrontBlock*)thread_pinned(sizeof(FrontBlock) * blocks.size(), 0);
-  int32_t* nL = keep.get<int32_t>(n);
-  int32_t* nU = keep.get<int32_t>(n);
   int32_t* flags = keep.get<int32_t>(n);
   int64_t* pos = keep.get<int64_t>((size_t)n + 1);
   void* tmp = keep.get<unsigned char>(scan_tmp_bytes(n));
@@ -1056,8 +1073,6 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
   } while (0)
   std::memcpy(stage, blocks.data(), sizeof(FrontBlock) * blocks.size());
   RK(cudaMemcpyAsync(d_blocks, stage, sizeof(FrontBlock) * blocks.size(), cudaMemcpyHostToDevice, st));
-  FrontEmit e;
-  std::memset(&e, 0, sizeof(e));
   e.n = n;
   e.blocks = d_blocks;
   e.own = l.own;
@@ -1066,6 +1081,7 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
   e.piece_next = l.piece_next;
   e.piece_blk = l.piece_blk;
   e.piece_row = l.piece_row;
+  e.piece_nL = l.piece_nL;
   e.row_nL = nL;
   e.row_nU = nU;
   e.fill = fill;

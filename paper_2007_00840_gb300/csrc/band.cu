@@ -810,9 +810,23 @@ __global__ void __launch_bounds__(512, 1) front_elim_kernel(FrontArgs a) {
         const uint32_t* x = panel_rows<C>(B, P);
         const uint32_t* pu = S.pu + (size_t)32 * B.us * (P & 1);
         uint32_t* o = out + (size_t)32 * P * W;
-        for (int r = warp - 1; r < rows; r += nwk)
-          for (int c = lane; c < W; c += 32)
-            o[(size_t)r * W + c] = c < P ? x[r * B.xs + c] : (c == P ? S.pw[32 * (P & 1) + r] : pu[r * B.us + c - P - 1]);
+        for (int r = warp - 1; r < rows; r += nwk) {
+          uint32_t cnt = 0u;  // entries below the diagonal, and 2^16 times those above
+          for (int c = lane; c < W; c += 32) {
+            const uint32_t w =
+                c < P ? x[r * B.xs + c] : (c == P ? S.pw[32 * (P & 1) + r] : pu[r * B.us + c - P - 1]);
+            o[(size_t)r * W + c] = w;
+            if (c < P) cnt += __popc(w);
+            else if (c > P) cnt += __popc(w) << 16;
+            else cnt += __popc(w & lt_mask(r)) + (__popc(w & gt_mask(r)) << 16);
+          }
+          cnt = __reduce_add_sync(FULL, cnt);
+          if (lane == 0) {
+            const int v = a.gid[d.first_vertex + 32 * P + r];
+            a.row_nL[v] = (int)(cnt & 0xFFFFu);
+            a.row_nU[v] = (int)(cnt >> 16) + 1;
+          }
+        }
       }
     }
     if constexpr (C > 1) {
@@ -832,7 +846,14 @@ __global__ void __launch_bounds__(512, 1) front_elim_kernel(FrontArgs a) {
     if (q % C != rank) continue;
     const uint32_t* row = panel_rows<C>(B, q) + (i & 31) * B.xs;
     uint32_t* o = out + (size_t)(32 * pivots + i) * W;
-    for (int c = lane; c < W; c += 32) o[c] = row[c];
+    int cnt = 0;
+    for (int c = lane; c < W; c += 32) {
+      const uint32_t w = row[c];
+      o[c] = w;
+      if (c < pivots) cnt += __popc(w);
+    }
+    cnt = __reduce_add_sync(FULL, cnt);
+    if (lane == 0) a.piece_nL[d.br_base + i] = cnt;
   }
 }
 
@@ -1120,13 +1141,13 @@ size_t front_smem_bytes(int sz, int nr, int nb, int C) {
 
 namespace {
 template <int C>
-cudaError_t launch_front(const FrontArgs& a, int count, size_t smem, cudaStream_t st) {
+cudaError_t launch_front(const FrontArgs& a, int count, int threads, size_t smem, cudaStream_t st) {
   cudaError_t e =
       cudaFuncSetAttribute(front_elim_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, BAND_SMEM_MAX);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(count * C));
-  cfg.blockDim = dim3(512);
+  cfg.blockDim = dim3((unsigned)threads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
@@ -1140,13 +1161,13 @@ cudaError_t launch_front(const FrontArgs& a, int count, size_t smem, cudaStream_
 }
 }  // namespace
 
-cudaError_t launch_front_elim(const FrontArgs& a, int count, int C, size_t smem, cudaStream_t st) {
+cudaError_t launch_front_elim(const FrontArgs& a, int count, int C, int threads, size_t smem, cudaStream_t st) {
   if (count <= 0) return cudaSuccess;
   switch (C) {
-    case 1: return launch_front<1>(a, count, smem, st);
-    case 2: return launch_front<2>(a, count, smem, st);
-    case 4: return launch_front<4>(a, count, smem, st);
-    default: return launch_front<8>(a, count, smem, st);
+    case 1: return launch_front<1>(a, count, threads, smem, st);
+    case 2: return launch_front<2>(a, count, threads, smem, st);
+    case 4: return launch_front<4>(a, count, threads, smem, st);
+    default: return launch_front<8>(a, count, threads, smem, st);
   }
 }
 

@@ -66,10 +66,13 @@ struct FrontArgs {
   const uint2* right;              // their places (FrontLevel::right), or null: searched in bc
   int32_t right_words;             // words of a block in right
   uint32_t* bits;
+  const int32_t* gid;              // vertices of the level: original numbers
+  int32_t *row_nL, *row_nU;        // per original vertex: entries of its own row in the block, and from the diagonal on
+  int32_t* piece_nL;               // per row above a block: its entries in the block
 };
 
 size_t front_smem_bytes(int sz, int nr, int nb, int C);
-cudaError_t launch_front_elim(const FrontArgs& a, int count, int C, size_t smem, cudaStream_t st);
+cudaError_t launch_front_elim(const FrontArgs& a, int count, int C, int threads, size_t smem, cudaStream_t st);
 
 size_t band_smem_bytes(int LB, int UB, int C);
 struct BandShape {

@@ -396,6 +396,39 @@ __global__ void front_right_list_kernel(FrontLevel l) {
   }
 }
 
+// Calls put(column, rank) for the bits of 32 words, lane's word w0 + lane, and returns
+// their number: a lane per word and its bits in turn, or a lane per bit and the words in
+// turn, whichever has fewer turns.  (Four turns together are slower: 103 against 80 us for
+// the rows of a 512 x 512 grid, by the instructions for turns that are not there.)
+// AUX: also passes the word's aux.
+template <bool AUX = false, class F>
+__device__ __forceinline__ int each_bit(uint32_t mine, int w0, F put, int aux = 0) {
+  const int lane = threadIdx.x & 31;
+  unsigned any = __ballot_sync(FULL, mine != 0u);
+  if (!any) return 0;
+  const int cnt = __popc(mine);
+  if (__reduce_max_sync(FULL, cnt) < __popc(any)) {
+    int s = cnt;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(FULL, s, o);
+      if (lane >= o) s += x;
+    }
+    int at = s - cnt;
+    for (uint32_t m = mine; m; m &= m - 1) put(32 * (w0 + lane) + __ffs(m) - 1, at++, aux);
+    return __shfl_sync(FULL, s, 31);
+  }
+  int before = 0;
+  while (any) {
+    const int k = __ffs(any) - 1;
+    any &= any - 1;
+    const uint32_t m = __shfl_sync(FULL, mine, k);
+    const int of = AUX ? __shfl_sync(FULL, aux, k) : 0;
+    if ((m >> lane) & 1u) put(32 * (w0 + k) + lane, before + __popc(m & lt_bits(lane)), of);
+    before += __popc(m);
+  }
+  return before;
+}
+
 // Entries a reduced row may have: those outside blocks (counted) and all columns right of
 // the blocks below it.
 __global__ void front_bound_kernel(FrontLevel l) {
@@ -422,22 +455,83 @@ __global__ void front_reduce_kernel(FrontLevel l, int32_t n1, const FrontMat* fr
     const uint32_t old = atomicOr(set + (x >> 5), bit);
     if (old == 0u) atomicOr(sum + (x >> 10), 1u << ((x >> 5) & 31));
   };
-  for (int i = blockIdx.x * nw + warp; i < l.n; i += gridDim.x * nw) {
-    if (l.blk[i] >= 0) continue;
+  const int step = gridDim.x * nw;
+  unsigned todo = 0u;
+  for (int i0 = blockIdx.x * nw + warp, base = i0;;) {
+    if (!todo) {  // the next of this warp's vertices that remain
+      if (i0 >= l.n) break;
+      base = i0;
+      const long long mine = (long long)i0 + (long long)lane * step;
+      todo = __ballot_sync(FULL, mine < l.n && l.blk[mine] < 0);
+      i0 = (int)min((long long)l.n, (long long)i0 + 32LL * step);
+      continue;
+    }
+    const int i = base + (__ffs(todo) - 1) * step;
+    todo &= todo - 1;
     const int v = l.gid ? l.gid[i] : i;
     const int e = l.end[i];
+#pragma unroll 4
     for (int k = l.beg[i] + lane; k < e; k += 32) {
       const int c = l.col[k];
       if (l.blk[c] < 0) put((int)l.rank[c]);
     }
-    // this level's pieces are the newest on the vertex's list
-    for (int p = l.head[v]; p >= l.pieces_before; p = l.piece_next[p]) {
-      const FrontMat f = fronts[l.piece_blk[p] - l.blocks_before];
-      const int pivots = (f.sz + 31) >> 5, W = pivots + ((f.nb + 31) >> 5);
-      const uint32_t* row = bits + f.bits_base + (size_t)l.piece_row[p] * W + pivots;
-      for (int w = lane; w < W - pivots; w += 32) {
-        for (uint32_t m = row[w]; m; m &= m - 1) {
-          put((int)l.rank[l.bc[f.bc_base + 32 * w + __ffs(m) - 1]]);
+    // this level's pieces are the newest on the vertex's list: a lane looks up each, then
+    // all lanes take its words.  A word's columns mostly follow one another on the next
+    // level too and go over as two words; the others column by column, four words in flight
+    // (all columns so, one after the other: 891 us on a level of 1M vertices, 47,000 left)
+    int p = l.head[v];
+    while (p >= l.pieces_before) {
+      int np = 0, id = -1;
+      for (; p >= l.pieces_before && np < 32; np++) {
+        if (lane == np) id = p;
+        p = l.piece_next[p];
+      }
+      const uint32_t* row = nullptr;
+      int nw_right = 0, bc0 = 0;
+      if (id >= 0) {
+        const FrontMat f = fronts[l.piece_blk[id] - l.blocks_before];
+        const int pivots = (f.sz + 31) >> 5;
+        nw_right = (f.nb + 31) >> 5;
+        row = bits + f.bits_base + (size_t)l.piece_row[id] * (pivots + nw_right) + pivots;
+        bc0 = f.bc_base;
+      }
+      for (int q = 0; q < np; q++) {
+        const uint32_t* x = (const uint32_t*)__shfl_sync(FULL, (unsigned long long)row, q);
+        const int nx = __shfl_sync(FULL, nw_right, q);
+        const int32_t* to = l.bc_next + __shfl_sync(FULL, bc0, q);
+        for (int w0 = 0; w0 < nx; w0 += 32) {
+          uint32_t mine = w0 + lane < nx ? x[w0 + lane] : 0u;
+          if (mine) {
+            const int32_t* t = to + 32 * (w0 + lane);
+            const int lo = __ffs(mine) - 1, hi = 31 - __clz(mine);
+            const int c = t[lo];
+            if (t[hi] - c == hi - lo) {
+              const uint32_t m = mine >> lo, m1 = (c & 31) ? m >> (32 - (c & 31)) : 0u;
+              atomicOr(set + (c >> 5), m << (c & 31));
+              atomicOr(sum + (c >> 10), 1u << ((c >> 5) & 31));
+              if (m1) {
+                atomicOr(set + (c >> 5) + 1, m1);
+                atomicOr(sum + ((c >> 5) + 1 >> 5), 1u << (((c >> 5) + 1) & 31));
+              }
+              mine = 0u;
+            }
+          }
+          unsigned any = __ballot_sync(FULL, mine != 0u);
+          while (any) {
+            int at[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+              at[j] = -1;
+              if (any) {
+                const int w = __ffs(any) - 1;
+                any &= any - 1;
+                if ((__shfl_sync(FULL, mine, w) >> lane) & 1u) at[j] = to[32 * (w0 + w) + lane];
+              }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+              if (at[j] >= 0) put(at[j]);
+          }
         }
       }
     }
@@ -454,15 +548,7 @@ __global__ void front_reduce_kernel(FrontLevel l, int32_t n1, const FrontMat* fr
       const int w = 32 * sw + lane;
       uint32_t m = (some >> lane) & 1u ? set[w] : 0u;
       if (m) set[w] = 0u;
-      const int cnt = __popc(m);
-      int s = cnt;
-      for (int o = 1; o < 32; o <<= 1) {
-        const int x = __shfl_up_sync(FULL, s, o);
-        if (lane >= o) s += x;
-      }
-      int to_at = at + s - cnt;
-      for (; m; m &= m - 1) col1[to_at++] = 32 * w + __ffs(m) - 1;
-      at += __shfl_sync(FULL, s, 31);
+      at += each_bit(m, 32 * sw, [&](int c, int k, int) { col1[at + k] = c; });
     }
     if (lane == 0) end1[to] = at;
     __syncwarp();
@@ -483,156 +569,226 @@ __global__ void front_iota_kernel(int32_t* out, int32_t n) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) out[i] = i;
 }
 
-__global__ void front_gids_kernel(const int32_t* gid, const int32_t* cols, int32_t count, int32_t* out) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x)
-    out[i] = gid ? gid[cols[i]] : cols[i];
+__global__ void front_gids_kernel(FrontLevel l, int32_t count, int32_t* out) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
+    const int c = l.bc[i];
+    out[i] = l.gid ? l.gid[c] : c;
+    l.bc_next[i] = (int)l.rank[c];
+  }
 }
 
 // ------------------------------------------------------------ rows of the result
-// One warp per vertex: sizes.
+// Row sizes: the own row of a vertex and its pieces, counted where they were written.
 __global__ void front_count_kernel(FrontEmit e) {
+  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < e.n; v += gridDim.x * blockDim.x) {
+    int nl = e.row_nL[v];
+    for (int p = e.head[v]; p >= 0; p = e.piece_next[p]) nl += e.piece_nL[p];
+    e.row_nL[v] = nl;
+    e.fill[v] = nl + e.row_nU[v] - e.fill[v];
+  }
+}
+
+// Column c of a block's bitmap rows.  The blocks of the first level are consecutive vertices.
+__device__ __forceinline__ int block_column(const FrontBlock& b, int c) {
+  if (c >= 32 * b.pivots) return __ldg(b.bcols + c - 32 * b.pivots);
+  return b.first >= 0 ? b.first + c : __ldg(b.cols + c);
+}
+
+// Columns of the rows without pieces, by far the most: one bitmap row holds L, the diagonal
+// and U as they stand.  A warp looks EXPAND_ROWS of them up together.
+constexpr int EXPAND_ROWS = 8;
+__global__ void __launch_bounds__(256) front_expand_kernel(FrontEmit e) {
   const int lane = threadIdx.x & 31;
-  const int step = (gridDim.x * blockDim.x) >> 5;
-  for (int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < e.n; v += step) {
-    const FrontBlock b = e.blocks[e.own[v]];
-    const int r = e.own_row[v];
-    const uint32_t* row = b.bits + (size_t)r * b.W;
-    int nl = 0, nu = 0;
-    for (int w = lane; w < b.W; w += 32) {
-      const uint32_t m = row[w];
-      if (w < r >> 5) nl += __popc(m);
-      else if (w > r >> 5) nu += __popc(m);
-      else {
-        nl += __popc(m & lt_bits(r & 31));
-        nu += __popc(m & gt_bits(r & 31));
+  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
+  for (int v0 = gw * EXPAND_ROWS; v0 < e.n; v0 += nwarps * EXPAND_ROWS) {
+    const int many = min(EXPAND_ROWS, e.n - v0);
+    int my_blk = 0, my_row = 0, my_nl = 0;
+    long long my_L = 0, my_U = 0;
+    bool mine_too = false;
+    if (lane < many) {
+      mine_too = e.head[v0 + lane] < 0;
+      my_blk = e.own[v0 + lane];
+      my_row = e.own_row[v0 + lane];
+      my_nl = e.row_nL[v0 + lane];
+      my_L = e.L_rowptr[v0 + lane];
+      my_U = e.U_rowptr[v0 + lane];
+    }
+    for (unsigned todo = __ballot_sync(FULL, mine_too); todo; todo &= todo - 1) {
+      const int j = __ffs(todo) - 1;
+      const FrontBlock b = e.blocks[__shfl_sync(FULL, my_blk, j)];
+      const int r = __shfl_sync(FULL, my_row, j), nl = __shfl_sync(FULL, my_nl, j);
+      const uint32_t* row = b.bits + (size_t)r * b.W;
+      int32_t* L = e.L_colidx + __shfl_sync(FULL, my_L, j);
+      int32_t* U = e.U_colidx + __shfl_sync(FULL, my_U, j) + 1;
+      if (lane == 0) U[-1] = v0 + j;
+      int before = 0;
+      for (int w0 = 0; w0 < b.W; w0 += 32) {
+        uint32_t mine = w0 + lane < b.W ? row[w0 + lane] : 0u;
+        if (w0 + lane == r >> 5) mine &= ~(1u << (r & 31));
+        before += each_bit(mine, w0, [&](int c, int at, int) {
+          const int x = block_column(b, c);
+          at += before;
+          if (at < nl) L[at] = x;
+          else U[at - nl] = x;
+        });
       }
-    }
-    for (int p = e.head[v]; p >= 0; p = e.piece_next[p]) {
-      const FrontBlock q = e.blocks[e.piece_blk[p]];
-      const uint32_t* x = q.bits + (size_t)e.piece_row[p] * q.W;
-      for (int w = lane; w < q.pivots; w += 32) nl += __popc(x[w]);
-    }
-    nl = __reduce_add_sync(FULL, nl);
-    nu = __reduce_add_sync(FULL, nu) + 1;
-    if (lane == 0) {
-      e.row_nL[v] = nl;
-      e.row_nU[v] = nu;
-      e.fill[v] = nl + nu - e.fill[v];
     }
   }
 }
 
-// One warp per vertex: columns.  L(v,:) comes from the vertex's pieces and the lower part
-// of its own row (the last piece).  An entry's place is its rank in its piece plus the
-// sizes of the pieces before it: of pieces of its level or below, those that end before
-// it; of pieces above, their entries before its block.
-__global__ void __launch_bounds__(256) front_expand_kernel(FrontEmit e) {
+// Columns of the rows with pieces, a CTA each.  L(v,:) comes from the vertex's pieces and
+// the lower part of its own row (the last piece).  An entry's place is its rank in its piece
+// plus the sizes of the pieces before it: of pieces of its level or below, those that end
+// before it; of pieces above, their entries before its block.  Only vertices that the first
+// level leaves have pieces; a CTA takes one, the last separators', which are longest, first.
+// (One warp per vertex: 247 us on a 512 x 512 grid; CTAs that look for their vertices among
+// all: 144 to 190.)
+constexpr int MERGE_PAIRS = 512;
+__global__ void __launch_bounds__(64) front_merge_kernel(FrontEmit e) {
   struct Piece {
     const uint32_t* row;
     const int32_t* cols;
-    int words, size, level, first, last, count;
+    int words, size, level, first, last, count, base, order;
     uint32_t mask;  // of the last word
   };
-  __shared__ Piece s_piece[8][FRONT_PIECES + 1];
+  __shared__ Piece pc[FRONT_PIECES + 1];
+  __shared__ int sorted[FRONT_PIECES + 1], s_sum[2][FRONT_PIECES + 2], s_np, s_pairs;
+  __shared__ uint16_t pair[MERGE_PAIRS];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  Piece* pc = s_piece[warp];
-  const int step = (gridDim.x * blockDim.x) >> 5;
-  for (int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; v < e.n; v += step) {
+  int* sum = s_sum[warp];
+  for (int i = blockIdx.x; i < e.left; i += gridDim.x) {
+    const int v = e.left_gid[e.left - 1 - i];
+    if (e.head[v] < 0) continue;
     const FrontBlock b = e.blocks[e.own[v]];
-    const int r = e.own_row[v];
+    const int r = e.own_row[v], nl = e.row_nL[v];
     const uint32_t* row = b.bits + (size_t)r * b.W;
-    // U: the diagonal, the block's columns above v, the columns right of the block
-    int32_t* U = e.U_colidx + e.U_rowptr[v];
-    if (lane == 0) U[0] = v;
-    U++;
-    for (int w0 = r >> 5; w0 < b.W; w0 += 32) {
-      uint32_t mine = w0 + lane < b.W ? row[w0 + lane] : 0u;
-      if (w0 + lane == r >> 5) mine &= gt_bits(r & 31);
-      unsigned any = __ballot_sync(FULL, mine != 0u);
-      while (any) {
-        const int k = __ffs(any) - 1;
-        any &= any - 1;
-        const uint32_t m = __shfl_sync(FULL, mine, k);
-        const int w = w0 + k;
-        if ((m >> lane) & 1u)
-          U[__popc(m & lt_bits(lane))] = w < b.pivots ? b.cols[32 * w + lane] : b.bcols[32 * (w - b.pivots) + lane];
-        U += __popc(m);
-      }
-    }
-    // the pieces of L
-    int np = 0;
-    for (int p = e.head[v]; p >= 0; p = e.piece_next[p]) {
-      if (lane == 0) {
-        const FrontBlock q = e.blocks[e.piece_blk[p]];
-        pc[np] = Piece{q.bits + (size_t)e.piece_row[p] * q.W, q.cols, q.pivots, q.sz, q.level, q.cols[0], q.cols[q.sz - 1], 0, FULL};
-      }
-      np++;
-    }
-    if (lane == 0) pc[np] = Piece{row, b.cols, (r >> 5) + 1, r, b.level, b.cols[0], v - 1, 0, lt_bits(r & 31)};
-    np++;
-    __syncwarp();
-    for (int p = 0; p < np; p++) {
-      int c = 0;
-      for (int w = lane; w < pc[p].words; w += 32) {
-        uint32_t m = pc[p].row[w];
-        if (w == pc[p].words - 1) m &= pc[p].mask;
-        c += __popc(m);
-      }
-      c = __reduce_add_sync(FULL, c);
-      if (lane == 0) pc[p].count = c;
-    }
-    __syncwarp();
     int32_t* L = e.L_colidx + e.L_rowptr[v];
-    for (int p = 0; p < np; p++) {
+    int32_t* U = e.U_colidx + e.U_rowptr[v];
+    if (warp == 0) {
+      int np = 0, count = 0;
+      for (int p = e.head[v]; p >= 0;) {  // a lane looks up each piece
+        int id = -1, some = 0;
+        for (; p >= 0 && some < 32; some++) {
+          if (lane == some) id = p;
+          p = e.piece_next[p];
+        }
+        if (id >= 0) {
+          const FrontBlock q = e.blocks[e.piece_blk[id]];
+          const int nq = e.piece_nL[id];
+          pc[np + lane] = Piece{q.bits + (size_t)e.piece_row[id] * q.W, q.cols, q.pivots, q.sz, q.level, q.cols[0],
+                                q.cols[q.sz - 1], nq, 0, 0, FULL};
+          count += nq;
+        }
+        np += some;
+      }
+      const int own = nl - __reduce_add_sync(FULL, count);
+      if (lane == 0) {
+        pc[np] = Piece{row, b.cols, (r >> 5) + 1, r, b.level, b.cols[0], v - 1, own, 0, 0, lt_bits(r & 31)};
+        s_np = np + 1;
+        s_pairs = 0;
+        U[0] = v;
+      }
+    }
+    __syncthreads();
+    const int np = s_np;
+    // a pair of pieces per thread: their order by last column, and the entries before a piece's
+    // block in pieces of its level or above.  Those that need a search are few and collected
+    // first (with a search wherever a pair comes up, rows of 60 pieces took 100 us)
+    auto before_block = [&](int p, int q) {
+      const int first = pc[p].first;
+      const int32_t* cols = pc[q].cols;
+      int lo = 0, hi = pc[q].size;  // columns of q below first: its first lo
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(cols + mid) < first) lo = mid + 1; else hi = mid;
+      }
+      const uint32_t* words = pc[q].row;
+      const int last = pc[q].words - 1;
+      int c = 0;
+#pragma unroll 8
+      for (int w = 0; w < lo >> 5; w++) c += __popc(__ldg(words + w) & (w == last ? pc[q].mask : FULL));
+      if (lo & 31) c += __popc(words[lo >> 5] & lt_bits(lo & 31) & (lo >> 5 == last ? pc[q].mask : FULL));
+      if (c) atomicAdd(&pc[p].base, c);
+    };
+    for (int x = threadIdx.x; x < np * np; x += blockDim.x) {
+      const int p = x / np, q = x - p * np;
+      if (p == q) continue;
+      if (pc[q].last < pc[p].last || (pc[q].last == pc[p].last && q < p)) atomicAdd(&pc[p].order, 1);
+      if (pc[p].count == 0 || pc[q].count == 0 || pc[q].level < pc[p].level) continue;
+      if (pc[q].last < pc[p].first) {
+        atomicAdd(&pc[p].base, pc[q].count);
+      } else if (pc[q].level > pc[p].level && pc[q].first < pc[p].first) {
+        const int at = atomicAdd(&s_pairs, 1);
+        if (at < MERGE_PAIRS) pair[at] = (uint16_t)(p << 8 | q);
+        else before_block(p, q);
+      }
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < min(s_pairs, MERGE_PAIRS); x += blockDim.x) before_block(pair[x] >> 8, pair[x] & 255);
+    __syncthreads();
+    for (int p = threadIdx.x; p < np; p += blockDim.x) sorted[pc[p].order] = pc[p].last;
+    __syncthreads();
+    int level = -1;
+    for (int p = warp; p < np; p += blockDim.x >> 5) {
       const Piece me = pc[p];
       if (me.count == 0) continue;
-      // entries before this piece's block in pieces of its level or above
-      int base = 0;
-      bool lower = false;
-      for (int q = 0; q < np; q++) {
-        if (q == p || pc[q].count == 0) continue;
-        if (pc[q].level < me.level) {
-          lower = true;
-        } else if (pc[q].level == me.level) {
-          if (pc[q].last < me.first) base += pc[q].count;
-        } else {
-          // columns of q below me.first: its first `lo`
-          int lo = 0, hi = pc[q].size;
-          while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (pc[q].cols[mid] < me.first) lo = mid + 1; else hi = mid;
+      if (me.level != level) {
+        // pieces of levels below lie between this one's columns: sum[k] is the number of
+        // their entries among the first k by last column
+        level = me.level;
+        __syncwarp();
+        for (int q = lane; q < np; q += 32) sum[pc[q].order + 1] = pc[q].level < level ? pc[q].count : 0;
+        __syncwarp();
+        int carry = 0;
+        for (int q0 = 0; q0 < np; q0 += 32) {
+          int s = q0 + lane < np ? sum[q0 + lane + 1] : 0;
+          for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(FULL, s, o);
+            if (lane >= o) s += x;
           }
-          int c = 0;
-          for (int w = lane; w < pc[q].words && 32 * w < lo; w += 32) {
-            uint32_t m = pc[q].row[w];
-            if (w == pc[q].words - 1) m &= pc[q].mask;
-            if (lo - 32 * w < 32) m &= lt_bits(lo - 32 * w);
-            c += __popc(m);
-          }
-          base += __reduce_add_sync(FULL, c);
+          if (q0 + lane < np) sum[q0 + lane + 1] = carry + s;
+          carry += __shfl_sync(FULL, s, 31);
         }
+        if (lane == 0) sum[0] = 0;
+        __syncwarp();
       }
+      const bool below = sum[np] > 0;
+      int base = me.base;
       for (int w0 = 0; w0 < me.words; w0 += 32) {
         uint32_t mine = w0 + lane < me.words ? me.row[w0 + lane] : 0u;
         if (w0 + lane == me.words - 1) mine &= me.mask;
-        unsigned any = __ballot_sync(FULL, mine != 0u);
-        while (any) {
-          const int k = __ffs(any) - 1;
-          any &= any - 1;
-          const uint32_t m = __shfl_sync(FULL, mine, k);
-          if ((m >> lane) & 1u) {
-            const int c = me.cols[32 * (w0 + k) + lane];
-            int at = base + __popc(m & lt_bits(lane));
-            if (lower)
-              for (int q = 0; q < np; q++)
-                if (pc[q].level < me.level && pc[q].last < c) at += pc[q].count;
-            L[at] = c;
+        // entries of levels below before a word's columns: the same number for all where its
+        // first and last column have no piece between them (-1: they do)
+        auto pieces_before = [&](int x) {
+          int lo = 0, hi = np;
+          while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (sorted[mid] < x) lo = mid + 1; else hi = mid;
           }
-          base += __popc(m);
+          return lo;
+        };
+        int word_add = 0;
+        if (below && mine) {
+          const int32_t* cols = me.cols + 32 * (w0 + lane);
+          const int lo = pieces_before(__ldg(cols + __ffs(mine) - 1)), hi = pieces_before(__ldg(cols + 31 - __clz(mine)));
+          word_add = lo == hi ? sum[lo] : -1;
         }
+        base += each_bit<true>(mine, w0, [&](int c, int at, int add) {
+          const int x = __ldg(me.cols + c);
+          L[base + at + (add >= 0 ? add : sum[pieces_before(x)])] = x;
+        }, word_add);
       }
     }
-    __syncwarp();
+    // U: the block's columns above v and the columns right of the block
+    if (warp == np % (blockDim.x >> 5)) {
+      int before = 1;
+      for (int w0 = r >> 5; w0 < b.W; w0 += 32) {
+        uint32_t mine = w0 + lane < b.W ? row[w0 + lane] : 0u;
+        if (w0 + lane == r >> 5) mine &= gt_bits(r & 31);
+        before += each_bit(mine, w0, [&](int c, int at, int) { U[at + before] = block_column(b, c); });
+      }
+    }
+    __syncthreads();
   }
 }
 
@@ -693,19 +849,20 @@ cudaError_t launch_front_iota(int32_t* out, int32_t n, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_front_gids(const FrontLevel& l, const int32_t* cols, int32_t count, int32_t* out, cudaStream_t st) {
+cudaError_t launch_front_gids(const FrontLevel& l, int32_t count, int32_t* out, cudaStream_t st) {
   if (count <= 0) return cudaSuccess;
-  front_gids_kernel<<<grid_for(count, 256, 1024), 256, 0, st>>>(l.gid, cols, count, out);
+  front_gids_kernel<<<grid_for(count, 256, 1024), 256, 0, st>>>(l, count, out);
   return cudaGetLastError();
 }
 
 cudaError_t launch_front_count(const FrontEmit& e, cudaStream_t st) {
-  front_count_kernel<<<grid_for(32LL * e.n, 256, 16384), 256, 0, st>>>(e);
+  front_count_kernel<<<grid_for(e.n, 256, 16384), 256, 0, st>>>(e);
   return cudaGetLastError();
 }
 
 cudaError_t launch_front_expand(const FrontEmit& e, cudaStream_t st) {
-  front_expand_kernel<<<grid_for(32LL * e.n, 256, 16384), 256, 0, st>>>(e);
+  front_expand_kernel<<<grid_for(32LL * ((e.n + EXPAND_ROWS - 1) / EXPAND_ROWS), 256, 16384), 256, 0, st>>>(e);
+  if (e.left > 0) front_merge_kernel<<<e.left, 64, 0, st>>>(e);
   return cudaGetLastError();
 }
 

@@ -38,6 +38,7 @@ struct FrontLevel {
   int32_t *b_first, *b_size, *b_nr, *b_nb, *b_fill, *b_br, *b_bc;  // per block
   int32_t *br_row, *br_b, *br_e;  // rows above blocks: vertex, entries in the block's columns
   int32_t* bc;         // columns right of blocks
+  int32_t* bc_next;    // the same as vertices of the next level
   int32_t bc_cap;
   uint2* right;        // wide: per block and 32 vertices, the columns right of it: bits, number before
   // per original vertex
@@ -48,6 +49,7 @@ struct FrontLevel {
   int32_t* piece_next; // per piece
   int32_t* piece_blk;
   int32_t* piece_row;
+  int32_t* piece_nL;   // entries in the block
   int32_t blocks_before;  // blocks of earlier levels
   int32_t pieces_before;
   int32_t piece_cap, br_cap;
@@ -59,16 +61,18 @@ struct FrontBlock {
   const int32_t* cols;  // original numbers of its vertices
   const int32_t* bcols; // and of the columns right of it
   int32_t level, sz, nb, pivots, W;
-  int32_t pad;
+  int32_t first;        // its first vertex where they are consecutive, else -1
 };
 
 struct FrontEmit {
   int32_t n;
   const FrontBlock* blocks;
-  const int32_t *own, *own_row, *head, *piece_next, *piece_blk, *piece_row;
-  int32_t *row_nL, *row_nU, *fill;
+  const int32_t *own, *own_row, *head, *piece_next, *piece_blk, *piece_row, *piece_nL;
+  int32_t *row_nL, *row_nU, *fill;  // row_nL: of the own row alone before launch_front_count
   const int64_t *L_rowptr, *U_rowptr;
   int32_t *L_colidx, *U_colidx;
+  const int32_t* left_gid;          // vertices that the first level leaves, increasing
+  int32_t left;
 };
 
 cudaError_t launch_front_blocks(const FrontLevel& l, cudaStream_t st);   // low .. rem
@@ -79,7 +83,8 @@ cudaError_t launch_front_reduce(const FrontLevel& l, int32_t n1, const FrontMat*
                                 int32_t* beg, int32_t* end, int32_t* col, int32_t* gid, cudaStream_t st);
 cudaError_t launch_front_whole(const FrontLevel& l, cudaStream_t st);    // every vertex into block 0
 cudaError_t launch_front_iota(int32_t* out, int32_t n, cudaStream_t st);
-cudaError_t launch_front_gids(const FrontLevel& l, const int32_t* cols, int32_t count, int32_t* out, cudaStream_t st);
+// The columns right of blocks as original vertices and as vertices of the next level.
+cudaError_t launch_front_gids(const FrontLevel& l, int32_t count, int32_t* out, cudaStream_t st);
 cudaError_t launch_front_count(const FrontEmit& e, cudaStream_t st);
 cudaError_t launch_front_expand(const FrontEmit& e, cudaStream_t st);
 // Vertices of a next level that launch_front_reduce can take.
