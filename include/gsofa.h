@@ -301,6 +301,12 @@ void gsofa_server_destroy(gsofa_server *server);
  * them; the caller must not use them afterwards. */
 void gsofa_free(gsofa_result *res);
 
+/* A device array of *res as a DLPack managed tensor (DLManagedTensor*), field 0 .. 5 in the
+ * order L_rowptr, L_colidx, U_rowptr, U_colidx, fill_count, super_start.  It keeps the
+ * result's memory until its deleter is called, also after gsofa_free(res).  NULL for an
+ * empty array, a host result or a field that does not exist. */
+void *gsofa_dlpack(const gsofa_result *res, int32_t field);
+
 /* Human-readable name of an error code. */
 const char *gsofa_strerror(int code);
 

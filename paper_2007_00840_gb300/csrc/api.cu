@@ -16,6 +16,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <new>
 #include <thread>
 #include <vector>
 
@@ -70,6 +71,7 @@ struct Priv {
   void* host_block = nullptr;   // host results: one pinned block holding every array
   size_t host_cap = 0;
   SharedBlock* shared = nullptr;  // batch results: arrays point into this block
+  std::atomic<int> refs{1};       // the result, and every array of it handed out by gsofa_dlpack
 };
 
 // Pinned host blocks are expensive to create (page locking), so results of the
@@ -2513,9 +2515,58 @@ int gsofa_default_options(gsofa_options* opt) {
   return GSOFA_OK;
 }
 
+// The DLPack exchange format (version 0.x, the layout of its C structs): what a framework
+// takes as a tensor over memory that it does not own.
+struct DlpackTensor {
+  void* data;
+  int32_t device_type, device_id;
+  int32_t ndim;
+  uint8_t type_code, type_bits;
+  uint16_t type_lanes;
+  int64_t *shape, *strides;
+  uint64_t byte_offset;
+  void* manager;
+  void (*deleter)(DlpackTensor*);
+  // from here on ours
+  int64_t count;
+  gsofa_result res;
+};
+
+void* gsofa_dlpack(const gsofa_result* res, int32_t field) {
+  if (!res || !res->on_device || !res->_priv || field < 0 || field > 5) return nullptr;
+  Priv* pv = (Priv*)res->_priv;
+  void* const data[6] = {res->L_rowptr, res->L_colidx, res->U_rowptr, res->U_colidx, res->fill_count, res->super_start};
+  const int64_t count[6] = {(int64_t)res->n + 1, res->nnz_L, (int64_t)res->n + 1, res->nnz_U, res->n,
+                            (int64_t)res->n_super + 1};
+  if (!data[field] || count[field] == 0) return nullptr;
+  DlpackTensor* t = new (std::nothrow) DlpackTensor();
+  if (!t) return nullptr;
+  t->data = data[field];
+  t->device_type = 2;  // CUDA
+  t->device_id = pv->device;
+  t->ndim = 1;
+  t->type_code = 0;  // signed integers
+  t->type_bits = field == 0 || field == 2 ? 64 : 32;
+  t->type_lanes = 1;
+  t->count = count[field];
+  t->shape = &t->count;
+  t->strides = nullptr;  // contiguous
+  t->res = *res;
+  t->deleter = [](DlpackTensor* x) {
+    gsofa_free(&x->res);
+    delete x;
+  };
+  pv->refs.fetch_add(1);
+  return t;
+}
+
 void gsofa_free(gsofa_result* res) {
   if (!res) return;
   Priv* pv = (Priv*)res->_priv;
+  if (pv && pv->refs.fetch_sub(1) > 1) {  // arrays handed out hold the rest
+    std::memset(res, 0, sizeof(*res));
+    return;
+  }
   if (res->on_device && pv && pv->shared) {
     SharedBlock* b = pv->shared;
     if (b->refs.fetch_sub(1) == 1) {
