@@ -12,8 +12,9 @@ Prints ONE JSON line (rank 0).  ``value`` is nnz(L+U) per second over all
 ranks (each rank factors its own replica: the method needs no exchange);
 ``e2e`` is the same metric through ``gsofa_symbolic`` with host buffers
 (pinned input, host->device and device->host copies inside the timed region);
-``roofline`` relates the traversal kernel's algorithmic bytes to the measured
-HBM copy bandwidth; ``cpu_baseline`` times the CPU oracle on a row sample.
+``roofline`` relates the bytes that a call cannot do without (the pattern in, the result
+out) to the measured HBM copy bandwidth, or, where options select the traversal, its
+algorithmic bytes; ``cpu_baseline`` times the CPU oracle on a row sample.
 ``--impl reference`` times the CPU oracle itself as the reference arm.
 """
 from __future__ import annotations
@@ -132,6 +133,12 @@ def algorithmic_bytes(vscan, escan, nnz_rows, n):
     8 B per expanded vertex (two row pointers), 4 B column + 4 B maxId per scanned
     adjacency entry, 4 B per output column, plus 16 B of per-row metadata."""
     return float(8 * vscan.sum() + 8 * escan.sum() + 4 * nnz_rows.sum() + 16 * n)
+
+
+def call_bytes(n, nnz_a, nnz_lu, nsup):
+    """Bytes a whole call cannot do without: the CSR in, both CSRs, fill counts and
+    supernodes out."""
+    return float(4 * (n + 1) + 4 * nnz_a + 16 * (n + 1) + 4 * nnz_lu + 4 * n + 4 * (nsup + 1))
 
 
 class ClockSampler:
@@ -293,7 +300,7 @@ def main():
         sampler.start()
     ev0 = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps)]
     ev1 = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps)]
-    trav_ms, launches, nnz_step, stats0 = [], 0, 0, None
+    trav_ms, total_ms, launches, nnz_step, nsup_step, stats0 = [], [], 0, 0, 0, None
     barrier()
     w0 = time.perf_counter()
     for s in range(args.steps):
@@ -302,8 +309,9 @@ def main():
         r = gs.symbolic_device(rp, ci, opts=opts, stream=stream)
         ev1[s].record(stream)
         trav_ms.append(r.stats["ms_traverse_smem"] + r.stats["ms_traverse_global"])
+        total_ms.append(r.stats["ms_total"])
         launches += r.stats["kernel_launches"]
-        nnz_step = r.nnz_L + r.nnz_U
+        nnz_step, nsup_step = r.nnz_L + r.nnz_U, r.n_super
         stats0 = r.stats
         del r
     barrier()
@@ -358,21 +366,28 @@ def main():
         pass
     hbm_peak = float(peaks.get("hbm_gbs", 6800.0))
     peak_src = "measured" if "hbm_gbs" in peaks else "fallback"
-    # algorithmic bytes of the traversal launch from the oracle's per-row minimum work
     cores = len(os.sched_getaffinity(0)) if hasattr(os, "sched_getaffinity") else os.cpu_count()
     orc = oracle.symbolic(A, nthreads=cores)
-    nnz_rows = np.diff(orc["L_rowptr"]) + np.diff(orc["U_rowptr"])
-    alg = algorithmic_bytes(orc["vscan"], orc["escan"], nnz_rows, n)
-    t_trav = statistics.mean(trav_ms) / 1000.0
-    achieved = alg / t_trav / 1e9
-    # DRAM bytes per launch from an ncu capture of this kernel source (default options only)
-    traffic = stored_traffic(name) if not extra else None
-
-    # the dominant traversal tier of this matrix
-    if stats0["ms_traverse_global"] > stats0["ms_traverse_smem"]:  # the class-ordered kernel's time
-        kernel_name = "trav_class_kernel (class-ordered maxId traversal on a visited bitmap, one warp per source)"
+    if max(trav_ms) > 0.0:
+        # options selected the traversal: its algorithmic bytes, from the oracle's per-row
+        # minimum work, against its launch; DRAM bytes per launch from an ncu capture of this
+        # kernel source (default options only)
+        nnz_rows = np.diff(orc["L_rowptr"]) + np.diff(orc["U_rowptr"])
+        alg = algorithmic_bytes(orc["vscan"], orc["escan"], nnz_rows, n)
+        t_trav = statistics.mean(trav_ms) / 1000.0
+        traffic = stored_traffic(name) if not extra else None
+        if stats0["ms_traverse_global"] > stats0["ms_traverse_smem"]:  # the dominant tier of this matrix
+            kernel_name = "trav_class_kernel (class-ordered maxId traversal on a visited bitmap, one warp per source)"
+        else:
+            kernel_name = "trav_smem_kernel (maxId traversal, one CTA per source)"
     else:
-        kernel_name = "trav_smem_kernel (maxId traversal, one CTA per source)"
+        # elimination on chip is bound by the chain of its panels, not by memory: the whole call
+        alg = call_bytes(n, A.nnz, nnz_step, nsup_step)
+        t_trav = statistics.mean(total_ms) / 1000.0
+        traffic = None
+        kernel_name = "all kernels of the call (band_elim_kernel or front_elim_kernel: boolean elimination on chip)"
+    achieved = alg / t_trav / 1e9
+
     line = {
         "metric": "nnz(L+U)/s", "value": value, "unit": "nnz(L+U)/s", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": 1000.0 * t_dev / args.steps,
@@ -467,7 +482,7 @@ def run_batch_bench(args, rank, world, local):
         sampler.start()
     e0 = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps)]
     e1 = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps)]
-    nnz, trav, launches = 0, [], 0
+    nnz, nsup, trav, total, launches = 0, 0, [], [], 0
     if world > 1:
         torch.distributed.barrier()
     torch.cuda.synchronize(dev)
@@ -477,7 +492,10 @@ def run_batch_bench(args, rank, world, local):
         res = gs.batch_device(dmats, opts=opts)
         e1[s_].record(stream)
         nnz = sum(r.nnz_L + r.nnz_U for r in res)
-        trav.append(res[0].stats["ms_traverse"])
+        nsup = sum(r.n_super for r in res)
+        st = res[0].stats
+        trav.append(st["ms_traverse_smem"] + st["ms_traverse_global"])
+        total.append(st["ms_total"])
         launches += res[0].stats["kernel_launches"]
         del res
     torch.cuda.synchronize(dev)
@@ -511,10 +529,18 @@ def run_batch_bench(args, rank, world, local):
     if rank != 0:
         return 0
     cores = len(os.sched_getaffinity(0)) if hasattr(os, "sched_getaffinity") else os.cpu_count()
-    alg = _oracle_alg_bytes(mats, cores)
-    t_trav = statistics.mean(trav) / 1000.0
-    if t_trav <= 0:
-        t_trav = t / args.steps  # whole step as an upper bound when the launch was not timed
+    if max(trav) > 0.0:
+        alg = _oracle_alg_bytes(mats, cores)
+        t_trav = statistics.mean(trav) / 1000.0
+        kernel_name = ("trav_class_kernel (batched, class-ordered, one warp per source)"
+                       if tuned and tuned["kernel"] == "warp_per_source_class"
+                       else "trav_smem_kernel (batched, one CTA per source)")
+    else:
+        alg = call_bytes(rows, sum(A.nnz for A in mats), nnz, nsup)
+        t_trav = statistics.mean(total) / 1000.0
+        kernel_name = "all kernels of the call (band_elim_kernel: boolean elimination on chip)"
+        if t_trav <= 0:
+            t_trav = t / args.steps  # whole step as an upper bound when the call was not timed
     peak, src = _peak_hbm()
     # CPU baseline: the oracle on every 16th matrix (all rows)
     import oracle
@@ -534,9 +560,7 @@ def run_batch_bench(args, rank, world, local):
                    "l2": "flushed between steps (256 MB write)", "parallelism": f"replicas x{world}"},
         "rows_per_s": world * args.steps * rows / t, "matrices_per_s": world * args.steps * len(mats) / t,
         "e2e": e2e, "gpu_launches": launches,
-        "roofline": {"bound": "hbm", "kernel": ("trav_class_kernel (batched, class-ordered, one warp per source)"
-                                                if tuned and tuned["kernel"] == "warp_per_source_class"
-                                                else "trav_smem_kernel (batched, one CTA per source)"),
+        "roofline": {"bound": "hbm", "kernel": kernel_name,
                      "achieved": alg / t_trav / 1e9,
                      "peak": peak, "unit": "GB/s", "frac": alg / t_trav / 1e9 / peak, "traffic": None,
                      "peak_source": f"{src} (copy bandwidth, burst)", "algorithmic_bytes_per_launch": alg,

@@ -64,9 +64,11 @@ typedef struct gsofa_options {
     int32_t fill_first;          /* 1: skip lowering the maxId of a vertex already known to be a fill
                                     (the optional "line 9.5" of Section 4); same result */
     int32_t collect_stats;       /* 1: record per-phase CUDA-event times and work counters (expanded vertices,
-                                    scanned entries: extra loads in the traversal), 2: the times only */
-    int32_t validate;            /* 0 or 1: check the CSR on the device first (default 1); 2: skip */
-    int32_t autotune;            /* 1 = time candidates once and keep the fastest: gsofa_batch per batch shape
+                                    scanned entries: extra loads in the traversal, which then runs where
+                                    elimination would), 2: the times only */
+    int32_t validate;            /* 0 or 1: check the CSR on the device first (default 1); 2: skip (and
+                                    traverse: elimination measures the band in the same pass as the checks) */
+    int32_t autotune;            /* traversals: 1 = time candidates once and keep the fastest: gsofa_batch per batch shape
                                     (kernel, block size, CTAs or warps per SM, frontier list capacity,
                                     work items per fetch, the fill-first check); single matrices per
                                     (n, nnz) (frontier order, and the fill-first check for breadth-first).
@@ -78,11 +80,14 @@ typedef struct gsofa_options {
                                     level parity (default 512 with visited bitmaps in global memory,
                                     else 128; 32-1024) */
     int32_t max_ctas;            /* cap on traversal CTAs per launch, so concurrent launches share the GPU
-                                    (default 0: one full wave) */
-    int32_t frontier_order;      /* 0: automatic: class order for every source (sources below an explicit
-                                    smem_max_source stay breadth-first in shared memory); with
-                                    autotune = 1 both orders are timed once per (n, nnz) and the faster
-                                    kept.  1: breadth-first levels (shared-memory tier wherever the
+                                    (default 0: one full wave).  Elimination: CTAs of one banded matrix; a
+                                    batch and a dissection take one CTA or cluster per matrix or block */
+    int32_t frontier_order;      /* 0: automatic: elimination on chip where the pattern is banded or, from
+                                    order 16,384 on, a nested dissection, and every option that concerns
+                                    the traversal alone has its default; else class order for every
+                                    source (sources below an explicit smem_max_source stay breadth-first
+                                    in shared memory); with autotune = 1 both orders are timed once per
+                                    (n, nnz) and the faster kept.  1: breadth-first levels (shared-memory tier wherever the
                                     maxId array fits on chip, class order above).  2: by increasing
                                     maxId class for every source (visited bitmaps, one warp per
                                     source).  Same result */
@@ -125,13 +130,17 @@ typedef struct gsofa_options {
 typedef struct gsofa_stats {
     float ms_validate, ms_traverse, ms_emit, ms_supernode, ms_total;
     float ms_traverse_smem;      /* breadth-first shared-memory kernel (sources below smem_max_source) */
-    float ms_traverse_global;    /* class-ordered kernel (every other source; all of them by default) */
+    float ms_traverse_global;    /* class-ordered kernel (every other source).  Elimination: both are 0 and
+                                    ms_traverse is its time (a dissection: with all of its levels),
+                                    ms_supernode the counts and supernodes, ms_emit the columns (a
+                                    dissection: ms_supernode sizes and columns, ms_emit the supernodes) */
     int32_t traverse_launches;
     int32_t kernel_launches;     /* every kernel this call launched */
     int64_t vertices_expanded;   /* frontier expansions, revisits included */
     int64_t edges_scanned;       /* adjacency entries read by expansions */
     int64_t pool_retries;        /* times the row pool had to grow and the traversal rerun */
-    int64_t levels;              /* frontier levels summed over sources (both kernels) */
+    int64_t levels;              /* frontier levels summed over sources (both kernels); elimination: panels
+                                    of 32 rows, or blocks of a dissection */
     int64_t cycles_traverse;     /* shared-memory tier: SM cycles in frontier levels, summed over sources */
     int64_t cycles_emit;         /* shared-memory tier: SM cycles emitting rows, summed over sources */
 } gsofa_stats;

@@ -584,6 +584,7 @@ struct BandRun {
   cudaStream_t st = nullptr;
   BandArgs a;
   std::vector<BandMat> mats;
+  int max_ctas = 0;  // of a single matrix's elimination, 0: the whole GPU
   unsigned char* ctr = nullptr;   // BandCounters | band | mat_tot | nsuper | cross: zeroed together
   unsigned char* hctr = nullptr;  // pinned copy (all but cross)
   size_t ctr_bytes = 0, host_bytes = 0;
@@ -702,7 +703,8 @@ int band_run(BandRun& b, int64_t words, Events& ev) {
   if (B == 1) {
     const BandShape s = band_shape(a.one.LB, a.one.UB, true);
     const int panels = (a.one.n + 31) / 32;
-    const int parts = std::max(1, std::min(panels, c->sms / s.C));
+    const int ctas = b.max_ctas > 0 ? std::min(b.max_ctas, c->sms) : c->sms;
+    const int parts = std::max(1, std::min(panels, ctas / s.C));
     if (e == cudaSuccess) e = launch_band_elim(a, parts, s.C, s.threads, s.smem, st);
     b.launches++;
   } else {
@@ -751,7 +753,7 @@ int band_run(BandRun& b, int64_t words, Events& ev) {
 
 void band_times(Events& ev, gsofa_stats* s) {
   s->ms_validate = ev.ms(0, 1);
-  s->ms_traverse = s->ms_traverse_global = ev.ms(2, 3);
+  s->ms_traverse = ev.ms(2, 3);
   s->ms_supernode = ev.ms(3, 4);
   s->ms_emit = ev.ms(4, 5);
   s->ms_total = ev.ms(0, 5);
@@ -1157,6 +1159,7 @@ int run_band_single(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, con
   m.colidx = ci;
   m.n = n;
   b.mats.push_back(m);
+  b.max_ctas = o.max_ctas;
   int rc = band_measure(b, o);
   ev.rec(1, st);
   int64_t words = -1;
@@ -1197,6 +1200,7 @@ int run_band_single(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, con
     if (rc == GSOFA_E_TIMEOUT || rc == GSOFA_E_CUDA) wait_stream(st);
     cudaGetLastError();
     b.free_results();
+    if (rc == GSOFA_E_NOMEM) rc = GSOFA_OK;  // no room for the bitmaps: the traversal needs less
     *taken = rc != GSOFA_OK;
     return rc;
   }
@@ -1289,6 +1293,10 @@ int run_band_batch(Ctx* c, const std::vector<int32_t>& idx, const int32_t* n, co
       if (rc != GSOFA_E_INVAL) wait_stream(st);
       cudaGetLastError();
       b.free_results();
+      if (rc == GSOFA_E_NOMEM) {  // no room for the bitmaps: the traversal needs less
+        rest->insert(rest->end(), order.begin(), order.end());
+        return GSOFA_OK;
+      }
       return rc;
     }
     SharedBlock* blk = new SharedBlock();

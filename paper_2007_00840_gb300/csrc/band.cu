@@ -79,71 +79,129 @@ __device__ __forceinline__ int mat_at(const BandArgs& a, long long x, bool group
 }  // namespace
 
 // ------------------------------------------------------------ check and measure
-// Eight lanes per row: the checks of validate_kernel, the row's distance from the
-// diagonal on both sides (largest over each matrix in band[2m], band[2m+1]), and the
-// row's entries of A with the diagonal counted as present.  One matrix: also the panel
-// boundaries that an entry below the diagonal crosses; where none does, the rows after
-// the boundary take nothing from the rows before it.
-__global__ void band_scan_kernel(BandArgs a) {
-  const int sub = threadIdx.x & 7;
-  const long long step = ((long long)gridDim.x * blockDim.x) >> 3;
-  const long long first = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
-  // every lane of a warp runs the same rounds
-  for (long long base = first - ((threadIdx.x & 31) >> 3); base < a.rows; base += step) {
-    const long long r = base + ((threadIdx.x & 31) >> 3);
-    int bl = 0, bu = 0, m = 0, i = 0;
-    bool diag = false;
-    int rb = 0, re = 0, bad = 0;
+// The checks of validate_kernel, the rows' distance from the diagonal on both sides
+// (largest over each matrix in band[2m], band[2m+1]), and every row's entries of A with the
+// diagonal counted as present.  One matrix: also the panel boundaries that an entry below
+// the diagonal crosses; where none does, the rows after the boundary take nothing from the
+// rows before it.  A warp takes 32 rows and reports once (per CTA for one matrix): a look
+// at the two maxima per row, all at one address, took 198 us on 1M rows, this 42.
+__global__ void __launch_bounds__(256) band_scan_kernel(BandArgs a) {
+  __shared__ int s_l[8], s_u[8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane & 7;
+  const long long chunks = (a.rows + 31) >> 5, step = (long long)gridDim.x * 8;
+  int max_l = 0, max_u = 0;
+  // (indices are unsigned: a row that starts at the largest index wraps out of its range)
+  for (long long q = (long long)blockIdx.x * 8 + warp; q < chunks; q += step) {
+    // a row per lane
+    const long long r = 32 * q + lane;
+    int m = 0, i = 0, n = 0, rb = 0, re = 0, bad = 0;
+    const int32_t* col = nullptr;
     if (r < a.rows) {
       m = a.mats ? mat_at(a, r, false) : 0;
       const BandMat d = a.mats ? a.mats[m] : a.one;
       i = (int)(r - d.row_base);
+      n = d.n;
+      col = d.colidx;
       rb = d.rowptr[i];
       re = d.rowptr[i + 1];
-      if (re < rb || rb < 0 || (i == 0 && rb != 0)) {
-        bad = ERR_ROWPTR;
-      } else {
-        for (int e = rb + sub; e < re; e += 8) {
-          const int c = d.colidx[e];
-          if ((unsigned)c >= (unsigned)d.n) {
-            bad |= ERR_COL_RANGE;
-            continue;
-          }
-          if (e > rb && d.colidx[e - 1] >= c) bad |= ERR_UNSORTED;
-          bl = max(bl, i - c);
-          bu = max(bu, c - i);
-          diag |= c == i;
+      if (re < rb || rb < 0 || (i == 0 && rb != 0)) bad = ERR_ROWPTR;
+    }
+    const int stop = bad ? rb : re;
+    const int m0 = __shfl_sync(FULL, m, 0);
+    const bool one = __all_sync(FULL, m == m0 || r >= a.rows);
+    // then eight lanes per row, four rows at a time; the first eight columns of all rows in flight
+    int c8[8];
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+      const int row = 4 * k + (lane >> 3);
+      const unsigned e = (unsigned)(__shfl_sync(FULL, rb, row) + sub);
+      const int32_t* x = (const int32_t*)__shfl_sync(FULL, (unsigned long long)col, row);
+      c8[k] = e < (unsigned)__shfl_sync(FULL, stop, row) ? x[e] : 0;
+    }
+    int bl = 0, bu = 0, low = INT_MAX;
+    unsigned has = 0u;  // bit x: row x has its diagonal
+#pragma unroll
+    for (int k = 0; k < 8; k++) {
+      const int row = 4 * k + (lane >> 3);
+      const unsigned b = (unsigned)__shfl_sync(FULL, rb, row), e1 = (unsigned)__shfl_sync(FULL, stop, row);
+      const int at = __shfl_sync(FULL, i, row), nr = __shfl_sync(FULL, n, row);
+      const int32_t* x = (const int32_t*)__shfl_sync(FULL, (unsigned long long)col, row);
+      int wrong = 0, dg = 0, l = 0, u = 0;
+      for (unsigned e = b + sub; e < e1; e += 8) {
+        const int c = e == b + sub ? c8[k] : x[e];
+        if ((unsigned)c >= (unsigned)nr) {
+          wrong |= ERR_COL_RANGE;
+          continue;
         }
+        if (e > b && x[e - 1] >= c) wrong |= ERR_UNSORTED;
+        l = max(l, at - c);
+        u = max(u, c - at);
+        dg |= c == at;
+        if (at - c < BAND_REACH_MAX) low = min(low, c);
+      }
+      const unsigned d = __ballot_sync(FULL, dg);
+#pragma unroll
+      for (int g = 0; g < 4; g++)
+        if ((d >> (8 * g)) & 0xFFu) has |= 1u << (4 * k + g);
+      if (__any_sync(FULL, wrong != 0)) {
+        for (int o = 4; o >= 1; o >>= 1) wrong |= __shfl_xor_sync(FULL, wrong, o);
+        const int mine = __shfl_sync(FULL, wrong, 8 * (lane & 3));
+        if (lane >> 2 == k) bad |= mine;
+      }
+      bl = max(bl, l);
+      bu = max(bu, u);
+      if (!one) {  // rows of several matrices: each row its own
+        int32_t* band = a.band + 2 * (size_t)__shfl_sync(FULL, m, row);
+        if (l > *(volatile int32_t*)band) atomicMax(band, l);
+        if (u > *(volatile int32_t*)(band + 1)) atomicMax(band + 1, u);
       }
     }
-    // the row's eight lanes together
-    int dg = diag;
-#pragma unroll
-    for (int o = 4; o >= 1; o >>= 1) {
-      bl = max(bl, __shfl_xor_sync(FULL, bl, o));
-      bu = max(bu, __shfl_xor_sync(FULL, bu, o));
-      dg |= __shfl_xor_sync(FULL, dg, o);
-      bad |= __shfl_xor_sync(FULL, bad, o);
-    }
-    if (r < a.rows && sub == 0) {
-      a.fill[r] = (re - rb) + (dg ? 0 : 1);
+    if (r < a.rows) {
+      a.fill[r] = (re - rb) + ((has >> lane) & 1u ? 0 : 1);
       if (bad) {
         atomicOr(&a.ctr->err, bad);
         atomicMax(&a.ctr->bad_row, INT_MAX - (int)r);
       }
-      int32_t* b = a.band + 2 * (size_t)m;
-      if (bl > *(volatile int32_t*)b) atomicMax(b, bl);
-      if (bu > *(volatile int32_t*)(b + 1)) atomicMax(b + 1, bu);
-      // panel boundaries between the row and its leftmost entry (no wider band fits on chip)
-      if (a.cross && !bad && bl < BAND_REACH_MAX) {
-        const int q0 = ((i - bl) >> 5) + 1, q1 = i >> 5;
-        for (int w = q0 >> 5; w <= q1 >> 5 && q0 <= q1; w++) {
+    }
+    if (!one) continue;
+    bl = __reduce_max_sync(FULL, bl);
+    bu = __reduce_max_sync(FULL, bu);
+    if (a.mats) {
+      if (lane == 0) {
+        int32_t* band = a.band + 2 * (size_t)m0;
+        if (bl > *(volatile int32_t*)band) atomicMax(band, bl);
+        if (bu > *(volatile int32_t*)(band + 1)) atomicMax(band + 1, bu);
+      }
+      continue;
+    }
+    max_l = max(max_l, bl);
+    max_u = max(max_u, bu);
+    if (a.cross) {
+      // panel boundaries between these rows, one panel, and their leftmost entry (no wider
+      // band fits on chip, and more marks than needed only keep stretches together)
+      low = __reduce_min_sync(FULL, low);
+      const int q1 = (int)q, q0 = low == INT_MAX ? q1 + 1 : (low >> 5) + 1;
+      if (q0 <= q1)
+        for (int w = (q0 >> 5) + lane; w <= q1 >> 5; w += 32) {
           const int lo = max(q0 - 32 * w, 0), hi = min(q1 - 32 * w, 31);
           const uint32_t bits = (0xFFFFFFFFu << lo) & (0xFFFFFFFFu >> (31 - hi));
           if ((*(volatile uint32_t*)(a.cross + w) & bits) != bits) atomicOr(a.cross + w, bits);
         }
-      }
     }
+  }
+  if (a.mats) return;
+  if (lane == 0) {
+    s_l[warp] = max_l;
+    s_u[warp] = max_u;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; w++) {
+      max_l = max(max_l, s_l[w]);
+      max_u = max(max_u, s_u[w]);
+    }
+    if (max_l > *(volatile int32_t*)a.band) atomicMax(a.band, max_l);
+    if (max_u > *(volatile int32_t*)(a.band + 1)) atomicMax(a.band + 1, max_u);
   }
 }
 
@@ -521,6 +579,11 @@ __device__ __forceinline__ void step_below(const Band& B, const PanelBufs& S, in
 
 }  // namespace
 
+// Bound by the latency of the chain, one panel after the other (shared-memory loads, 31
+// dependent shuffles to close the block, two barriers, cluster-wide with more than one CTA):
+// per panel of 32 rows 1.5 us on a 64 x 64 grid, 2.2 at band 211, 2.4 at 317 (cluster of
+// 4), 4.2 at 1,024 (of 8).  Elimination against the traversal: 32^3 grid 8.7 -> 4.3 ms,
+// 317 x 293 63 -> 7.0, band 211 of order 15,013 4.9 -> 1.05.
 // Warps of a CTA: 0 the chain, the last the loader (rows into the window), the others
 // workers (B, C and finished rows out).
 template <int C>
@@ -1094,7 +1157,7 @@ BandShape band_shape(int LB, int UB, bool alone) {
 }
 
 cudaError_t launch_band_scan(const BandArgs& a, cudaStream_t st) {
-  long long grid = (a.rows * 8 + 255) / 256;
+  long long grid = (a.rows + 255) / 256;
   if (grid > 4096) grid = 4096;
   band_scan_kernel<<<(int)grid, 256, 0, st>>>(a);
   return cudaGetLastError();
