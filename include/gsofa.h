@@ -82,9 +82,9 @@ typedef struct gsofa_options {
     int32_t max_ctas;            /* cap on traversal CTAs per launch, so concurrent launches share the GPU
                                     (default 0: one full wave).  Elimination: CTAs of one banded matrix; a
                                     batch and a dissection take one CTA or cluster per matrix or block */
-    int32_t frontier_order;      /* 0: automatic: elimination on chip where the pattern is banded or, from
-                                    order 16,384 on, a nested dissection, and every option that concerns
-                                    the traversal alone has its default; else class order for every
+    int32_t frontier_order;      /* 0: automatic: elimination on chip where the pattern is banded or a
+                                    nested dissection (of order 2,600 or more) and every option that
+                                    concerns the traversal alone has its default; else class order for every
                                     source (sources below an explicit smem_max_source stay breadth-first
                                     in shared memory); with autotune = 1 both orders are timed once per
                                     (n, nnz) and the faster kept.  1: breadth-first levels (shared-memory tier wherever the

@@ -760,9 +760,23 @@ void band_times(Events& ev, gsofa_stats* s) {
 }
 
 // ---------------------------------------------------------------- nested dissection
-// Orders from which the blocks of a dissection are looked for (below, the traversal takes
-// about as long as the search), and up to which what remains is one front.
+// Orders from which the blocks of a dissection are looked for: any pattern whose band does
+// not fit, and one that looks like a dissection (entries near the diagonal, few far out).
+// Dissections of square grids, traversal / blocks: order 2,025 414 / 455 us, 2,809 468 /
+// 452, 4,900 628 / 469, 10,000 993 / 561, 16,256 1,351 / 631.
 constexpr int32_t FRONT_MIN_ORDER = 16384;
+constexpr int32_t FRONT_NEAR_ORDER = 2600;
+// Up to this order a dissection is one wide band (order 900: 283 us by traversal, 219 as a
+// band; 1,600: 370 / 357; 2,025: 414 / 483); between the two lines it is traversed.
+constexpr int32_t NEAR_BAND_ORDER = 1600;
+// A band of more words than this needs a cluster of eight, 4 us per panel whatever is in it;
+// with fewer entries than this in all the traversal is as fast or faster (3D grids: 27 x 27
+// x 9, 37k entries, 942 us by traversal, 1,177 as a band; 33 x 33 x 9, 52k: 1,688 / 1,834;
+// 27 x 27 x 20, 82k: 2,408 / 2,212; 33 x 33 x 20, 119k: 4,702 / 3,788), except for small
+// orders (band 1,000 of order 3,000: 1,025 / 651).
+constexpr int32_t WIDE_BAND = 16;
+constexpr unsigned long long WIDE_NNZ = 56000;
+constexpr int32_t WIDE_MIN_ORDER = 4096;
 constexpr int32_t FRONT_LAST_ORDER = 2900;
 constexpr int32_t FRONT_FIRST_BLOCK = 512;
 // threads of a front where there are more fronts than SMs: two CTAs fit an SM (1024 x 1024
@@ -836,7 +850,7 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
   ev.rec(2, st);
   for (int level = 0; level < 16; level++) {
     std::vector<FrontMat> fronts;
-    const bool whole = l.n <= FRONT_LAST_ORDER;
+    const bool whole = level > 0 && l.n <= FRONT_LAST_ORDER;
     int32_t n1 = 0, br_total = 0;
     int64_t room = 0;
     int32_t* bcg = nullptr;
@@ -1163,16 +1177,26 @@ int run_band_single(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, con
   int rc = band_measure(b, o);
   ev.rec(1, st);
   int64_t words = -1;
+  bool near = false;
   if (rc == GSOFA_OK) {
     if (b.counters()->err) {
       rc = GSOFA_E_INVAL;
       out->err_detail = b.counters()->bad_row ? INT_MAX - b.counters()->bad_row : -1;
     } else {
+      // near: most entries lie close to the diagonal and few far out, as in a dissection (mean
+      // distance 0.04 of the band or less; bands and natural grids have 0.2 or more, with one
+      // far entry per row 0.09)
+      const BandCounters& h = *b.counters();
+      const int32_t width = std::max(b.h_band()[0], b.h_band()[1]);
+      near = h.spread < h.nnz * (unsigned long long)width / 16;
       words = band_layout(b);
+      const bool wide = b.mats[0].LB > WIDE_BAND;
+      if (words >= 0 && wide && (near ? n > NEAR_BAND_ORDER : n >= WIDE_MIN_ORDER && h.nnz < WIDE_NNZ))
+        words = -1;
       if (words >= 0) rc = band_run(b, words, ev);
     }
   }
-  if (rc == GSOFA_OK && words < 0 && n >= FRONT_MIN_ORDER) {
+  if (rc == GSOFA_OK && words < 0 && n >= (near ? FRONT_NEAR_ORDER : FRONT_MIN_ORDER)) {
     bool fronts = false;
     int launches = b.launches;
     rc = run_fronts(c, n, rp, ci, o, st, b.fill, out, ev, &launches, &fronts);

@@ -87,9 +87,11 @@ __device__ __forceinline__ int mat_at(const BandArgs& a, long long x, bool group
 // at the two maxima per row, all at one address, took 198 us on 1M rows, this 42.
 __global__ void __launch_bounds__(256) band_scan_kernel(BandArgs a) {
   __shared__ int s_l[8], s_u[8];
+  __shared__ unsigned long long s_nnz[8], s_spread[8];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane & 7;
   const long long chunks = (a.rows + 31) >> 5, step = (long long)gridDim.x * 8;
   int max_l = 0, max_u = 0;
+  unsigned long long nnz = 0, spread = 0;
   // (indices are unsigned: a row that starts at the largest index wraps out of its range)
   for (long long q = (long long)blockIdx.x * 8 + warp; q < chunks; q += step) {
     // a row per lane
@@ -136,6 +138,7 @@ __global__ void __launch_bounds__(256) band_scan_kernel(BandArgs a) {
         if (e > b && x[e - 1] >= c) wrong |= ERR_UNSORTED;
         l = max(l, at - c);
         u = max(u, c - at);
+        spread += (unsigned)abs(at - c);
         dg |= c == at;
         if (at - c < BAND_REACH_MAX) low = min(low, c);
       }
@@ -158,6 +161,7 @@ __global__ void __launch_bounds__(256) band_scan_kernel(BandArgs a) {
     }
     if (r < a.rows) {
       a.fill[r] = (re - rb) + ((has >> lane) & 1u ? 0 : 1);
+      nnz += (unsigned)(stop - rb);
       if (bad) {
         atomicOr(&a.ctr->err, bad);
         atomicMax(&a.ctr->bad_row, INT_MAX - (int)r);
@@ -190,16 +194,26 @@ __global__ void __launch_bounds__(256) band_scan_kernel(BandArgs a) {
     }
   }
   if (a.mats) return;
+  for (int o = 16; o >= 1; o >>= 1) {
+    nnz += __shfl_xor_sync(FULL, nnz, o);
+    spread += __shfl_xor_sync(FULL, spread, o);
+  }
   if (lane == 0) {
     s_l[warp] = max_l;
     s_u[warp] = max_u;
+    s_nnz[warp] = nnz;
+    s_spread[warp] = spread;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < 8; w++) {
       max_l = max(max_l, s_l[w]);
       max_u = max(max_u, s_u[w]);
+      nnz += s_nnz[w];
+      spread += s_spread[w];
     }
+    atomicAdd(&a.ctr->nnz, nnz);
+    atomicAdd(&a.ctr->spread, spread);
     if (max_l > *(volatile int32_t*)a.band) atomicMax(a.band, max_l);
     if (max_u > *(volatile int32_t*)(a.band + 1)) atomicMax(a.band + 1, max_u);
   }

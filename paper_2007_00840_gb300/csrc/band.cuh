@@ -11,6 +11,7 @@ constexpr int BAND_REACH_MAX = 8192;  // above the widest band that eight CTAs h
 // Counters of one call.
 struct BandCounters {
   unsigned long long total_L, total_U;
+  unsigned long long nnz, spread;  // one matrix: entries of A, and the sum of their distances from the diagonal
   int32_t err;          // ERR_* bits
   int32_t bad_row;      // INT_MAX - first offending row (0: none)
   int32_t n_super;
