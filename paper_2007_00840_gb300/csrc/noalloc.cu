@@ -102,7 +102,14 @@ extern "C" int gsofa_row_counts_noalloc(int32_t n, const int32_t* d_rowptr, cons
     b.one.LB = (m.band[0] + 31) / 32;
     b.one.UB = (m.band[1] + 31) / 32;
     const BandShape s = band_shape(b.one.LB, b.one.UB, true);
-    if (s.C) {
+    // a wide band, which takes a cluster, pays from order 4,096 on (18 x 18 x 18 grid 845 us by
+    // traversal, 726 as a band; 12 x 12 x 12 with far entries 220 / 292; 18 x 18 x 9 322 / 352),
+    // and where most entries lie close to the diagonal, as in a dissection, up to 1,600 (40 x
+    // 40 348 / 290, 47 x 47 435 / 465)
+    const unsigned long long width = (unsigned long long)(m.band[0] > m.band[1] ? m.band[0] : m.band[1]);
+    const bool near = m.c.spread < m.c.nnz * width / 16;
+    const bool traverse = s.C == 0 || (b.one.LB > 8 && (near ? n > 1600 : n < 4096));
+    if (!traverse) {
       const int panels = (n + 31) / 32, most = sms / s.C;
       if (launch_band_elim(b, panels < most ? panels : most, s.C, s.threads, s.smem, st) != cudaSuccess)
         return GSOFA_E_CUDA;
@@ -129,7 +136,8 @@ extern "C" int gsofa_row_counts_noalloc(int32_t n, const int32_t* d_rowptr, cons
 
   // the counters must start at zero on every call; the overflow lists need no reset
   if (launch_init_counters(ctr, st) != cudaSuccess) return GSOFA_E_CUDA;
-  if (launch_validate(n, d_rowptr, d_colidx, ctr, st) != cudaSuccess) return GSOFA_E_CUDA;
+  // (the scan above has checked the rows)
+  if (n == 0 && launch_validate(n, d_rowptr, d_colidx, ctr, st) != cudaSuccess) return GSOFA_E_CUDA;
   if (n > 0) {
     TravArgs a;
     memset(&a, 0, sizeof(a));
