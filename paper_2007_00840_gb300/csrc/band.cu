@@ -39,8 +39,6 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-constexpr int BAND_STAGE = 512;  // column indices of one panel staged ahead (more: read in place)
-
 __device__ __forceinline__ uint32_t gt_mask(int k) { return k >= 31 ? 0u : 0xFFFFFFFEu << k; }  // bits above k
 __device__ __forceinline__ uint32_t lt_mask(int k) { return (1u << k) - 1u; }                   // bits below k
 // all ones where bit k of x is set (two shifts: shorter than a predicate's way to the OR)
@@ -1143,33 +1141,6 @@ __global__ void band_expand_kernel(BandArgs a) {
 }
 
 // ------------------------------------------------------------ launchers
-size_t band_smem_bytes(int LB, int UB, int C) {
-  const int wx = LB + UB + 1;
-  const size_t slots = (size_t)(LB + 2 + C - 1) / C;
-  return 4 * (128 + 64 + 68 + 192 * (size_t)(UB | 1) + 4 * BAND_STAGE + slots * 32 * (size_t)((wx | 1) + 1));
-}
-
-// Launch shape for a band of LB words left and UB words right of a row's own.  One matrix
-// (alone) is spread over a cluster once its window is wide enough for the split to pay for
-// the cluster's barriers (us per 32 rows with 1 / 4 / 8 CTAs: LB 3: 1.6 / 2.3 / 2.4, LB 7:
-// 2.3 / 2.2 / 2.4, LB 10: 3.1 / 2.5 / 2.7, LB 33: - / 5.0 / 4.4).  Batches have other
-// matrices to fill the chip with and take the smallest cluster that holds the window.
-BandShape band_shape(int LB, int UB, bool alone) {
-  BandShape s;
-  for (int C = !alone || LB <= 8 ? 1 : (LB <= 16 ? 4 : 8); C <= 8; C *= 2) {
-    const size_t b = band_smem_bytes(LB, UB, C);
-    if (b > BAND_SMEM_MAX - 1024) continue;
-    s.C = C;
-    s.smem = b;
-    break;
-  }
-  if (!s.C) return s;
-  // 14 worker warps: a batch's longest matrix sets its time (512 matrices: 1.28 ms; with 256
-  // threads 1.90, with 128 3.99)
-  s.threads = 512;
-  return s;
-}
-
 cudaError_t launch_band_scan(const BandArgs& a, cudaStream_t st) {
   long long grid = (a.rows + 255) / 256;
   if (grid > 4096) grid = 4096;
@@ -1207,13 +1178,6 @@ cudaError_t launch_band_elim(const BandArgs& a, int count, int C, int threads, s
     case 4: return launch_elim<4>(a, count, threads, smem, st);
     default: return launch_elim<8>(a, count, threads, smem, st);
   }
-}
-
-// Clusters of C CTAs for fronts [a.first, a.first + count).
-size_t front_smem_bytes(int sz, int nr, int nb, int C) {
-  const int pivots = (sz + 31) / 32, panels = pivots + (nr + 31) / 32, W = pivots + (nb + 31) / 32;
-  const size_t slots = (size_t)(panels + C - 1) / C;
-  return 4 * (128 + 64 + 68 + 192 * (size_t)((W - 1) | 1) + slots * 32 * (size_t)((W | 1) + 1));
 }
 
 namespace {

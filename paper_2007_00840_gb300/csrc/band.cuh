@@ -6,6 +6,7 @@
 namespace gsofa {
 
 constexpr int BAND_SMEM_MAX = 227 * 1024;
+constexpr int BAND_STAGE = 512;       // column indices of one panel staged ahead (more: read in place)
 constexpr int BAND_REACH_MAX = 8192;  // above the widest band that eight CTAs hold
 
 // Counters of one call.
@@ -72,18 +73,47 @@ struct FrontArgs {
   int32_t* piece_nL;               // per row above a block: its entries in the block
 };
 
-size_t front_smem_bytes(int sz, int nr, int nb, int C);
+inline size_t front_smem_bytes(int sz, int nr, int nb, int C) {
+  const int pivots = (sz + 31) / 32, panels = pivots + (nr + 31) / 32, W = pivots + (nb + 31) / 32;
+  const size_t slots = (size_t)(panels + C - 1) / C;
+  return 4 * (128 + 64 + 68 + 192 * (size_t)((W - 1) | 1) + slots * 32 * (size_t)((W | 1) + 1));
+}
+// Clusters of C CTAs for fronts [a.first, a.first + count).
 cudaError_t launch_front_elim(const FrontArgs& a, int count, int C, int threads, size_t smem, cudaStream_t st);
 
-size_t band_smem_bytes(int LB, int UB, int C);
+inline size_t band_smem_bytes(int LB, int UB, int C) {
+  const int wx = LB + UB + 1;
+  const size_t slots = (size_t)(LB + 2 + C - 1) / C;
+  return 4 * (128 + 64 + 68 + 192 * (size_t)(UB | 1) + 4 * BAND_STAGE + slots * 32 * (size_t)((wx | 1) + 1));
+}
+
 struct BandShape {
   int C = 0;  // CTAs per matrix (0: the band does not fit on chip)
   int threads = 0;
   size_t smem = 0;
 };
-// Launch shape for a band of LB words left and UB words right of a row's own; alone: one
-// matrix has the device.
-BandShape band_shape(int LB, int UB, bool alone);
+
+// Launch shape for a band of LB words left and UB words right of a row's own.  One matrix
+// (alone) is spread over a cluster once its window is wide enough for the split to pay for
+// the cluster's barriers (us per 32 rows with 1 / 4 / 8 CTAs: LB 3: 1.6 / 2.3 / 2.4, LB 7:
+// 2.3 / 2.2 / 2.4, LB 10: 3.1 / 2.5 / 2.7, LB 33: - / 5.0 / 4.4).  Batches have other
+// matrices to fill the chip with and take the smallest cluster that holds the window.
+inline BandShape band_shape(int LB, int UB, bool alone) {
+  BandShape s;
+  for (int C = !alone || LB <= 8 ? 1 : (LB <= 16 ? 4 : 8); C <= 8; C *= 2) {
+    const size_t b = band_smem_bytes(LB, UB, C);
+    if (b > BAND_SMEM_MAX - 1024) continue;
+    s.C = C;
+    s.smem = b;
+    break;
+  }
+  if (!s.C) return s;
+  // 14 worker warps: a batch's longest matrix sets its time (512 matrices: 1.28 ms; with 256
+  // threads 1.90, with 128 3.99)
+  s.threads = 512;
+  return s;
+}
+
 cudaError_t launch_band_scan(const BandArgs& a, cudaStream_t st);
 // `count` matrices from a.first on, or the parts one matrix's panels are dealt to: C CTAs (a cluster) each.
 cudaError_t launch_band_elim(const BandArgs& a, int count, int C, int threads, size_t smem, cudaStream_t st);
