@@ -666,8 +666,8 @@ int64_t band_layout(BandRun& b) {
   int64_t words = 0;
   for (size_t m = 0; m < b.mats.size(); m++) {
     BandMat& d = b.mats[m];
-    d.LB = (b.h_band()[2 * m] + 31) / 32;
-    d.UB = (b.h_band()[2 * m + 1] + 31) / 32;
+    d.LB = band_words_left(b.h_band()[2 * m]);
+    d.UB = band_words_right(b.h_band()[2 * m + 1]);
     if (!band_shape(d.LB, d.UB, false).C) return -1;
     d.bits_base = words;
     words += (int64_t)d.n * (d.LB + d.UB + 1);
@@ -1294,7 +1294,7 @@ int run_band_batch(Ctx* c, const std::vector<int32_t>& idx, const int32_t* n, co
       std::vector<int> size(order.size());
       bool sorted = true;
       for (size_t m = 0; m < order.size(); m++) {
-        size[m] = band_shape((b.h_band()[2 * m] + 31) / 32, (b.h_band()[2 * m + 1] + 31) / 32, false).C;
+        size[m] = band_shape(band_words_left(b.h_band()[2 * m]), band_words_right(b.h_band()[2 * m + 1]), false).C;
         if (size[m] == 0) rest->push_back(order[m]);
         if (size[m] == 0 || (m && size[m] < size[m - 1])) sorted = false;
       }

@@ -406,7 +406,7 @@ template <int C, bool FRONT>
 __device__ __forceinline__ void step_chain(const Band& B, const PanelBufs& S, int P, int sync_threads) {
   const int lane = threadIdx.x & 31, at = 32 * (P & 1) + lane;
   const uint32_t* x1 = panel_rows<C>(B, P + 1) + lane * B.xs + word0<FRONT>(B, P + 1) + P;
-  uint32_t m = FRONT || B.LB > 0 ? x1[0] : 0u, y = x1[1];
+  uint32_t m = x1[0], y = x1[1];
   uint32_t first = 0u;
   const bool right = words_right<FRONT>(B, P) > 0;
   if constexpr (C == 1) {

@@ -19,7 +19,14 @@ struct BandCounters {
   int32_t groups_done;
 };
 
-// One matrix.  LB, UB: words of columns left and right of a row's own word that the band reaches.
+// Words of columns that a band of `reach` columns takes left and right of a row's own word.
+// Left at least one: the window is the panels P .. P + LB, and while step P reads panel P + 1
+// the loader writes panel P + LB + 1.  With none a batch's chain read panel P + 1 before it
+// was there (a single matrix without entries below the diagonal is one stretch per panel).
+inline int band_words_left(int32_t reach) { return reach > 32 ? (reach + 31) / 32 : 1; }
+inline int band_words_right(int32_t reach) { return (reach + 31) / 32; }
+
+// One matrix.  LB, UB: band_words_left and band_words_right of its band.
 struct BandMat {
   const int32_t* rowptr;
   const int32_t* colidx;

@@ -99,8 +99,8 @@ extern "C" int gsofa_row_counts_noalloc(int32_t n, const int32_t* d_rowptr, cons
     rc = wait_stream(st);
     if (rc) return rc;
     if (m.c.err) return GSOFA_E_INVAL;
-    b.one.LB = (m.band[0] + 31) / 32;
-    b.one.UB = (m.band[1] + 31) / 32;
+    b.one.LB = band_words_left(m.band[0]);
+    b.one.UB = band_words_right(m.band[1]);
     const BandShape s = band_shape(b.one.LB, b.one.UB, true);
     // a wide band, which takes a cluster, pays from order 4,096 on (18 x 18 x 18 grid 845 us by
     // traversal, 726 as a band; 12 x 12 x 12 with far entries 220 / 292; 18 x 18 x 9 322 / 352),

@@ -1,0 +1,33 @@
+"""Bands in one batch call and through the server: the edges of words, panels and windows,
+with members that have nothing below (or above) the diagonal beside others.  Several
+matrices of one call have no stretch cuts, unlike a matrix alone."""
+import pytest
+
+from tests.gpu_util import assert_same, oracle_full, to_device
+from tests.test_gpu_band import _edge
+
+pytestmark = pytest.mark.gpu
+
+BANDS = [(0, 0), (0, 40), (40, 0), (1, 1), (0, 31), (0, 33), (33, 64), (0, 700), (0, 1500), (1300, 0), (600, 590), (1400, 1450)]
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 64, 65, 129, 517, 1700])
+def test_batch_edges(n):
+    import paper_2007_00840_gb300 as gs
+    mats = [_edge(n, min(bl, n - 1), min(bu, n - 1), seed=n + 10 * k) for k, (bl, bu) in enumerate(BANDS)]
+    dev = [to_device(A) for A in mats]
+    want = [oracle_full(A) for A in mats]
+    for r, o in zip(gs.batch_device(dev), want):
+        assert_same(r.to_host(), o)
+
+
+def test_served_upper_triangles():
+    """A burst of patterns without entries below the diagonal, some with them between."""
+    import paper_2007_00840_gb300 as gs
+    mats = [_edge(200 + 37 * k, 0 if k % 3 else 30, 20 + 11 * k, seed=k) for k in range(24)]
+    dev = [to_device(A) for A in mats]
+    srv = gs.Server()
+    tickets = [srv.submit(*d) for d in dev]
+    for t, A in zip(tickets, mats):
+        assert_same(srv.wait(t)[0].to_host(), oracle_full(A))
+    srv.close()

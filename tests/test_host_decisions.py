@@ -1,0 +1,48 @@
+"""What the host side decides, without a GPU: api.cu and noalloc.cu compiled as plain C++
+over a runtime and launchers that only keep books (host_fake.cpp)."""
+import functools
+import os
+import subprocess
+
+import pytest
+
+from paper_2007_00840_gb300 import build
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@functools.lru_cache(None)
+def _program(tmp):
+    inc = ["-I", build.INCLUDE, "-I", build.CSRC,
+           "-I", os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build._nvcc()))), "include")]
+    src = [os.path.join(build.CSRC, f) for f in ("api.cu", "noalloc.cu")] + [os.path.join(HERE, "host_fake.cpp")]
+    exe = os.path.join(tmp, "host_fake")
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-w", "-x", "c++"] + src + inc + ["-o", exe, "-lpthread"])
+    return exe
+
+
+@pytest.fixture(scope="session")
+def decide(tmp_path_factory):
+    exe = _program(str(tmp_path_factory.mktemp("host")))
+
+    def run(**kw):
+        out = subprocess.run([exe] + [f"{k}={v}" for k, v in kw.items()], capture_output=True, text=True, timeout=60)
+        assert out.returncode == 0, out.stderr
+        return out.stdout.splitlines()
+    return run
+
+
+def _elim(lines):
+    """(matrices or parts, CTAs of each, words left, words right) of every band elimination."""
+    return [tuple(int(w) for w in (x.split()[1], x.split()[2], x.split()[4], x.split()[6]))
+            for x in lines if x.startswith("band_elim")]
+
+
+@pytest.mark.parametrize("right", [0, 40, 300, 700])
+@pytest.mark.parametrize("call", [dict(count=1), dict(count=3), dict(counts=1)])
+def test_window_holds_the_next_panel(decide, right, call):
+    """A step of the elimination reads the next panel while the panel after the window is
+    loaded: the window has to reach one panel down also where no entry is below the diagonal."""
+    lines = decide(n=1000, left=0, right=right, **call)
+    assert "rc 0" in lines
+    assert _elim(lines) and all(left >= 1 for _, _, left, _ in _elim(lines)), lines
