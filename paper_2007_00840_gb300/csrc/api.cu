@@ -1155,10 +1155,12 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
 
 // One matrix by elimination on chip: as a band, or (larger ones) block by block of a
 // nested dissection.  *taken: the call is done (whatever it returns); otherwise nothing is
-// left behind and the traversal runs.
+// left behind and the traversal runs.  *checked: the CSR was checked and is valid (where
+// memory ran out before the scan it was not looked at).
 int run_band_single(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gsofa_options& o, cudaStream_t st,
-                    gsofa_result* out, bool* taken) {
+                    gsofa_result* out, bool* taken, bool* checked) {
   *taken = false;
+  *checked = false;
   zero_result(out);
   out->err_detail = -1;
   Events ev;
@@ -1183,6 +1185,7 @@ int run_band_single(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, con
       rc = GSOFA_E_INVAL;
       out->err_detail = b.counters()->bad_row ? INT_MAX - b.counters()->bad_row : -1;
     } else {
+      *checked = true;
       // near: most entries lie close to the diagonal and few far out, as in a dissection (mean
       // distance 0.04 of the band or less; bands and natural grids have 0.2 or more, with one
       // far entry per row 0.09)
@@ -2406,8 +2409,8 @@ int run_batch(Ctx* c, int32_t count, const int32_t* n, const int32_t* const* rp,
   for (size_t j = 0; rc == GSOFA_OK && j < singles.size(); j++) {
     const int32_t k = singles[j];
     if (n[k] >= FRONT_MIN_ORDER && band_allowed(o)) {
-      bool taken = false;
-      rc = run_band_single(c, n[k], rp[k], ci[k], o, st, &outs[k], &taken);
+      bool taken = false, checked = false;
+      rc = run_band_single(c, n[k], rp[k], ci[k], o, st, &outs[k], &taken, &checked);
       if (taken) {
         if (rc == GSOFA_OK) launches += outs[k].stats.kernel_launches;
         continue;
@@ -2635,10 +2638,10 @@ namespace {
 int run_single(Ctx* c, int32_t n, const int32_t* d_rowptr, const int32_t* d_colidx, gsofa_options o,
                cudaStream_t st, gsofa_result* out, int64_t nnz_known) {
   if (n > 0 && band_allowed(o)) {
-    bool taken = false;
-    const int rc = run_band_single(c, n, d_rowptr, d_colidx, o, st, out, &taken);
+    bool taken = false, checked = false;
+    const int rc = run_band_single(c, n, d_rowptr, d_colidx, o, st, out, &taken, &checked);
     if (taken) return rc;
-    o.validate = 2;  // checked above
+    if (checked) o.validate = 2;
   }
   const bool tune = o.autotune && o.frontier_order == 0 && n > 0;
   if (o.frontier_order == 0 && !tune) {

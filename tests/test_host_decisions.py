@@ -46,3 +46,13 @@ def test_window_holds_the_next_panel(decide, right, call):
     lines = decide(n=1000, left=0, right=right, **call)
     assert "rc 0" in lines
     assert _elim(lines) and all(left >= 1 for _, _, left, _ in _elim(lines)), lines
+
+
+def test_unscanned_pattern_is_validated(decide):
+    """Where memory runs out before the scan, the traversal checks the rows itself; where the
+    scan has checked them, it does not do so again."""
+    for at in (0, 1):
+        lines = decide(n=1000, left=40, right=40, fail_at=at)
+        assert "band_scan" not in lines and "validate" in lines and "rc 0" in lines, (at, lines)
+    lines = decide(n=20000, left=15000, right=15000)
+    assert "band_scan" in lines and "validate" not in lines and any(x.startswith("trav_class") for x in lines), lines
