@@ -625,7 +625,8 @@ int band_measure(BandRun& b, const gsofa_options& o) {
     rows += m.n;
     groups += ((int64_t)m.n + a.group_rows - 1) / a.group_rows;
   }
-  if (rows > INT32_MAX - 1024) return GSOFA_E_NOMEM;
+  // the loader looks up to LB + 3 panels past the last one (LB is at most 112 words)
+  if (rows > INT32_MAX - 4096) return GSOFA_E_NOMEM;
   a.nmats = (int32_t)B;
   a.one = b.mats[0];
   a.rows = rows;

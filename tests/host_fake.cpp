@@ -17,7 +17,6 @@
 
 // ---------------------------------------------------------------- what a scenario sets
 static int g_band_left = 0, g_band_right = 0;      // what the scan measures, for every matrix
-static long long g_fail_above = -1;                // pool allocations of more bytes fail
 static int g_fail_count = 0, g_fail_at = -1;       // the g_fail_at-th pool allocation from now on fails
 static std::map<void*, size_t> g_held;             // pool memory: bytes by block
 static size_t g_now = 0, g_peak = 0;
@@ -38,8 +37,7 @@ cudaError_t cudaMemPoolGetAttribute(cudaMemPool_t, cudaMemPoolAttr, void* v) { *
 cudaError_t cudaMemGetInfo(size_t* f, size_t* t) { *f = *t = (size_t)270 << 30; return cudaSuccess; }
 cudaError_t cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t, cudaStream_t) {
   *p = nullptr;
-  if ((g_fail_at >= 0 && g_fail_count++ == g_fail_at) || (g_fail_above >= 0 && (long long)n > g_fail_above))
-    return cudaErrorMemoryAllocation;
+  if (g_fail_at >= 0 && g_fail_count++ == g_fail_at) return cudaErrorMemoryAllocation;
   *p = std::calloc(1, n);
   if (!*p) return cudaErrorMemoryAllocation;
   g_held[*p] = n;
@@ -56,7 +54,10 @@ cudaError_t cudaFreeAsync(void* p, cudaStream_t) {
   std::free(p);
   return cudaSuccess;
 }
-cudaError_t cudaMalloc(void** p, size_t n) { *p = std::calloc(1, n); return *p ? cudaSuccess : cudaErrorMemoryAllocation; }
+cudaError_t cudaMalloc(void** p, size_t n) {
+  *p = n < (size_t)1 << 30 ? std::calloc(1, n) : nullptr;
+  return *p ? cudaSuccess : cudaErrorMemoryAllocation;
+}
 cudaError_t cudaFree(void* p) { std::free(p); return cudaSuccess; }
 cudaError_t cudaMallocHost(void** p, size_t n) { return cudaMalloc(p, n); }
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return cudaMalloc(p, n); }

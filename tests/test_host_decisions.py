@@ -56,3 +56,11 @@ def test_unscanned_pattern_is_validated(decide):
         assert "band_scan" not in lines and "validate" in lines and "rc 0" in lines, (at, lines)
     lines = decide(n=20000, left=15000, right=15000)
     assert "band_scan" in lines and "validate" not in lines and any(x.startswith("trav_class") for x in lines), lines
+
+
+@pytest.mark.parametrize("below", [2, 1100, 3700])
+def test_orders_near_the_largest_index(decide, below):
+    """The elimination's loader computes rows of up to LB + 4 panels past the end in 32 bits."""
+    n = 2**31 - 1 - below
+    assert n + 31 + 32 * (112 + 4) > 2**31 - 1
+    assert "band_scan" not in decide(n=n, rows=1, left=3500, right=1)
