@@ -80,8 +80,9 @@ typedef struct gsofa_options {
                                     level parity (default 512 with visited bitmaps in global memory,
                                     else 128; 32-1024) */
     int32_t max_ctas;            /* cap on traversal CTAs per launch, so concurrent launches share the GPU
-                                    (default 0: one full wave).  Elimination: CTAs of one banded matrix; a
-                                    batch and a dissection take one CTA or cluster per matrix or block */
+                                    (default 0: one full wave).  Elimination keeps to it as well (a batch
+                                    or a dissection in as many launches as that takes); a band or block
+                                    that needs a larger cluster of CTAs is traversed */
     int32_t frontier_order;      /* 0: automatic: elimination on chip where the pattern is banded or a
                                     nested dissection (of order 2,600 or more) and every option that
                                     concerns the traversal alone has its default; else class order for every

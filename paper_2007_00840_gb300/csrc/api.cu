@@ -578,13 +578,19 @@ bool band_allowed(const gsofa_options& o) {
          o.clean_heads == 0;
 }
 
+// CTAs that elimination may have on the GPU at a time: max_ctas, or no limit where the whole
+// GPU holds no more (four CTAs of 512 threads per SM).
+int cta_share(const Ctx* c, const gsofa_options& o) {
+  return o.max_ctas > 0 && o.max_ctas < 4 * c->sms ? o.max_ctas : INT_MAX;
+}
+
 // Device memory and results of one banded call (one matrix or a batch).
 struct BandRun {
   Ctx* c = nullptr;
   cudaStream_t st = nullptr;
   BandArgs a;
   std::vector<BandMat> mats;
-  int max_ctas = 0;  // of a single matrix's elimination, 0: the whole GPU
+  int share = INT_MAX;  // cta_share
   unsigned char* ctr = nullptr;   // BandCounters | band | mat_tot | nsuper | cross: zeroed together
   unsigned char* hctr = nullptr;  // pinned copy (all but cross)
   size_t ctr_bytes = 0, host_bytes = 0;
@@ -669,7 +675,7 @@ int64_t band_layout(BandRun& b) {
     BandMat& d = b.mats[m];
     d.LB = band_words_left(b.h_band()[2 * m]);
     d.UB = band_words_right(b.h_band()[2 * m + 1]);
-    if (!band_shape(d.LB, d.UB, false).C) return -1;
+    if (!band_shape(d.LB, d.UB, false, b.share).C) return -1;
     d.bits_base = words;
     words += (int64_t)d.n * (d.LB + d.UB + 1);
   }
@@ -702,20 +708,19 @@ int band_run(BandRun& b, int64_t words, Events& ev) {
   }
   ev.rec(2, st);
   if (B == 1) {
-    const BandShape s = band_shape(a.one.LB, a.one.UB, true);
+    const BandShape s = band_shape(a.one.LB, a.one.UB, true, b.share);
     const int panels = (a.one.n + 31) / 32;
-    const int ctas = b.max_ctas > 0 ? std::min(b.max_ctas, c->sms) : c->sms;
-    const int parts = std::max(1, std::min(panels, ctas / s.C));
+    const int parts = std::max(1, std::min(panels, std::min(b.share, c->sms) / s.C));
     if (e == cudaSuccess) e = launch_band_elim(a, parts, s.C, s.threads, s.smem, st);
     b.launches++;
   } else {
-    // matrices are sorted by shape: one launch per cluster size
+    // matrices are sorted by shape: one launch per cluster size (and share of the GPU)
     for (size_t m = 0; m < B && e == cudaSuccess;) {
-      const int C = band_shape(b.mats[m].LB, b.mats[m].UB, false).C;
+      const int C = band_shape(b.mats[m].LB, b.mats[m].UB, false, b.share).C;
       int threads = 0;
       size_t smem = 0, k = m;
-      for (; k < B; k++) {
-        const BandShape s = band_shape(b.mats[k].LB, b.mats[k].UB, false);
+      for (; k < B && k - m < (size_t)(b.share / C); k++) {
+        const BandShape s = band_shape(b.mats[k].LB, b.mats[k].UB, false, b.share);
         if (s.C != C) break;
         threads = std::max(threads, s.threads);
         smem = std::max(smem, s.smem);
@@ -845,6 +850,7 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
   l.end = rp + 1;
   l.col = ci;
   l.gid = gid0;
+  const int share = cta_share(c, o);
   std::vector<FrontBlock> blocks;
   FrontEmit e;
   std::memset(&e, 0, sizeof(e));
@@ -955,9 +961,9 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
         smem[b] = front_smem_bytes(m.sz, m.nr, m.nb, C);
         if (smem[b] <= BAND_SMEM_MAX - 1024) cs[b] = C;
       }
-      if (!cs[b]) return GSOFA_OK;
+      if (!cs[b] || cs[b] > share) return GSOFA_OK;
       // few fronts: more CTAs each
-      while (cs[b] < 8 && B * 2 * cs[b] <= (size_t)c->sms && pivots + (m.nr + 31) / 32 > 4 * cs[b]) {
+      while (cs[b] < 8 && B * 2 * cs[b] <= (size_t)std::min(c->sms, share) && pivots + (m.nr + 31) / 32 > 4 * cs[b]) {
         cs[b] *= 2;
         smem[b] = front_smem_bytes(m.sz, m.nr, m.nb, cs[b]);
       }
@@ -996,7 +1002,7 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
     f.piece_nL = l.piece_nL + l.pieces_before;
     for (size_t b = 0; b < B;) {
       size_t k = b, most = 0;
-      for (; k < B && cs[order[k]] == cs[order[b]]; k++) most = std::max(most, smem[order[k]]);
+      for (; k < B && cs[order[k]] == cs[order[b]] && k - b < (size_t)(share / cs[order[b]]); k++) most = std::max(most, smem[order[k]]);
       f.first = (int32_t)b;
       FK(launch_front_elim(f, (int)(k - b), cs[order[b]], (int)(k - b) > c->sms ? FRONT_MANY_THREADS : 512, most, st));
       *launches += 1;
@@ -1176,7 +1182,7 @@ int run_band_single(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, con
   m.colidx = ci;
   m.n = n;
   b.mats.push_back(m);
-  b.max_ctas = o.max_ctas;
+  b.share = cta_share(c, o);
   int rc = band_measure(b, o);
   ev.rec(1, st);
   int64_t words = -1;
@@ -1279,6 +1285,7 @@ int run_band_batch(Ctx* c, const std::vector<int32_t>& idx, const int32_t* n, co
     BandRun b;
     b.c = c;
     b.st = st;
+    b.share = cta_share(c, o);
     for (int32_t k : order) {
       BandMat m;
       std::memset(&m, 0, sizeof(m));
@@ -1298,7 +1305,7 @@ int run_band_batch(Ctx* c, const std::vector<int32_t>& idx, const int32_t* n, co
       std::vector<int> size(order.size());
       bool sorted = true;
       for (size_t m = 0; m < order.size(); m++) {
-        size[m] = band_shape(band_words_left(b.h_band()[2 * m]), band_words_right(b.h_band()[2 * m + 1]), false).C;
+        size[m] = band_shape(band_words_left(b.h_band()[2 * m]), band_words_right(b.h_band()[2 * m + 1]), false, b.share).C;
         if (size[m] == 0) rest->push_back(order[m]);
         if (size[m] == 0 || (m && size[m] < size[m - 1])) sorted = false;
       }

@@ -105,9 +105,12 @@ struct BandShape {
 // the cluster's barriers (us per 32 rows with 1 / 4 / 8 CTAs: LB 3: 1.6 / 2.3 / 2.4, LB 7:
 // 2.3 / 2.2 / 2.4, LB 10: 3.1 / 2.5 / 2.7, LB 33: - / 5.0 / 4.4).  Batches have other
 // matrices to fill the chip with and take the smallest cluster that holds the window.
-inline BandShape band_shape(int LB, int UB, bool alone) {
+// most: CTAs that one matrix may take (a caller's cap).
+inline BandShape band_shape(int LB, int UB, bool alone, int most = 8) {
   BandShape s;
-  for (int C = !alone || LB <= 8 ? 1 : (LB <= 16 ? 4 : 8); C <= 8; C *= 2) {
+  int first = !alone || LB <= 8 ? 1 : (LB <= 16 ? 4 : 8);
+  while (first > 1 && first > most) first /= 2;
+  for (int C = first; C <= 8 && C <= most; C *= 2) {
     const size_t b = band_smem_bytes(LB, UB, C);
     if (b > BAND_SMEM_MAX - 1024) continue;
     s.C = C;

@@ -17,6 +17,7 @@
 
 // ---------------------------------------------------------------- what a scenario sets
 static int g_band_left = 0, g_band_right = 0;      // what the scan measures, for every matrix
+static int g_blocks = 0;                           // a dissection: it falls into closed blocks
 static int g_fail_count = 0, g_fail_at = -1;       // the g_fail_at-th pool allocation from now on fails
 static std::map<void*, size_t> g_held;             // pool memory: bytes by block
 static size_t g_now = 0, g_peak = 0;
@@ -159,7 +160,16 @@ cudaError_t launch_band_count(const BandArgs&, cudaStream_t) { return cudaSucces
 cudaError_t launch_band_expand(const BandArgs&, cudaStream_t) { return cudaSuccess; }
 
 cudaError_t launch_front_blocks(const FrontLevel&, cudaStream_t) { std::puts("front_blocks"); return cudaSuccess; }
-cudaError_t launch_front_above(const FrontLevel&, cudaStream_t) { return cudaSuccess; }
+// blocks of 500 vertices that leave nothing for a next level, or none
+cudaError_t launch_front_above(const FrontLevel& l, cudaStream_t) {
+  if (!g_blocks) l.ctr->overflow = 1;
+  for (int b = 0; g_blocks && 500 * b < l.n; b++) {
+    l.ctr->nblocks = b + 1;
+    l.b_first[b] = 500 * b;
+    l.b_size[b] = l.n - 500 * b < 500 ? l.n - 500 * b : 500;
+  }
+  return cudaSuccess;
+}
 cudaError_t launch_front_reduce(const FrontLevel&, int32_t, const FrontMat*, const uint32_t*, int32_t*, int32_t*, int32_t*,
                                 int32_t*, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_front_whole(const FrontLevel&, cudaStream_t) { return cudaSuccess; }
@@ -189,8 +199,10 @@ int main(int argc, char** argv) {
   g_band_left = (int)get("left", 0);
   g_band_right = (int)get("right", 0);
   g_fail_at = (int)get("fail_at", -1);
+  g_blocks = (int)get("blocks", 0);
   gsofa_options o;
   gsofa_default_options(&o);
+  o.max_ctas = (int32_t)get("max_ctas", 0);
   std::vector<int32_t> rp((size_t)(get("rows", n) + 1), 0), ci(1, 0);
   std::vector<gsofa_result> out(count);
   int rc;

@@ -3,6 +3,8 @@ with members that have nothing below (or above) the diagonal beside others.  Sev
 matrices of one call have no stretch cuts, unlike a matrix alone."""
 import pytest
 
+import synth
+
 from tests.gpu_util import assert_same, oracle_full, to_device
 from tests.test_gpu_band import _edge
 
@@ -31,3 +33,19 @@ def test_served_upper_triangles():
     for t, A in zip(tickets, mats):
         assert_same(srv.wait(t)[0].to_host(), oracle_full(A))
     srv.close()
+
+
+@pytest.mark.parametrize("cap", [1, 5, 12])
+def test_capped_ctas(cap):
+    """Under a cap the elimination runs in several launches, or leaves a matrix to the traversal."""
+    import paper_2007_00840_gb300 as gs
+    opt = gs.options(max_ctas=cap)
+    mats = [_edge(900, bl, bu, seed=cap + bl) for bl, bu in [(5, 9), (300, 40), (600, 590), (0, 700), (870, 880)] * 3]
+    dev = [to_device(A) for A in mats]
+    want = [oracle_full(A) for A in mats]
+    for r, o in zip(gs.batch_device(dev, opts=opt), want):
+        assert_same(r.to_host(), o)
+    for d, o in list(zip(dev, want))[:5]:
+        assert_same(gs.symbolic_device(*d, opts=opt).to_host(), o)
+    nd = synth.grid2d_nd(130, 0.8, seed=cap)
+    assert_same(gs.symbolic_device(*to_device(nd), opts=opt).to_host(), oracle_full(nd, nthreads=16))

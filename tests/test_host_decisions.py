@@ -64,3 +64,30 @@ def test_orders_near_the_largest_index(decide, below):
     n = 2**31 - 1 - below
     assert n + 31 + 32 * (112 + 4) > 2**31 - 1
     assert "band_scan" not in decide(n=n, rows=1, left=3500, right=1)
+
+
+@pytest.mark.parametrize("cap", [1, 3, 7, 8, 20, 607])
+@pytest.mark.parametrize("reach", [30, 300, 700, 1200])
+@pytest.mark.parametrize("count", [1, 2, 45])
+def test_cap_on_ctas(decide, cap, reach, count):
+    """No launch of the elimination has more CTAs than max_ctas; every matrix is eliminated once
+    or traversed."""
+    lines = decide(n=9000, left=reach, right=reach, count=count, max_ctas=cap)
+    assert "rc 0" in lines
+    got = _elim(lines)
+    assert all(k * c <= cap for k, c, _, _ in got), lines
+    if any(x.startswith("trav") for x in lines):
+        assert not got and cap < 8 and reach > 30
+    else:
+        assert got if count == 1 else sum(k for k, _, _, _ in got) == count
+
+
+@pytest.mark.parametrize("cap", [0, 1, 5, 12, 39, 608])
+def test_cap_on_ctas_of_blocks(decide, cap):
+    lines = decide(n=20000, left=15000, right=15000, max_ctas=cap, blocks=1)
+    got = [tuple(map(int, x.split()[1:])) for x in lines if x.startswith("front_elim")]
+    assert sum(k for k, _ in got) == 40
+    if 0 < cap < 608:
+        assert all(k * c <= cap for k, c in got), lines
+    else:
+        assert len(got) == 1
