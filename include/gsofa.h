@@ -317,6 +317,11 @@ void gsofa_free(gsofa_result *res);
  * empty array, a host result or a field that does not exist. */
 void *gsofa_dlpack(const gsofa_result *res, int32_t field);
 
+/* What tells the device blocks of batch results apart: results with the same value have each
+ * field in one allocation, one matrix after the other (a batch may use several blocks: its
+ * bands and the matrices it traverses).  NULL: the result has its own allocations. */
+const void *gsofa_block(const gsofa_result *res);
+
 /* Human-readable name of an error code. */
 const char *gsofa_strerror(int code);
 

@@ -82,10 +82,9 @@ class DeviceResult:
     result and every tensor taken from it are gone).  Tensors are created on
     first access."""
 
-    def __init__(self, res: gsofa_result, stream: int, group=None):
+    def __init__(self, res: gsofa_result, stream: int):
         self._owner = _Owner(res)
         self._stream = stream
-        self._group = group  # results of one gsofa_batch call share one device block
         self._t = [None] * len(_FIELDS)
         self._stats = None
         self.n = res.n
@@ -98,6 +97,10 @@ class DeviceResult:
         if self._stats is None:
             self._stats = _stats(self._owner.res)
         return self._stats
+
+    def _block(self):
+        """The device block that this result shares with others of its batch call, None: its own."""
+        return _lib.load().gsofa_block(self._owner.ref)
 
     def _raw(self, name: str):
         """(device pointer, element count, typestr, torch dtype) of one output array."""
@@ -141,13 +144,14 @@ class DeviceResult:
 
 def results_to_host(results) -> list:
     """Copy device results to host arrays through pinned memory on the current
-    stream, with one synchronisation for all.  Arrays of one batch call that are
-    adjacent in device memory (its results share one block per field) are copied
-    as one span, so a batch costs a few large copies instead of six per matrix;
-    arrays of different calls are separate allocations and are copied apart."""
+    stream, with one synchronisation for all.  Adjacent arrays of one device block
+    (batch results share a block, with one allocation per field) are copied as one
+    span, so a batch costs a few large copies instead of six per matrix; arrays of
+    different blocks are separate allocations and are copied apart."""
     import torch
     out = [[None] * len(_FIELDS) for _ in results]
     pending = []
+    blocks = [r._block() for r in results]
     for f, nm in enumerate(_FIELDS):
         arrs = []
         for k, r in enumerate(results):
@@ -155,10 +159,7 @@ def results_to_host(results) -> list:
             if count == 0:
                 out[k][f] = (torch.empty(0, dtype=dtype), 0, 0)
             else:
-                # members of one batch call share a block (matrices above the on-chip
-                # limit, and empty ones, run alone and report their own traversal launches)
-                member = r._group is not None and r.n > 0 and r.stats.get("traverse_launches", 1) == 0
-                arrs.append((int(ptr), int(count), typestr, dtype, k, ("batch", r._group) if member else ("one", k)))
+                arrs.append((int(ptr), int(count), typestr, dtype, k, blocks[k]))
         arrs.sort(key=lambda x: x[0])
         i = 0
         while i < len(arrs):
@@ -167,7 +168,7 @@ def results_to_host(results) -> list:
             end = ptr0 + arrs[i][1] * esz
             j = i + 1
             while (j < len(arrs) and arrs[j][2] == typestr and arrs[j][0] == end and arrs[j][5] == arrs[i][5]
-                   and arrs[i][5][0] == "batch"):
+                   and arrs[i][5] is not None):
                 end += arrs[j][1] * esz
                 j += 1
             group = arrs[i:j]
@@ -298,11 +299,7 @@ def batch_device(mats, opts: gsofa_options | None = None, stream=None) -> list:
                          ctypes.c_void_p(sh), ctypes.cast(outs, ctypes.c_void_p))
     if rc != 0:
         raise GsofaError(rc, -1, "gsofa_batch")
-    res = []
-    group = object()
-    for i in range(k):
-        res.append(DeviceResult(gsofa_result.from_buffer_copy(outs[i]), sh, group))
-    return res
+    return [DeviceResult(gsofa_result.from_buffer_copy(outs[i]), sh) for i in range(k)]
 
 
 def row_counts_noalloc(rowptr, colidx, nnzL, nnzU, fill_count, stream=None) -> None:

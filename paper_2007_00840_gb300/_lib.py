@@ -137,6 +137,7 @@ SIGNATURES = {
     "gsofa_server_get_stats": (ctypes.c_int, [_P, ctypes.POINTER(gsofa_server_stats)]),
     "gsofa_server_destroy": (None, [_P]),
     "gsofa_free": (None, [ctypes.POINTER(gsofa_result)]),
+    "gsofa_block": (_P, [ctypes.POINTER(gsofa_result)]),
     "gsofa_dlpack": (_P, [ctypes.POINTER(gsofa_result), _I32]),
     "gsofa_strerror": (ctypes.c_char_p, [ctypes.c_int]),
     "gsofa_version": (ctypes.c_int, []),

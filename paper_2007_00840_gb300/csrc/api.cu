@@ -2603,6 +2603,10 @@ void* gsofa_dlpack(const gsofa_result* res, int32_t field) {
   return t;
 }
 
+const void* gsofa_block(const gsofa_result* res) {
+  return res && res->on_device && res->_priv ? ((const Priv*)res->_priv)->shared : nullptr;
+}
+
 void gsofa_free(gsofa_result* res) {
   if (!res) return;
   Priv* pv = (Priv*)res->_priv;

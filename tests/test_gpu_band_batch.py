@@ -49,3 +49,11 @@ def test_capped_ctas(cap):
         assert_same(gs.symbolic_device(*d, opts=opt).to_host(), o)
     nd = synth.grid2d_nd(130, 0.8, seed=cap)
     assert_same(gs.symbolic_device(*to_device(nd), opts=opt).to_host(), oracle_full(nd, nthreads=16))
+
+
+def test_bands_and_traversed_members_to_host_together():
+    import paper_2007_00840_gb300 as gs
+    mats = [A for k in range(6) for A in (_edge(512, 16 * k, 32, seed=k), synth.grid2d_nd(64, 0.8, seed=k))]
+    dev = [to_device(A) for A in mats]
+    for A, h in zip(mats, gs.results_to_host(gs.batch_device(dev))):
+        assert_same(h, oracle_full(A))
