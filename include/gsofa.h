@@ -60,7 +60,9 @@ typedef struct gsofa_options {
     int32_t max_concurrent;      /* global-label tier: concurrent source slots, one warp each (default: 32 per SM
                                     within the memory budget) */
     int64_t mem_budget_bytes;    /* global-label tier: half of it bounds the slots' memory (default: half of
-                                    the device memory free at first use, at most 96 GiB) */
+                                    the device memory free at first use, at most 96 GiB).  The same half
+                                    bounds the scratch of a dissection's elimination; a dissection that
+                                    needs more is traversed */
     int32_t fill_first;          /* 1: skip lowering the maxId of a vertex already known to be a fill
                                     (the optional "line 9.5" of Section 4); same result */
     int32_t collect_stats;       /* 1: record per-phase CUDA-event times and work counters (expanded vertices,

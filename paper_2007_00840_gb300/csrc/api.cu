@@ -789,38 +789,52 @@ constexpr int32_t FRONT_FIRST_BLOCK = 512;
 // grid 5.56 -> 5.23 ms; 256 the same, 192 5.32, 128 5.82)
 constexpr int FRONT_MANY_THREADS = 384;
 
-// Pool memory of one call, freed together.
+// Pool memory of one call, freed together; `left` is what the call may still take (shared by
+// all that it holds), past which an allocation fails.
 struct Held {
   Ctx* c;
   cudaStream_t st;
+  int64_t* left;
   std::vector<void*> ptrs;
+  int64_t bytes = 0;
   bool ok = true;
   template <typename T>
   T* get(size_t count) {
     T* p = nullptr;
-    if (!ok || palloc(c, &p, count, st) != cudaSuccess) {
+    const int64_t b = (int64_t)(sizeof(T) * count);
+    if (!ok || b > *left || palloc(c, &p, count, st) != cudaSuccess) {
       cudaGetLastError();
       ok = false;
       return nullptr;
     }
+    *left -= b;
+    bytes += b;
     ptrs.push_back(p);
     return p;
   }
   void free_all() {
     for (void* p : ptrs) cudaFreeAsync(p, st);
     ptrs.clear();
+    *left += bytes;
+    bytes = 0;
+  }
+  void swap(Held& o) {
+    std::swap(ptrs, o.ptrs);
+    std::swap(bytes, o.bytes);
   }
   ~Held() { free_all(); }
 };
 
 // One matrix by elimination of its dissection blocks (fronts.cu).  The CSR has been
 // checked; fill holds every row's entries of A (diagonal counted) and becomes the result's
-// fill counts.  *taken: done (whatever it returns); otherwise the pattern is not ordered
-// for it, or memory ran out, and nothing is left behind but fill as it was.
+// fill counts.  Its scratch keeps to the memory that the traversal's slots may take: a server
+// charges a large request for those.  *taken: done (whatever it returns); otherwise the
+// pattern is not ordered for it, or memory ran out, and nothing is left behind but fill as it was.
 int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gsofa_options& o, cudaStream_t st,
                int32_t* fill, gsofa_result* out, Events& ev, int* launches, bool* taken) {
   *taken = false;
-  Held keep{c, st}, level_mem{c, st}, next_mem{c, st};
+  int64_t left = global_budget(c, o);
+  Held keep{c, st, &left}, level_mem{c, st, &left}, next_mem{c, st, &left};
   const int32_t pcap = n > (1 << 27) ? 0 : 4 * n + 1024;
   if (!pcap) return GSOFA_OK;
   FrontLevel l;
@@ -1037,7 +1051,7 @@ int run_fronts(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, const gs
         e.left = n1;
       }
       level_mem.free_all();
-      std::swap(level_mem.ptrs, next_mem.ptrs);
+      level_mem.swap(next_mem);
       l.blocks_before = (int32_t)(b0 + B);
       l.pieces_before += br_total;
       l.n = n1;

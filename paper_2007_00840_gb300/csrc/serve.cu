@@ -275,6 +275,8 @@ void worker_loop(gsofa_server* S, int slot) {
       gsofa_options o = S->cfg.opts;
       if (take[0]->budget > 0) o.mem_budget_bytes = take[0]->budget;
       if (big_budget > 0) o.mem_budget_bytes = big_budget;
+      // what was charged for its slots, also where it is eliminated block by block
+      if (o.mem_budget_bytes == 0 && reserved > 0) o.mem_budget_bytes = 2 * reserved;
       if (o.max_ctas == 0) o.max_ctas = S->sms * 4;
       run_alone(0, o);
     }

@@ -178,7 +178,7 @@ cudaError_t launch_front_gids(const FrontLevel&, int32_t, int32_t*, cudaStream_t
 cudaError_t launch_front_count(const FrontEmit&, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_front_expand(const FrontEmit&, cudaStream_t) { return cudaSuccess; }
 cudaError_t launch_front_elim(const FrontArgs&, int count, int C, int, size_t, cudaStream_t) {
-  std::printf("front_elim %d %d\n", count, C);
+  std::printf("front_elim %d %d held %zu\n", count, C, g_now);
   return cudaSuccess;
 }
 
@@ -203,6 +203,7 @@ int main(int argc, char** argv) {
   gsofa_options o;
   gsofa_default_options(&o);
   o.max_ctas = (int32_t)get("max_ctas", 0);
+  o.mem_budget_bytes = get("budget", 0);
   std::vector<int32_t> rp((size_t)(get("rows", n) + 1), 0), ci(1, 0);
   std::vector<gsofa_result> out(count);
   int rc;

@@ -85,9 +85,25 @@ def test_cap_on_ctas(decide, cap, reach, count):
 @pytest.mark.parametrize("cap", [0, 1, 5, 12, 39, 608])
 def test_cap_on_ctas_of_blocks(decide, cap):
     lines = decide(n=20000, left=15000, right=15000, max_ctas=cap, blocks=1)
-    got = [tuple(map(int, x.split()[1:])) for x in lines if x.startswith("front_elim")]
+    got = [tuple(map(int, x.split()[1:3])) for x in lines if x.startswith("front_elim")]
     assert sum(k for k, _ in got) == 40
     if 0 < cap < 608:
         assert all(k * c <= cap for k, c in got), lines
     else:
         assert len(got) == 1
+
+
+@pytest.mark.parametrize("budget", [1 << 18, 1 << 20, 1 << 22, 1 << 23, 1 << 24, 1 << 25, 0])
+def test_budget_of_blocks(decide, budget):
+    """The elimination of a dissection holds no more scratch than the traversal's slots might;
+    past that the matrix is traversed, with the slots that fit."""
+    n = 20000
+    lines = decide(n=n, left=15000, right=15000, blocks=1, budget=budget)
+    assert "rc 0" in lines and "held 0" in lines
+    held = [int(x.split()[4]) for x in lines if x.startswith("front_elim")]
+    if budget in (0, 1 << 25):
+        assert held
+    if held:
+        assert budget == 0 or max(held) <= budget // 2 + 5 * n  # besides counters and fill counts
+    else:
+        assert any(x.startswith("trav_class") for x in lines)
