@@ -24,6 +24,7 @@
 #include "fronts.cuh"
 #include "gsofa.h"
 #include "internal.cuh"
+#include "route.cuh"
 
 namespace gsofa {
 
@@ -591,7 +592,7 @@ struct BandRun {
   BandArgs a;
   std::vector<BandMat> mats;
   int share = INT_MAX;  // cta_share
-  unsigned char* ctr = nullptr;   // BandCounters | band | mat_tot | nsuper | cross: zeroed together
+  unsigned char* ctr = nullptr;   // BandCounters | reach | band | mat_tot | nsuper | cross: zeroed together
   unsigned char* hctr = nullptr;  // pinned copy (all but cross)
   size_t ctr_bytes = 0, host_bytes = 0;
   BandMat* d_mats = nullptr;
@@ -603,9 +604,10 @@ struct BandRun {
   int launches = 0;
 
   const BandCounters* counters() const { return (const BandCounters*)hctr; }
-  int32_t* h_band() const { return (int32_t*)(hctr + 64); }
-  unsigned long long* h_tot() const { return (unsigned long long*)(hctr + 64 + 8 * mats.size()); }
-  int32_t* h_nsuper() const { return (int32_t*)(hctr + 64 + 24 * mats.size()); }
+  const BandReach& h_reach(size_t m) const { return ((const BandReach*)(hctr + 64))[m]; }
+  int32_t* h_band() const { return (int32_t*)(hctr + 64 + 16 * mats.size()); }
+  unsigned long long* h_tot() const { return (unsigned long long*)(hctr + 64 + 24 * mats.size()); }
+  int32_t* h_nsuper() const { return (int32_t*)(hctr + 64 + 40 * mats.size()); }
   void free_scratch() {
     pfree(ctr, st); pfree(d_mats, st); pfree(nL, st); pfree(nU, st); pfree(flags, st);
     pfree(part, st); pfree(bits, st);
@@ -615,8 +617,11 @@ struct BandRun {
   }
 };
 
-// Lay out the matrices, check them and measure their bands (one wait).
-int band_measure(BandRun& b, const gsofa_options& o) {
+static_assert(sizeof(BandCounters) <= 64 && sizeof(BandReach) == 16, "the layout of BandRun::ctr");
+
+// Lay out the matrices, check them and measure their bands and the reach of the first
+// `sampled` of them (one wait).
+int band_measure(BandRun& b, const gsofa_options& o, int32_t sampled) {
   Ctx* c = b.c;
   cudaStream_t st = b.st;
   const size_t B = b.mats.size();
@@ -638,7 +643,7 @@ int band_measure(BandRun& b, const gsofa_options& o) {
   a.rows = rows;
   a.groups = groups;
   const size_t cross_words = B == 1 ? (size_t)rows / 1024 + 2 : 0;
-  b.host_bytes = 64 + 28 * B;
+  b.host_bytes = 64 + 44 * B;
   b.ctr_bytes = ((b.host_bytes + 15) & ~(size_t)15) + 4 * cross_words;
   b.hctr = (unsigned char*)thread_pinned(b.host_bytes, 1);
   if (!b.hctr) return GSOFA_E_NOMEM;
@@ -657,14 +662,22 @@ int band_measure(BandRun& b, const gsofa_options& o) {
     a.mats = b.d_mats;
   }
   a.ctr = (BandCounters*)b.ctr;
-  a.band = (int32_t*)(b.ctr + 64);
-  a.mat_tot = B > 1 ? (unsigned long long*)(b.ctr + 64 + 8 * B) : nullptr;
-  a.mat_nsuper = (int32_t*)(b.ctr + 64 + 24 * B);
+  a.reach = (BandReach*)(b.ctr + 64);
+  a.band = (int32_t*)(b.ctr + 64 + 16 * B);
+  a.mat_tot = B > 1 ? (unsigned long long*)(b.ctr + 64 + 24 * B) : nullptr;
+  a.mat_nsuper = (int32_t*)(b.ctr + 64 + 40 * B);
+  a.sampled = sampled;
+  a.reach_rows = reach_rows(sampled);
+  a.most_rows = b.mats[0].n;  // (a batch is sampled largest first)
   a.cross = cross_words ? (uint32_t*)(b.ctr + ((b.host_bytes + 15) & ~(size_t)15)) : nullptr;
   a.fill = b.fill;
   if (launch_band_scan(a, st) != cudaSuccess) return GSOFA_E_CUDA;
   b.launches++;
-  if (cudaMemcpyAsync(b.hctr, b.ctr, 64 + 8 * B, cudaMemcpyDeviceToHost, st) != cudaSuccess) return GSOFA_E_CUDA;
+  if (sampled > 0) {
+    if (launch_band_reach(a, false, st) != cudaSuccess) return GSOFA_E_CUDA;
+    b.launches++;
+  }
+  if (cudaMemcpyAsync(b.hctr, b.ctr, 64 + 24 * B, cudaMemcpyDeviceToHost, st) != cudaSuccess) return GSOFA_E_CUDA;
   return wait_stream(st);
 }
 
@@ -766,23 +779,6 @@ void band_times(Events& ev, gsofa_stats* s) {
 }
 
 // ---------------------------------------------------------------- nested dissection
-// Orders from which the blocks of a dissection are looked for: any pattern whose band does
-// not fit, and one that looks like a dissection (entries near the diagonal, few far out).
-// Dissections of square grids, traversal / blocks: order 2,025 414 / 455 us, 2,809 468 /
-// 452, 4,900 628 / 469, 10,000 993 / 561, 16,256 1,351 / 631.
-constexpr int32_t FRONT_MIN_ORDER = 16384;
-constexpr int32_t FRONT_NEAR_ORDER = 2600;
-// Up to this order a dissection is one wide band (order 900: 283 us by traversal, 219 as a
-// band; 1,600: 370 / 357; 2,025: 414 / 483); between the two lines it is traversed.
-constexpr int32_t NEAR_BAND_ORDER = 1600;
-// A band of more words than this needs a cluster of eight, 4 us per panel whatever is in it;
-// with fewer entries than this in all the traversal is as fast or faster (3D grids: 27 x 27
-// x 9, 37k entries, 942 us by traversal, 1,177 as a band; 33 x 33 x 9, 52k: 1,688 / 1,834;
-// 27 x 27 x 20, 82k: 2,408 / 2,212; 33 x 33 x 20, 119k: 4,702 / 3,788), except for small
-// orders (band 1,000 of order 3,000: 1,025 / 651).
-constexpr int32_t WIDE_BAND = 16;
-constexpr unsigned long long WIDE_NNZ = 56000;
-constexpr int32_t WIDE_MIN_ORDER = 4096;
 constexpr int32_t FRONT_LAST_ORDER = 2900;
 constexpr int32_t FRONT_FIRST_BLOCK = 512;
 // threads of a front where there are more fronts than SMs: two CTAs fit an SM (1024 x 1024
@@ -1197,30 +1193,40 @@ int run_band_single(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, con
   m.n = n;
   b.mats.push_back(m);
   b.share = cta_share(c, o);
-  int rc = band_measure(b, o);
+  int rc = band_measure(b, o, n >= REACH_MIN_ORDER ? 1 : 0);
   ev.rec(1, st);
   int64_t words = -1;
-  bool near = false;
+  bool near = false, blocks = false;
   if (rc == GSOFA_OK) {
     if (b.counters()->err) {
       rc = GSOFA_E_INVAL;
       out->err_detail = b.counters()->bad_row ? INT_MAX - b.counters()->bad_row : -1;
     } else {
       *checked = true;
-      // near: most entries lie close to the diagonal and few far out, as in a dissection (mean
-      // distance 0.04 of the band or less; bands and natural grids have 0.2 or more, with one
-      // far entry per row 0.09)
       const BandCounters& h = *b.counters();
-      const int32_t width = std::max(b.h_band()[0], b.h_band()[1]);
-      near = h.spread < h.nnz * (unsigned long long)width / 16;
+      near = near_diagonal(h, b.h_band());
       words = band_layout(b);
-      const bool wide = b.mats[0].LB > WIDE_BAND;
-      if (words >= 0 && wide && (near ? n > NEAR_BAND_ORDER : n >= WIDE_MIN_ORDER && h.nnz < WIDE_NNZ))
+      const BandMat& m = b.mats[0];
+      if (words >= 0 && m.LB > WIDE_BAND && (near ? n > NEAR_BAND_ORDER : n >= WIDE_MIN_ORDER && h.nnz < WIDE_NNZ))
         words = -1;
+      blocks = n >= (near ? FRONT_NEAR_ORDER : FRONT_MIN_ORDER);
+      if (b.a.sampled && b.h_reach(0).levels) {
+        const float traverse = traverse_us(n, b.h_reach(0), b.a.reach_rows, false);
+        if (words >= 0) {
+          const int C = band_shape(m.LB, m.UB, true, b.share).C;
+          const int chain = chain_panels(n, h.stretch, std::max(1, std::min(b.share, c->sms) / C));
+          if (ROUTE_MARGIN * traverse < band_us(n, chain, m.LB, m.UB, false)) {
+            words = -1;
+            blocks = false;
+          }
+        } else {
+          blocks = blocks && traverse > fronts_limit_us(n);
+        }
+      }
       if (words >= 0) rc = band_run(b, words, ev);
     }
   }
-  if (rc == GSOFA_OK && words < 0 && n >= (near ? FRONT_NEAR_ORDER : FRONT_MIN_ORDER)) {
+  if (rc == GSOFA_OK && words < 0 && blocks) {
     bool fronts = false;
     int launches = b.launches;
     rc = run_fronts(c, n, rp, ci, o, st, b.fill, out, ev, &launches, &fronts);
@@ -1309,7 +1315,9 @@ int run_band_batch(Ctx* c, const std::vector<int32_t>& idx, const int32_t* n, co
       b.mats.push_back(m);
     }
     ev.rec(0, st);
-    int rc = band_measure(b, o);
+    int32_t sampled = 0;  // once, the largest
+    while (pass == 0 && sampled < (int32_t)order.size() && n[order[sampled]] >= REACH_MIN_ORDER) sampled++;
+    int rc = band_measure(b, o, sampled);
     ev.rec(1, st);
     int64_t words = -1;
     if (rc == GSOFA_OK && b.counters()->err) rc = GSOFA_E_INVAL;
@@ -1318,8 +1326,20 @@ int run_band_batch(Ctx* c, const std::vector<int32_t>& idx, const int32_t* n, co
       std::vector<int32_t> next;
       std::vector<int> size(order.size());
       bool sorted = true;
+      std::vector<float> chain(order.size(), 0.f);  // us
+      float all = 0.f;
       for (size_t m = 0; m < order.size(); m++) {
-        size[m] = band_shape(band_words_left(b.h_band()[2 * m]), band_words_right(b.h_band()[2 * m + 1]), false, b.share).C;
+        const int LB = band_words_left(b.h_band()[2 * m]), UB = band_words_right(b.h_band()[2 * m + 1]);
+        size[m] = band_shape(LB, UB, false, b.share).C;
+        chain[m] = band_us(n[order[m]], (n[order[m]] + 31) / 32, LB, UB, false);
+        all += chain[m] * (float)size[m];
+      }
+      for (size_t m = 0; m < order.size(); m++) {
+        // a band that outlasts the others and that the traversal would have done sooner
+        if ((int32_t)m < sampled && size[m] && chain[m] > 2.f * all / (float)c->sms &&
+            b.h_reach(m).levels &&
+            ROUTE_MARGIN * traverse_us(n[order[m]], b.h_reach(m), b.a.reach_rows, false) < chain[m])
+          size[m] = 0;
         if (size[m] == 0) rest->push_back(order[m]);
         if (size[m] == 0 || (m && size[m] < size[m - 1])) sorted = false;
       }

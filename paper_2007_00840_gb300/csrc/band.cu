@@ -32,6 +32,7 @@
 #include <cooperative_groups.h>
 
 #include "band.cuh"
+#include "route.cuh"
 
 namespace gsofa {
 
@@ -214,6 +215,195 @@ __global__ void __launch_bounds__(256) band_scan_kernel(BandArgs a) {
     atomicAdd(&a.ctr->spread, spread);
     if (max_l > *(volatile int32_t*)a.band) atomicMax(a.band, max_l);
     if (max_u > *(volatile int32_t*)(a.band + 1)) atomicMax(a.band + 1, max_u);
+  }
+}
+
+// ------------------------------------------------------------ reach of sampled rows
+// A CTA per sampled row s (one in each of reach_rows equal parts of a matrix, at a place
+// that does not repeat with its structure): breadth-first search from s over vertices below
+// s, level by level, a thread (or eight) per vertex, vertices found marked in a bitmap.
+// Cut off after what the choice of the route can still use.  Bound by the latency of a
+// level: row pointers, columns, bitmap, a barrier, 1.3 us or more.  Takes 14 us beside the
+// 340 of a 64 x 64 grid, where it is left out, 45 on a band of 211 (1,290), 90 on 32^3
+// (4,690), 150 on 317 x 293 (7,360).  The last CTA finds the longest stretch of one matrix.
+namespace {
+constexpr int REACH_THREADS = 512;
+constexpr int REACH_QUEUE = 1024;   // vertices of a level
+constexpr int REACH_WORDS = 49152;  // of the bitmap at most: a search that goes further back is cut off
+// Words of the bitmap for orders up to n (a multiple of four; room for the stretches' sums).
+int reach_words(int n) {
+  const int w = ((n - 1) / 32 + 4) & ~3;
+  return w > REACH_WORDS ? REACH_WORDS : (w < 3 * REACH_THREADS ? 3 * REACH_THREADS : w);
+}
+}  // namespace
+__global__ void __launch_bounds__(REACH_THREADS) band_reach_kernel(BandArgs a, bool counts, int words) {
+  extern __shared__ __align__(16) uint32_t bsm[];
+  uint32_t* seen = bsm;                      // vertices first .. first + 32 words - 1
+  int32_t* queue = (int32_t*)(bsm + words);  // [2][REACH_QUEUE]
+  __shared__ int s_stretches;
+  __shared__ struct { int found, cut; uint32_t entries; } level[3];  // one barrier a level: read, written, cleared
+  const int m = blockIdx.x / a.reach_rows, k = blockIdx.x % a.reach_rows;
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (m >= a.sampled) {
+    // panel q > 0 starts a stretch where bit q of cross is clear; a thread takes some words in
+    // turn: first and last start in them, and the longest stretch between
+    const int panels = (a.one.n + 31) >> 5, cw = (panels + 31) >> 5;
+    const int some = (cw + REACH_THREADS - 1) / REACH_THREADS;
+    int first = -1, last = -1, most = 0;
+    for (int w = some * tid; w < min(cw, some * (tid + 1)); w++) {
+      uint32_t open = ~a.cross[w];
+      if (w == 0) open |= 1u;
+      for (; open; open &= open - 1) {
+        const int q = 32 * w + __ffs(open) - 1;
+        if (q >= panels) break;
+        if (first < 0) first = q;
+        else most = max(most, q - last);
+        last = q;
+      }
+    }
+    int32_t* part = (int32_t*)bsm;
+    part[tid] = first;
+    part[REACH_THREADS + tid] = last;
+    part[2 * REACH_THREADS + tid] = most;
+    __syncthreads();
+    if (tid == 0) {
+      int at = 0;
+      for (int t = 0; t < REACH_THREADS; t++) {
+        if (part[t] < 0) continue;
+        most = max(most, max(part[2 * REACH_THREADS + t], part[t] - at));
+        at = part[REACH_THREADS + t];
+      }
+      a.ctr->stretch = max(most, panels - at);
+    }
+    return;
+  }
+  const BandMat d = a.mats ? a.mats[m] : a.one;
+  const int n = d.n;
+  const int err = a.ctr->err, LB = band_words_left(a.band[2 * m]), UB = band_words_right(a.band[2 * m + 1]);
+  const int nnz = d.rowptr[n], panels = (n + 31) >> 5;
+  if (tid == 0) s_stretches = 1;
+  for (int i = tid; i < words / 4; i += REACH_THREADS) ((uint4*)seen)[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (err) return;  // nothing is followed unchecked
+  const bool fits = band_shape(LB, UB, false).C > 0;
+  if (!fits && a.mats) return;
+  // the panels in a chain: where there are stretches, about four of the mean length
+  int chain = panels;
+  if (a.cross) {
+    __syncthreads();
+    int open = 0;
+    for (int w = tid; 32 * w < panels; w += REACH_THREADS) {
+      const uint32_t inside = panels - 32 * w < 32 ? (1u << (panels & 31)) - 1u : FULL;
+      open += __popc(~a.cross[w] & inside & (w == 0 ? ~1u : FULL));
+    }
+    open = __reduce_add_sync(FULL, open);
+    if (lane == 0 && open) atomicAdd(&s_stretches, open);
+    __syncthreads();
+    chain = min(panels, 4 * (panels / s_stretches + 1));
+  }
+  const float band = fits ? band_us(n, chain, LB, UB, counts) : 0.f;
+  const float limit = reach_limit_us(n, band, counts);
+  if (limit <= 0.f) return;
+  const TraverseCost cost = traverse_cost(n, counts);
+  const float row_ns = 1e3f * limit / (float)n;
+  // a row is searched up to this cost: one and a half times its share, more where the elimination takes long
+  // (20 ms a share more: of a million rows of degree 1.3 some are long, 99 ms against 24)
+  const float most_ns = row_ns * (1.5f + 5e-5f * band);
+  // as many levels as take 2% of the elimination, at 1 us each
+  const int most_levels = max(6, (int)(0.02f * (fits ? band : fronts_us(n))));
+
+  const uint32_t place = ((uint32_t)k * 2654435761u) >> 16;
+  const int s = (int)((((long long)k << 16) + place) * n / ((long long)a.reach_rows << 16));
+  const int first = max(0, s - 32 * words + 1);
+  const int lanes = nnz / n > 16 ? 8 : 1;  // threads per vertex; rows of more than 64 entries each end the search
+  const int sub = tid & (lanes - 1);
+  if (tid == 0) {
+    queue[0] = s;
+    level[1] = {0, 0, 0u};
+  }
+  uint32_t all = 0u;
+  int levels = 0, count = 1;
+  bool cut = false;
+  __syncthreads();
+  while (count > 0) {
+    const int32_t* in = queue + REACH_QUEUE * (levels & 1);
+    int32_t* out = queue + REACH_QUEUE * ((levels & 1) ^ 1);
+    auto& next = level[(levels + 1) % 3];
+    if (tid == 0) level[(levels + 2) % 3] = {0, 0, 0u};
+    uint32_t entries = 0u;
+    for (int i0 = 0; i0 < count; i0 += REACH_THREADS / lanes) {
+      const int i = i0 + tid / lanes;
+      uint32_t b = 0, e = 0;  // unsigned: x may pass the largest index
+      if (i < count) {
+        const int v = in[i];
+        b = (uint32_t)d.rowptr[v];
+        e = (uint32_t)d.rowptr[v + 1];
+        if (sub == 0) entries += e - b;
+        if (e - b > 64u * lanes) {
+          next.cut = 1;
+          e = b;
+        }
+      }
+      for (uint32_t x = b + sub; __any_sync(FULL, x < e); x += 8 * lanes) {
+        // eight columns at a time: loads, then marks, in flight together (no mark: no bit of word 0)
+        int c[8];
+        uint32_t bit[8], old[8];
+#pragma unroll
+        for (int j = 0; j < 8; j++) c[j] = x + j * lanes < e ? d.colidx[x + j * lanes] : s;
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+          const bool in_range = c[j] < s && c[j] >= first;
+          bit[j] = in_range ? 1u << ((c[j] - first) & 31) : 0u;
+          old[j] = atomicOr(seen + (in_range ? (c[j] - first) >> 5 : 0), bit[j]);
+        }
+        unsigned fresh = 0u, far = 0u;
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+          if (bit[j] & ~old[j]) fresh |= 1u << j;
+          far |= c[j] < first;
+        }
+        if (far) next.cut = 1;
+        int before = __popc(fresh);
+        const int mine = before;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(FULL, before, o);
+          if (lane >= o) before += y;
+        }
+        int at = 0;
+        if (lane == 31 && before > 0) at = atomicAdd(&next.found, before);
+        at = __shfl_sync(FULL, at, 31) + before - mine;
+#pragma unroll
+        for (int j = 0; j < 8; j++)
+          if ((fresh >> j) & 1u) {
+            if (at < REACH_QUEUE) out[at] = c[j];
+            at++;
+          }
+      }
+    }
+    if (__any_sync(FULL, entries > 0u)) {
+      entries = __reduce_add_sync(FULL, entries);
+      if (lane == 0) atomicAdd(&next.entries, entries);
+    }
+    __syncthreads();
+    levels++;
+    count = next.found;
+    all += next.entries;
+    cut = next.cut || count > REACH_QUEUE || levels >= most_levels ||
+          cost.level * (float)levels + cost.entry * (float)all > most_ns ||
+          row_us((float)levels, (float)all) > 1.5f * limit;
+    if (cut) {
+      cut = next.cut || count > 0;
+      break;
+    }
+  }
+  if (tid == 0) {
+    unsigned long long entries = all;
+    // cut off: as if it reached every row before it, and never less than three times its share
+    if (cut) entries = max(entries, (unsigned long long)s * (unsigned long long)nnz / (unsigned long long)n);
+    atomicMax(&a.reach[m].longest, (uint32_t)fminf(row_us((float)levels, (float)entries), 4e9f) + 1u);
+    if (cut) entries = max(entries, (unsigned long long)(3.f * row_ns / cost.entry));
+    atomicAdd(&a.reach[m].entries, entries);
+    atomicAdd(&a.reach[m].levels, (uint32_t)levels);
   }
 }
 
@@ -1145,6 +1335,17 @@ cudaError_t launch_band_scan(const BandArgs& a, cudaStream_t st) {
   long long grid = (a.rows + 255) / 256;
   if (grid > 4096) grid = 4096;
   band_scan_kernel<<<(int)grid, 256, 0, st>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_band_reach(const BandArgs& a, bool counts, cudaStream_t st) {
+  if (a.sampled <= 0) return cudaSuccess;
+  const int words = reach_words(a.most_rows);
+  const size_t smem = 4 * ((size_t)words + 2 * REACH_QUEUE);
+  const cudaError_t e = cudaFuncSetAttribute(band_reach_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             4 * (REACH_WORDS + 2 * REACH_QUEUE));
+  if (e != cudaSuccess) return e;
+  band_reach_kernel<<<a.sampled * a.reach_rows + (a.cross ? 1 : 0), REACH_THREADS, smem, st>>>(a, counts, words);
   return cudaGetLastError();
 }
 

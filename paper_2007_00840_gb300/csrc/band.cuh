@@ -17,14 +17,22 @@ struct BandCounters {
   int32_t bad_row;      // INT_MAX - first offending row (0: none)
   int32_t n_super;
   int32_t groups_done;
+  int32_t stretch;      // one matrix: panels of its longest stretch between uncrossed boundaries (band_reach_kernel)
+};
+
+// What the sampled rows of a matrix reach: sums of the entries and levels of their searches,
+// and the longest of them by itself (row_us, rounded up).
+struct BandReach {
+  unsigned long long entries;
+  uint32_t levels, longest;
 };
 
 // Words of columns that a band of `reach` columns takes left and right of a row's own word.
 // Left at least one: the window is the panels P .. P + LB, and while step P reads panel P + 1
 // the loader writes panel P + LB + 1.  With none a batch's chain read panel P + 1 before it
 // was there (a single matrix without entries below the diagonal is one stretch per panel).
-inline int band_words_left(int32_t reach) { return reach > 32 ? (reach + 31) / 32 : 1; }
-inline int band_words_right(int32_t reach) { return (reach + 31) / 32; }
+__host__ __device__ inline int band_words_left(int32_t reach) { return reach > 32 ? (reach + 31) / 32 : 1; }
+__host__ __device__ inline int band_words_right(int32_t reach) { return (reach + 31) / 32; }
 
 // One matrix.  LB, UB: band_words_left and band_words_right of its band.
 struct BandMat {
@@ -47,6 +55,10 @@ struct BandArgs {
   int32_t group_rows;   // rows per group: a multiple of chunk
   BandCounters* ctr;
   int32_t* band;        // per matrix: largest i - j, largest j - i
+  BandReach* reach;     // per matrix
+  int32_t sampled;      // matrices whose rows are sampled: the first ones
+  int32_t reach_rows;   // rows sampled of each
+  int32_t most_rows;    // the largest order among them
   uint32_t* cross;      // one matrix: bit q set where an entry below the diagonal crosses row 32q (null: batch)
   uint32_t* bits;       // null (one matrix): per-row sizes and fill counts only
   int32_t *row_nL, *row_nU, *fill, *flags;
@@ -88,7 +100,7 @@ inline size_t front_smem_bytes(int sz, int nr, int nb, int C) {
 // Clusters of C CTAs for fronts [a.first, a.first + count).
 cudaError_t launch_front_elim(const FrontArgs& a, int count, int C, int threads, size_t smem, cudaStream_t st);
 
-inline size_t band_smem_bytes(int LB, int UB, int C) {
+__host__ __device__ inline size_t band_smem_bytes(int LB, int UB, int C) {
   const int wx = LB + UB + 1;
   const size_t slots = (size_t)(LB + 2 + C - 1) / C;
   return 4 * (128 + 64 + 68 + 192 * (size_t)(UB | 1) + 4 * BAND_STAGE + slots * 32 * (size_t)((wx | 1) + 1));
@@ -106,7 +118,7 @@ struct BandShape {
 // 2.3 / 2.2 / 2.4, LB 10: 3.1 / 2.5 / 2.7, LB 33: - / 5.0 / 4.4).  Batches have other
 // matrices to fill the chip with and take the smallest cluster that holds the window.
 // most: CTAs that one matrix may take (a caller's cap).
-inline BandShape band_shape(int LB, int UB, bool alone, int most = 8) {
+__host__ __device__ inline BandShape band_shape(int LB, int UB, bool alone, int most = 8) {
   BandShape s;
   int first = !alone || LB <= 8 ? 1 : (LB <= 16 ? 4 : 8);
   while (first > 1 && first > most) first /= 2;
@@ -125,6 +137,8 @@ inline BandShape band_shape(int LB, int UB, bool alone, int most = 8) {
 }
 
 cudaError_t launch_band_scan(const BandArgs& a, cudaStream_t st);
+// After the scan: reach and stretch of the first a.sampled matrices.  counts: for sizes alone.
+cudaError_t launch_band_reach(const BandArgs& a, bool counts, cudaStream_t st);
 // `count` matrices from a.first on, or the parts one matrix's panels are dealt to: C CTAs (a cluster) each.
 cudaError_t launch_band_elim(const BandArgs& a, int count, int C, int threads, size_t smem, cudaStream_t st);
 cudaError_t launch_band_count(const BandArgs& a, cudaStream_t st);

@@ -15,12 +15,13 @@
 #include "band.cuh"
 #include "gsofa.h"
 #include "internal.cuh"
+#include "route.cuh"
 
 namespace gsofa {
 namespace {
 
 static_assert(GSOFA_NOALLOC_SCRATCH_BYTES >= 4096, "scratch too small");
-static_assert(sizeof(BandCounters) <= 64, "counters of the banded path");
+static_assert(sizeof(BandCounters) <= 64 && sizeof(BandReach) == 16, "counters of the banded path");
 static_assert(sizeof(DevCounters) <= 256, "the counters block must fit ahead of the overflow lists");
 
 // Scratch of this entry point: [0, 256) counters, then frontier overflow lists.
@@ -82,7 +83,8 @@ extern "C" int gsofa_row_counts_noalloc(int32_t n, const int32_t* d_rowptr, cons
     unsigned char* p = (unsigned char*)base;
     const size_t cross_bytes = 4 * ((size_t)n / 1024 + 2);
     b.ctr = (BandCounters*)p;
-    b.band = (int32_t*)(p + 64);
+    b.reach = (BandReach*)(p + 64);
+    b.band = (int32_t*)(p + 80);
     b.cross = (uint32_t*)(p + 128);
     b.nmats = 1;
     b.one.rowptr = d_rowptr;
@@ -94,7 +96,11 @@ extern "C" int gsofa_row_counts_noalloc(int32_t n, const int32_t* d_rowptr, cons
     b.row_nU = d_nnzU;
     if (cudaMemsetAsync(p, 0, 128 + cross_bytes, st) != cudaSuccess) return GSOFA_E_CUDA;
     if (launch_band_scan(b, st) != cudaSuccess) return GSOFA_E_CUDA;
-    struct { BandCounters c; unsigned char pad[64 - sizeof(BandCounters)]; int32_t band[2]; } m;
+    b.sampled = n >= REACH_MIN_ORDER ? 1 : 0;
+    b.reach_rows = reach_rows(1);
+    b.most_rows = n;
+    if (launch_band_reach(b, true, st) != cudaSuccess) return GSOFA_E_CUDA;
+    struct { BandCounters c; unsigned char pad[64 - sizeof(BandCounters)]; BandReach reach; int32_t band[2]; } m;
     if (cudaMemcpyAsync(&m, p, sizeof(m), cudaMemcpyDeviceToHost, st) != cudaSuccess) return GSOFA_E_CUDA;
     rc = wait_stream(st);
     if (rc) return rc;
@@ -102,13 +108,12 @@ extern "C" int gsofa_row_counts_noalloc(int32_t n, const int32_t* d_rowptr, cons
     b.one.LB = band_words_left(m.band[0]);
     b.one.UB = band_words_right(m.band[1]);
     const BandShape s = band_shape(b.one.LB, b.one.UB, true);
-    // a wide band, which takes a cluster, pays from order 4,096 on (18 x 18 x 18 grid 845 us by
-    // traversal, 726 as a band; 12 x 12 x 12 with far entries 220 / 292; 18 x 18 x 9 322 / 352),
-    // and where most entries lie close to the diagonal, as in a dissection, up to 1,600 (40 x
-    // 40 348 / 290, 47 x 47 435 / 465)
-    const unsigned long long width = (unsigned long long)(m.band[0] > m.band[1] ? m.band[0] : m.band[1]);
-    const bool near = m.c.spread < m.c.nnz * width / 16;
-    const bool traverse = s.C == 0 || (b.one.LB > 8 && (near ? n > 1600 : n < 4096));
+    bool traverse = s.C == 0;
+    if (!traverse && b.one.LB > COUNTS_WIDE_BAND)
+      traverse = near_diagonal(m.c, m.band) ? n > NEAR_BAND_ORDER : n < WIDE_MIN_ORDER;
+    if (!traverse && b.sampled && m.reach.levels)
+      traverse = ROUTE_MARGIN * traverse_us(n, m.reach, b.reach_rows, true) <
+                 band_us(n, chain_panels(n, m.c.stretch, sms / s.C), b.one.LB, b.one.UB, true);
     if (!traverse) {
       const int panels = (n + 31) / 32, most = sms / s.C;
       if (launch_band_elim(b, panels < most ? panels : most, s.C, s.threads, s.smem, st) != cudaSuccess)

@@ -17,6 +17,7 @@
 
 // ---------------------------------------------------------------- what a scenario sets
 static int g_band_left = 0, g_band_right = 0;      // what the scan measures, for every matrix
+static long long g_reach = 1000000;                // entries that a sampled row reaches
 static int g_blocks = 0;                           // a dissection: it falls into closed blocks
 static int g_fail_count = 0, g_fail_at = -1;       // the g_fail_at-th pool allocation from now on fails
 static std::map<void*, size_t> g_held;             // pool memory: bytes by block
@@ -151,6 +152,14 @@ cudaError_t launch_band_scan(const BandArgs& a, cudaStream_t) {
   a.ctr->spread = a.ctr->nnz * (unsigned long long)(g_band_left > g_band_right ? g_band_left : g_band_right) / 2;
   return cudaSuccess;
 }
+cudaError_t launch_band_reach(const BandArgs& a, bool, cudaStream_t) {
+  for (int m = 0; m < a.sampled; m++) {
+    a.reach[m].entries = (unsigned long long)(g_reach * a.reach_rows);
+    a.reach[m].levels = 5u * (uint32_t)a.reach_rows;
+  }
+  a.ctr->stretch = (a.one.n + 31) / 32;
+  return cudaSuccess;
+}
 cudaError_t launch_band_elim(const BandArgs& a, int count, int C, int, size_t, cudaStream_t) {
   const BandMat& d = a.mats ? a.mats[a.first] : a.one;
   std::printf("band_elim %d %d left %d right %d\n", count, C, d.LB, d.UB);
@@ -200,6 +209,7 @@ int main(int argc, char** argv) {
   g_band_right = (int)get("right", 0);
   g_fail_at = (int)get("fail_at", -1);
   g_blocks = (int)get("blocks", 0);
+  g_reach = get("reach", 1000000);
   gsofa_options o;
   gsofa_default_options(&o);
   o.max_ctas = (int32_t)get("max_ctas", 0);

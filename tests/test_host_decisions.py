@@ -107,3 +107,33 @@ def test_budget_of_blocks(decide, budget):
         assert budget == 0 or max(held) <= budget // 2 + 5 * n  # besides counters and fill counts
     else:
         assert any(x.startswith("trav_class") for x in lines)
+
+
+@pytest.mark.parametrize("n,left,reach,traversed", [
+    (30000, 1000, 20, True), (30000, 1000, 2000, True), (30000, 1000, 100000, False), (30000, 100, 20, True),
+    (30000, 100, 30000, False), (40000, 30, 20, True), (40000, 30, 30000, False), (2047, 1000, 20, False)])
+def test_route_by_reach(decide, n, left, reach, traversed):
+    """A band whose rows reach little is traversed; the same one with long searches is not."""
+    lines = decide(n=n, left=left, right=left, reach=reach)
+    assert "rc 0" in lines and bool(_elim(lines)) == (not traversed), lines
+
+
+@pytest.mark.parametrize("n,left,reach,traversed", [
+    (30000, 1000, 20, True), (30000, 1000, 1000000, False), (10000, 100, 20, True), (10000, 100, 100000, False),
+    (2047, 200, 20, False)])
+def test_route_of_counts_by_reach(decide, n, left, reach, traversed):
+    lines = decide(n=n, left=left, right=left, reach=reach, counts=1)
+    assert "rc 0" in lines and bool(_elim(lines)) == (not traversed), lines
+
+
+def test_no_search_for_blocks_of_short_traversals(decide):
+    lines = decide(n=20000, left=15000, right=15000, blocks=1, reach=20)
+    assert "front_blocks" not in lines and any(x.startswith("trav_class") for x in lines), lines
+    assert "front_blocks" in decide(n=20000, left=15000, right=15000, blocks=1, reach=20000)
+
+
+@pytest.mark.parametrize("count,traversed", [(2, 2), (20, 20), (120, 0)])
+def test_batch_route_by_reach(decide, count, traversed):
+    """In a batch only bands that outlast the others are traversed."""
+    lines = decide(n=30000, left=200, right=200, reach=20, count=count)
+    assert "rc 0" in lines and sum(k for k, _, _, _ in _elim(lines)) == count - traversed, lines
