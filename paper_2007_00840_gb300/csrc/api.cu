@@ -619,9 +619,19 @@ struct BandRun {
 
 static_assert(sizeof(BandCounters) <= 64 && sizeof(BandReach) == 16, "the layout of BandRun::ctr");
 
-// Lay out the matrices, check them and measure their bands and the reach of the first
-// `sampled` of them (one wait).
-int band_measure(BandRun& b, const gsofa_options& o, int32_t sampled) {
+// The reach of the first `sampled` matrices of a scanned run, of order most_rows at most.
+int launch_reach(BandRun& b, int32_t sampled, int32_t most_rows) {
+  BandArgs& a = b.a;
+  a.sampled = sampled;
+  a.reach_rows = reach_rows(sampled);
+  a.most_rows = most_rows;
+  if (launch_band_reach(a, false, b.st) != cudaSuccess) return GSOFA_E_CUDA;
+  b.launches++;
+  return GSOFA_OK;
+}
+
+// Lay out the matrices, check them and measure their bands (one wait).
+int band_measure(BandRun& b, const gsofa_options& o) {
   Ctx* c = b.c;
   cudaStream_t st = b.st;
   const size_t B = b.mats.size();
@@ -666,19 +676,25 @@ int band_measure(BandRun& b, const gsofa_options& o, int32_t sampled) {
   a.band = (int32_t*)(b.ctr + 64 + 16 * B);
   a.mat_tot = B > 1 ? (unsigned long long*)(b.ctr + 64 + 24 * B) : nullptr;
   a.mat_nsuper = (int32_t*)(b.ctr + 64 + 40 * B);
-  a.sampled = sampled;
-  a.reach_rows = reach_rows(sampled);
-  a.most_rows = b.mats[0].n;  // (a batch is sampled largest first)
   a.cross = cross_words ? (uint32_t*)(b.ctr + ((b.host_bytes + 15) & ~(size_t)15)) : nullptr;
   a.fill = b.fill;
   if (launch_band_scan(a, st) != cudaSuccess) return GSOFA_E_CUDA;
   b.launches++;
-  if (sampled > 0) {
-    if (launch_band_reach(a, false, st) != cudaSuccess) return GSOFA_E_CUDA;
-    b.launches++;
+  if (B == 1 && reach_at_once(b.mats[0].n, false)) {
+    const int rc = launch_reach(b, 1, b.mats[0].n);
+    if (rc) return rc;
   }
   if (cudaMemcpyAsync(b.hctr, b.ctr, 64 + 24 * B, cudaMemcpyDeviceToHost, st) != cudaSuccess) return GSOFA_E_CUDA;
   return wait_stream(st);
+}
+
+// The same after band_measure (one more wait).
+int band_reach(BandRun& b, int32_t sampled, int32_t most_rows) {
+  const int rc = launch_reach(b, sampled, most_rows);
+  if (rc) return rc;
+  if (cudaMemcpyAsync(b.hctr, b.ctr, 64 + 16 * (size_t)sampled, cudaMemcpyDeviceToHost, b.st) != cudaSuccess)
+    return GSOFA_E_CUDA;
+  return wait_stream(b.st);
 }
 
 // Bitmap words of all matrices once their bands are known; -1 where one does not fit on chip.
@@ -1193,7 +1209,7 @@ int run_band_single(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, con
   m.n = n;
   b.mats.push_back(m);
   b.share = cta_share(c, o);
-  int rc = band_measure(b, o, n >= REACH_MIN_ORDER ? 1 : 0);
+  int rc = band_measure(b, o);
   ev.rec(1, st);
   int64_t words = -1;
   bool near = false, blocks = false;
@@ -1210,7 +1226,10 @@ int run_band_single(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, con
       if (words >= 0 && m.LB > WIDE_BAND && (near ? n > NEAR_BAND_ORDER : n >= WIDE_MIN_ORDER && h.nnz < WIDE_NNZ))
         words = -1;
       blocks = n >= (near ? FRONT_NEAR_ORDER : FRONT_MIN_ORDER);
-      if (b.a.sampled && b.h_reach(0).levels) {
+      const float band = words >= 0 ? band_us(n, (n + 31) / 32, m.LB, m.UB, false) : 0.f;
+      if (b.a.sampled == 0 && (words >= 0 || (blocks && !surely_blocks(n, h, near))) && reach_limit_us(n, band, false) > 0.f)
+        rc = band_reach(b, 1, n);
+      if (rc == GSOFA_OK && b.h_reach(0).levels) {
         const float traverse = traverse_us(n, b.h_reach(0), b.a.reach_rows, false);
         if (words >= 0) {
           const int C = band_shape(m.LB, m.UB, true, b.share).C;
@@ -1223,7 +1242,7 @@ int run_band_single(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, con
           blocks = blocks && traverse > fronts_limit_us(n);
         }
       }
-      if (words >= 0) rc = band_run(b, words, ev);
+      if (rc == GSOFA_OK && words >= 0) rc = band_run(b, words, ev);
     }
   }
   if (rc == GSOFA_OK && words < 0 && blocks) {
@@ -1315,9 +1334,7 @@ int run_band_batch(Ctx* c, const std::vector<int32_t>& idx, const int32_t* n, co
       b.mats.push_back(m);
     }
     ev.rec(0, st);
-    int32_t sampled = 0;  // once, the largest
-    while (pass == 0 && sampled < (int32_t)order.size() && n[order[sampled]] >= REACH_MIN_ORDER) sampled++;
-    int rc = band_measure(b, o, sampled);
+    int rc = band_measure(b, o);
     ev.rec(1, st);
     int64_t words = -1;
     if (rc == GSOFA_OK && b.counters()->err) rc = GSOFA_E_INVAL;
@@ -1334,27 +1351,36 @@ int run_band_batch(Ctx* c, const std::vector<int32_t>& idx, const int32_t* n, co
         chain[m] = band_us(n[order[m]], (n[order[m]] + 31) / 32, LB, UB, false);
         all += chain[m] * (float)size[m];
       }
+      // bands that outlast the others: those that the traversal would have done sooner go there
+      auto longest = [&](size_t m) {
+        return pass == 0 && size[m] && chain[m] > 2.f * all / (float)c->sms &&
+               reach_limit_us(n[order[m]], chain[m], false) > 0.f;
+      };
+      int32_t sampled = 0;
+      for (size_t m = 0; m < order.size(); m++)
+        if (longest(m)) sampled = (int32_t)m + 1;
+      if (sampled > 0 && b.a.sampled == 0) rc = band_reach(b, sampled, n[order[0]]);
+      if (rc == GSOFA_OK)
+        for (int32_t m = 0; m < sampled && m < b.a.sampled; m++)
+          if (longest(m) && b.h_reach(m).levels &&
+              ROUTE_MARGIN * traverse_us(n[order[m]], b.h_reach(m), b.a.reach_rows, false) < chain[m])
+            size[m] = 0;
       for (size_t m = 0; m < order.size(); m++) {
-        // a band that outlasts the others and that the traversal would have done sooner
-        if ((int32_t)m < sampled && size[m] && chain[m] > 2.f * all / (float)c->sms &&
-            b.h_reach(m).levels &&
-            ROUTE_MARGIN * traverse_us(n[order[m]], b.h_reach(m), b.a.reach_rows, false) < chain[m])
-          size[m] = 0;
         if (size[m] == 0) rest->push_back(order[m]);
         if (size[m] == 0 || (m && size[m] < size[m - 1])) sorted = false;
       }
       for (int C = 1; C <= 8; C *= 2)
         for (size_t m = 0; m < order.size(); m++)
           if (size[m] == C) next.push_back(order[m]);
-      if (!sorted) {  // lay the batch out again without them, in launch order
+      if (rc == GSOFA_OK && !sorted) {  // lay the batch out again without them, in launch order
         b.free_scratch();
         b.free_results();
         *launches += b.launches;
         order.swap(next);
         continue;
       }
-      words = band_layout(b);
-      rc = words < 0 ? GSOFA_E_CUDA : band_run(b, words, ev);
+      if (rc == GSOFA_OK) words = band_layout(b);
+      if (rc == GSOFA_OK) rc = words < 0 ? GSOFA_E_CUDA : band_run(b, words, ev);
     }
     b.free_scratch();
     *launches += b.launches;

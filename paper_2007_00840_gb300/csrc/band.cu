@@ -223,17 +223,18 @@ __global__ void __launch_bounds__(256) band_scan_kernel(BandArgs a) {
 // that does not repeat with its structure): breadth-first search from s over vertices below
 // s, level by level, a thread (or eight) per vertex, vertices found marked in a bitmap.
 // Cut off after what the choice of the route can still use.  Bound by the latency of a
-// level: row pointers, columns, bitmap, a barrier, 1.3 us or more.  Takes 14 us beside the
-// 340 of a 64 x 64 grid, where it is left out, 45 on a band of 211 (1,290), 90 on 32^3
-// (4,690), 150 on 317 x 293 (7,360).  The last CTA finds the longest stretch of one matrix.
+// level: row pointers, columns, bitmap, a barrier, 1.3 us or more.  Calls that stay with the
+// elimination take 40 us more on a band of 211 (1,274 before), 100 on 317 x 293 (7,325); 32^3 and
+// dissections differ by less than their runs do.  The last CTA finds the longest stretch of
+// one matrix.
 namespace {
-constexpr int REACH_THREADS = 512;
-constexpr int REACH_QUEUE = 1024;   // vertices of a level
+constexpr int REACH_THREADS = 256;
+constexpr int REACH_QUEUE = 256;    // vertices of a level: wider searches are long (a band of 211: 20 us against 45 with 1,024)
 constexpr int REACH_WORDS = 49152;  // of the bitmap at most: a search that goes further back is cut off
 // Words of the bitmap for orders up to n (a multiple of four; room for the stretches' sums).
 int reach_words(int n) {
   const int w = ((n - 1) / 32 + 4) & ~3;
-  return w > REACH_WORDS ? REACH_WORDS : (w < 3 * REACH_THREADS ? 3 * REACH_THREADS : w);
+  return w > REACH_WORDS ? REACH_WORDS : w < 3 * REACH_THREADS ? 3 * REACH_THREADS : w;
 }
 }  // namespace
 __global__ void __launch_bounds__(REACH_THREADS) band_reach_kernel(BandArgs a, bool counts, int words) {
@@ -285,7 +286,11 @@ __global__ void __launch_bounds__(REACH_THREADS) band_reach_kernel(BandArgs a, b
   for (int i = tid; i < words / 4; i += REACH_THREADS) ((uint4*)seen)[i] = make_uint4(0u, 0u, 0u, 0u);
   if (err) return;  // nothing is followed unchecked
   const bool fits = band_shape(LB, UB, false).C > 0;
-  if (!fits && a.mats) return;
+  if (!fits) {
+    if (a.mats || counts) return;
+    const bool near = near_diagonal(*a.ctr, a.band);
+    if (n < (near ? FRONT_NEAR_ORDER : FRONT_MIN_ORDER) || surely_blocks(n, *a.ctr, near)) return;
+  }
   // the panels in a chain: where there are stretches, about four of the mean length
   int chain = panels;
   if (a.cross) {
@@ -320,6 +325,7 @@ __global__ void __launch_bounds__(REACH_THREADS) band_reach_kernel(BandArgs a, b
     queue[0] = s;
     level[1] = {0, 0, 0u};
   }
+  const unsigned long long decided = (unsigned long long)(1.2f * row_ns / cost.entry * (float)a.reach_rows);
   uint32_t all = 0u;
   int levels = 0, count = 1;
   bool cut = false;
@@ -328,7 +334,11 @@ __global__ void __launch_bounds__(REACH_THREADS) band_reach_kernel(BandArgs a, b
     const int32_t* in = queue + REACH_QUEUE * (levels & 1);
     int32_t* out = queue + REACH_QUEUE * ((levels & 1) ^ 1);
     auto& next = level[(levels + 1) % 3];
-    if (tid == 0) level[(levels + 2) % 3] = {0, 0, 0u};
+    if (tid == 0) {
+      level[(levels + 2) % 3] = {0, 0, 0u};
+      // the other rows may have decided already
+      if ((levels & 3) == 3 && *(volatile unsigned long long*)&a.reach[m].entries > decided) next.cut = 1;
+    }
     uint32_t entries = 0u;
     for (int i0 = 0; i0 < count; i0 += REACH_THREADS / lanes) {
       const int i = i0 + tid / lanes;

@@ -96,9 +96,9 @@ extern "C" int gsofa_row_counts_noalloc(int32_t n, const int32_t* d_rowptr, cons
     b.row_nU = d_nnzU;
     if (cudaMemsetAsync(p, 0, 128 + cross_bytes, st) != cudaSuccess) return GSOFA_E_CUDA;
     if (launch_band_scan(b, st) != cudaSuccess) return GSOFA_E_CUDA;
-    b.sampled = n >= REACH_MIN_ORDER ? 1 : 0;
     b.reach_rows = reach_rows(1);
     b.most_rows = n;
+    b.sampled = reach_at_once(n, true) ? 1 : 0;
     if (launch_band_reach(b, true, st) != cudaSuccess) return GSOFA_E_CUDA;
     struct { BandCounters c; unsigned char pad[64 - sizeof(BandCounters)]; BandReach reach; int32_t band[2]; } m;
     if (cudaMemcpyAsync(&m, p, sizeof(m), cudaMemcpyDeviceToHost, st) != cudaSuccess) return GSOFA_E_CUDA;
@@ -111,7 +111,14 @@ extern "C" int gsofa_row_counts_noalloc(int32_t n, const int32_t* d_rowptr, cons
     bool traverse = s.C == 0;
     if (!traverse && b.one.LB > COUNTS_WIDE_BAND)
       traverse = near_diagonal(m.c, m.band) ? n > NEAR_BAND_ORDER : n < WIDE_MIN_ORDER;
-    if (!traverse && b.sampled && m.reach.levels)
+    if (!traverse && !b.sampled && reach_limit_us(n, band_us(n, (n + 31) / 32, b.one.LB, b.one.UB, true), true) > 0.f) {
+      b.sampled = 1;
+      if (launch_band_reach(b, true, st) != cudaSuccess) return GSOFA_E_CUDA;
+      if (cudaMemcpyAsync(&m, p, sizeof(m), cudaMemcpyDeviceToHost, st) != cudaSuccess) return GSOFA_E_CUDA;
+      rc = wait_stream(st);
+      if (rc) return rc;
+    }
+    if (!traverse && m.reach.levels)
       traverse = ROUTE_MARGIN * traverse_us(n, m.reach, b.reach_rows, true) <
                  band_us(n, chain_panels(n, m.c.stretch, sms / s.C), b.one.LB, b.one.UB, true);
     if (!traverse) {

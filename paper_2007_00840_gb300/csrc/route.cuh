@@ -23,7 +23,6 @@ namespace gsofa {
 constexpr int32_t FRONT_MIN_ORDER = 16384;
 constexpr int32_t FRONT_NEAR_ORDER = 2600;
 
-constexpr int REACH_MIN_ORDER = 2048;  // smaller orders are not sampled: a band takes 100 us there
 constexpr int REACH_ROWS = 128;        // rows sampled of one matrix
 constexpr int REACH_ROWS_MIN = 4;      // and at least of each matrix of a batch (about two per SM in all)
 
@@ -83,6 +82,13 @@ __host__ __device__ inline float reach_limit_us(int n, float band, bool counts) 
   return band < 1.6f * ROUTE_MARGIN * base ? 0.f : band / ROUTE_MARGIN - base;
 }
 
+// Orders whose narrowest band is sampled (from 4,900 on, counts 800): the search is launched with
+// the scan.  Below, the scan is waited for first (25 us more, where the band is wide; 10 us
+// less where it is not sampled).
+inline bool reach_at_once(int n, bool counts) {
+  return reach_limit_us(n, band_us(n, (n + 31) / 32, 1, 0, counts), counts) > 0.f;
+}
+
 // A traversal, from the sums over `rows` sampled rows (r.levels is 0 where none were).
 inline float traverse_us(int n, const BandReach& r, int rows, bool counts) {
   const TraverseCost t = traverse_cost(n, counts);
@@ -114,10 +120,16 @@ constexpr int32_t WIDE_MIN_ORDER = 4096;
 // diagonal, as in a dissection, up to 1,600 (40 x 40 348 / 290, 47 x 47 435 / 465).
 constexpr int32_t COUNTS_WIDE_BAND = 8;
 
+// A dissection with an entry per row beside the diagonal has long rows: blocks are looked for
+// without a sample.
+__host__ __device__ inline bool surely_blocks(int n, const BandCounters& h, bool near) {
+  return near && h.nnz >= 2ull * (unsigned long long)n;
+}
+
 // Most entries lie close to the diagonal and few far out, as in a dissection (mean distance
 // 0.04 of the band or less; bands and natural grids have 0.2 or more, with one far entry
 // per row 0.09).
-inline bool near_diagonal(const BandCounters& h, const int32_t* band) {
+__host__ __device__ inline bool near_diagonal(const BandCounters& h, const int32_t* band) {
   const int32_t width = band[0] > band[1] ? band[0] : band[1];
   return h.spread < h.nnz * (unsigned long long)width / 16;
 }

@@ -47,7 +47,7 @@ CASES = [
     (lambda: synth.grid2d(128, 0.8, seed=8), False),
     (lambda: synth.banded(15013, 211, seed=9), False),
     (lambda: synth.grid2d_nd(150, 0.8, seed=10), False),
-    (lambda: _random(2048, 0.45, 1500, 11), None),
+    (lambda: _random(2048, 0.45, 1500, 11), True),
 ]
 
 

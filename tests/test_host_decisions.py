@@ -111,7 +111,7 @@ def test_budget_of_blocks(decide, budget):
 
 @pytest.mark.parametrize("n,left,reach,traversed", [
     (30000, 1000, 20, True), (30000, 1000, 2000, True), (30000, 1000, 100000, False), (30000, 100, 20, True),
-    (30000, 100, 30000, False), (40000, 30, 20, True), (40000, 30, 30000, False), (2047, 1000, 20, False)])
+    (30000, 100, 30000, False), (40000, 30, 20, True), (40000, 30, 30000, False), (2047, 1000, 20, True), (900, 300, 20, False)])
 def test_route_by_reach(decide, n, left, reach, traversed):
     """A band whose rows reach little is traversed; the same one with long searches is not."""
     lines = decide(n=n, left=left, right=left, reach=reach)
@@ -120,7 +120,7 @@ def test_route_by_reach(decide, n, left, reach, traversed):
 
 @pytest.mark.parametrize("n,left,reach,traversed", [
     (30000, 1000, 20, True), (30000, 1000, 1000000, False), (10000, 100, 20, True), (10000, 100, 100000, False),
-    (2047, 200, 20, False)])
+    (2047, 200, 20, True), (300, 60, 20, False)])
 def test_route_of_counts_by_reach(decide, n, left, reach, traversed):
     lines = decide(n=n, left=left, right=left, reach=reach, counts=1)
     assert "rc 0" in lines and bool(_elim(lines)) == (not traversed), lines
