@@ -128,6 +128,10 @@ double timeout_seconds() {
   return 600.0;
 }
 
+// Waits of this thread that ran out.  Work that was not waited for may still read and write
+// the thread's pinned buffers, so calls after that take new ones and leave those alone.
+thread_local int t_abandoned = 0;
+
 }  // namespace
 
 // Bounded wait for all work queued on `st` (never an unbounded block).
@@ -140,7 +144,10 @@ int wait_stream(cudaStream_t st) {
     if (e == cudaSuccess) return GSOFA_OK;
     if (e != cudaErrorNotReady) return GSOFA_E_CUDA;
     const double el = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
-    if (el > limit) return GSOFA_E_TIMEOUT;
+    if (el > limit) {
+      t_abandoned++;
+      return GSOFA_E_TIMEOUT;
+    }
     if (++spins > 2000) std::this_thread::sleep_for(std::chrono::microseconds(50));
   }
 }
@@ -363,7 +370,9 @@ int ensure_slots(Ctx* c, int64_t cap, int slots, cudaStream_t st) {
 
 DevCounters* pinned_counters() {
   thread_local DevCounters* h = nullptr;
-  if (!h) {
+  thread_local int seen = 0;
+  if (!h || seen != t_abandoned) {
+    seen = t_abandoned;
     if (cudaMallocHost(&h, sizeof(DevCounters)) != cudaSuccess) h = nullptr;
   }
   return h;
@@ -555,6 +564,12 @@ int check_options(const gsofa_options* in, gsofa_options* o) {
 void* thread_pinned(size_t bytes, int slot) {
   thread_local void* buf[2] = {nullptr, nullptr};
   thread_local size_t cap[2] = {0, 0};
+  thread_local int seen = 0;
+  if (seen != t_abandoned) {
+    seen = t_abandoned;
+    buf[0] = buf[1] = nullptr;
+    cap[0] = cap[1] = 0;
+  }
   if (cap[slot] < bytes) {
     if (buf[slot]) cudaFreeHost(buf[slot]);
     buf[slot] = nullptr;

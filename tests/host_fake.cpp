@@ -8,6 +8,7 @@
 #include <cstring>
 #include <map>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "band.cuh"
@@ -22,6 +23,16 @@ static int g_blocks = 0;                           // a dissection: it falls int
 static int g_fail_count = 0, g_fail_at = -1;       // the g_fail_at-th pool allocation from now on fails
 static std::map<void*, size_t> g_held;             // pool memory: bytes by block
 static size_t g_now = 0, g_peak = 0;
+static int g_stuck = 0;                            // streams that never finish
+static std::vector<std::pair<const char*, size_t>> g_pinned_blocks, g_in_flight;  // pinned memory; what copies of a stuck stream use
+static void copied(const void* host, size_t n) {
+  for (auto& b : g_pinned_blocks) {
+    if ((const char*)host < b.first || (const char*)host >= b.first + b.second) continue;
+    for (auto& f : g_in_flight)
+      if (f.first < (const char*)host + n && (const char*)host < f.first + f.second && !g_stuck) std::puts("in flight");
+    if (g_stuck) g_in_flight.push_back({(const char*)host, n});
+  }
+}
 
 // ---------------------------------------------------------------- CUDA runtime
 extern "C" {
@@ -61,17 +72,22 @@ cudaError_t cudaMalloc(void** p, size_t n) {
   return *p ? cudaSuccess : cudaErrorMemoryAllocation;
 }
 cudaError_t cudaFree(void* p) { std::free(p); return cudaSuccess; }
-cudaError_t cudaMallocHost(void** p, size_t n) { return cudaMalloc(p, n); }
+cudaError_t cudaMallocHost(void** p, size_t n) {
+  const cudaError_t e = cudaMalloc(p, n);
+  if (*p) g_pinned_blocks.push_back({(const char*)*p, n});
+  return e;
+}
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return cudaMalloc(p, n); }
 cudaError_t cudaHostGetDevicePointer(void** d, void* h, unsigned) { *d = h; return cudaSuccess; }
 cudaError_t cudaFreeHost(void* p) { std::free(p); return cudaSuccess; }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { std::memcpy(d, s, n); return cudaSuccess; }
-cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind k, cudaStream_t) {
+  copied(k == cudaMemcpyDeviceToHost ? d : s, n);
   std::memcpy(d, s, n);
   return cudaSuccess;
 }
 cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t) { std::memset(d, v, n); return cudaSuccess; }
-cudaError_t cudaStreamQuery(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamQuery(cudaStream_t) { return g_stuck ? cudaErrorNotReady : cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = (cudaStream_t)1; return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
@@ -217,15 +233,24 @@ int main(int argc, char** argv) {
   std::vector<int32_t> rp((size_t)(get("rows", n) + 1), 0), ci(1, 0);
   std::vector<gsofa_result> out(count);
   int rc;
+  auto call = [&] {
+    if (count > 1) {
+      std::vector<int32_t> ns(count, n);
+      std::vector<const int32_t*> rps(count, rp.data()), cis(count, ci.data());
+      return gsofa_batch(count, ns.data(), rps.data(), cis.data(), &o, nullptr, out.data());
+    }
+    return gsofa_symbolic_device(n, rp.data(), ci.data(), &o, nullptr, &out[0]);
+  };
+  if (get("stuck", 0)) {  // a call whose wait runs out before the one that is looked at
+    g_stuck = 1;
+    std::printf("first rc %d\n", call());
+    g_stuck = 0;
+  }
   if (get("counts", 0)) {
     std::vector<int32_t> a(n), b(n), c(n);
     rc = gsofa_row_counts_noalloc(n, rp.data(), ci.data(), a.data(), b.data(), c.data(), nullptr);
-  } else if (count > 1) {
-    std::vector<int32_t> ns(count, n);
-    std::vector<const int32_t*> rps(count, rp.data()), cis(count, ci.data());
-    rc = gsofa_batch(count, ns.data(), rps.data(), cis.data(), &o, nullptr, out.data());
   } else {
-    rc = gsofa_symbolic_device(n, rp.data(), ci.data(), &o, nullptr, &out[0]);
+    rc = call();
   }
   std::printf("rc %d\n", rc);
   if (rc == GSOFA_OK && !get("counts", 0))

@@ -26,7 +26,8 @@ def decide(tmp_path_factory):
     exe = _program(str(tmp_path_factory.mktemp("host")))
 
     def run(**kw):
-        out = subprocess.run([exe] + [f"{k}={v}" for k, v in kw.items()], capture_output=True, text=True, timeout=60)
+        env = dict(os.environ, GSOFA_TIMEOUT_S="0.001") if kw.get("stuck") else None
+        out = subprocess.run([exe] + [f"{k}={v}" for k, v in kw.items()], capture_output=True, text=True, timeout=60, env=env)
         assert out.returncode == 0, out.stderr
         return out.stdout.splitlines()
     return run
@@ -137,3 +138,11 @@ def test_batch_route_by_reach(decide, count, traversed):
     """In a batch only bands that outlast the others are traversed."""
     lines = decide(n=30000, left=200, right=200, reach=20, count=count)
     assert "rc 0" in lines and sum(k for k, _, _, _ in _elim(lines)) == count - traversed, lines
+
+
+@pytest.mark.parametrize("kw", [dict(left=40), dict(left=40, count=5), dict(left=15000, blocks=1), dict(left=15000)])
+def test_buffers_of_abandoned_work_are_left_alone(decide, kw):
+    """After a wait that ran out, the next call of the thread uses other pinned buffers: the copies
+    of the first may still be under way."""
+    lines = decide(n=20000, right=kw["left"], stuck=1, **kw)
+    assert "first rc -5" in lines and "rc 0" in lines and "in flight" not in lines, lines
