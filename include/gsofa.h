@@ -86,7 +86,9 @@ typedef struct gsofa_options {
                                     or a dissection in as many launches as that takes); a band or block
                                     that needs a larger cluster of CTAs is traversed */
     int32_t frontier_order;      /* 0: automatic: elimination on chip where the pattern is banded or a
-                                    nested dissection (of order 2,600 or more) and every option that
+                                    nested dissection (of order 2,600 or more; in a batch only above the
+                                    orders that are traversed together), a sample of its rows does not
+                                    reach so little that a traversal is faster, and every option that
                                     concerns the traversal alone has its default; else class order for every
                                     source (sources below an explicit smem_max_source stay breadth-first
                                     in shared memory); with autotune = 1 both orders are timed once per
@@ -193,18 +195,21 @@ int gsofa_symbolic_device(int32_t n, const int32_t *d_rowptr, const int32_t *d_c
                           const gsofa_options *opt, void *stream, gsofa_result *out);
 
 /*
- * gsofa_batch - many independent matrices in one pass: the Section 4 traversal
- * and Section 5 supernode detection of every matrix, with the source rows of
- * all matrices scheduled together.  Matrix k is (n[k], d_rowptr[k],
- * d_colidx[k]) on the current device (borrowed).  Matrices whose maxId arrays
- * fit in shared memory run in ONE persistent traversal launch whose work items
- * are (matrix, source row) pairs, largest source row first across the batch;
- * the launch sequence up to the size read-back is captured once per batch
- * signature (matrix count, orders, input pointers, options) into a CUDA graph
- * and replayed on later calls with the same signature.  Larger matrices run
- * one after another through the single-matrix path.  outs[k] receives matrix
- * k's device result; batch members share one allocation that is released when
- * the last of them is passed to gsofa_free().  On error every out is zeroed.
+ * gsofa_batch - many independent matrices in one pass.  Matrix k is (n[k],
+ * d_rowptr[k], d_colidx[k]) on the current device (borrowed).  With options that
+ * leave the route to the library, one scan checks all matrices and measures their
+ * bands; those whose band fits on chip are eliminated together, one launch per
+ * cluster size, unless a band would outlast the others and a traversal is faster.
+ * The others whose maxId arrays fit in shared memory (orders up to 65,533) run in
+ * ONE persistent traversal launch (Sections 4 and 5) whose work items are
+ * (matrix, source row) pairs, largest source row first across the batch; the
+ * launch sequence up to the size read-back is captured once per signature of
+ * these matrices (positions, orders, input pointers, options) into a CUDA graph
+ * and replayed on later calls with the same signature.  Larger matrices run one
+ * after another through the single-matrix path (a dissection: by its blocks).
+ * outs[k] receives matrix k's device result; the eliminated members share one
+ * allocation, the traversed ones another, each released when the last of them is
+ * passed to gsofa_free().  On error every out is zeroed.
  */
 int gsofa_batch(int32_t count, const int32_t *n, const int32_t *const *d_rowptr,
                 const int32_t *const *d_colidx, const gsofa_options *opt, void *stream,

@@ -19,7 +19,7 @@
 //      holds q.  The few rows left (one in a dense band, about eight on a 2D grid) are
 //      combined in tables of 16 for every four of them, so that a word of a row costs one
 //      load per four panel rows.
-// The chain from one block to the next sets the pace: one warp finds the next panel's
+// The chain from one block to the next cannot be shortened by more warps: one finds the next panel's
 // block (panel P applied to that one word of its rows) and factors it while the other
 // warps do B and C of panel P for all words.
 // One CTA takes one matrix; wide bands are split over a cluster of up to eight (row
@@ -791,11 +791,14 @@ __device__ __forceinline__ void step_below(const Band& B, const PanelBufs& S, in
 
 }  // namespace
 
-// Bound by the latency of the chain, one panel after the other (shared-memory loads, 31
-// dependent shuffles to close the block, two barriers, cluster-wide with more than one CTA):
-// per panel of 32 rows 1.5 us on a 64 x 64 grid, 2.2 at band 211, 2.4 at 317 (cluster of
-// 4), 4.2 at 1,024 (of 8).  Elimination against the traversal: 32^3 grid 8.7 -> 4.3 ms,
-// 317 x 293 63 -> 7.0, band 211 of order 15,013 4.9 -> 1.05.
+// Bound by latency, one panel of 32 rows after the other: 1.5 us on a 64 x 64 grid, 2.2 at
+// band 211, 2.4 at 317 (cluster of 4), 4.3 at 1,024 (of 8).  With one CTA a narrow panel is the
+// chain (2,370 of about 3,200 cycles: closing the next rows, 31 dependent shuffles for their
+// first word, the factor), a wider one the workers' phases (band 211: 4,300 of 4,650, of which
+// C 1,330).  In a cluster the chain (2,320 to 2,630) is followed by B of the next panel and its
+// partnerless rows, stored to every CTA in turn: 1,800 and 3,300 cycles with four CTAs, 5,900
+// and 5,100 with eight, the larger part of the panel.  Elimination against the
+// traversal: 32^3 grid 8.7 -> 4.3 ms, 317 x 293 63 -> 7.0, band 211 of order 15,013 4.9 -> 1.05.
 // Warps of a CTA: 0 the chain, the last the loader (rows into the window), the others
 // workers (B, C and finished rows out).
 template <int C>

@@ -77,7 +77,6 @@ struct FrontEmit {
 
 cudaError_t launch_front_blocks(const FrontLevel& l, cudaStream_t st);   // low .. rem
 cudaError_t launch_front_above(const FrontLevel& l, cudaStream_t st);    // rows above, columns right of the blocks
-cudaError_t launch_front_bound(const FrontLevel& l, cudaStream_t st);
 // Rows of the next level: beg, end, col, gid of its n1 vertices.
 cudaError_t launch_front_reduce(const FrontLevel& l, int32_t n1, const FrontMat* fronts, const uint32_t* bits,
                                 int32_t* beg, int32_t* end, int32_t* col, int32_t* gid, cudaStream_t st);
