@@ -607,7 +607,7 @@ struct BandRun {
   BandArgs a;
   std::vector<BandMat> mats;
   int share = INT_MAX;  // cta_share
-  unsigned char* ctr = nullptr;   // BandCounters | reach | band | mat_tot | nsuper | cross: zeroed together
+  unsigned char* ctr = nullptr;   // BandCounters | reach | mat_tot | band | nsuper | entries | cross: zeroed together
   unsigned char* hctr = nullptr;  // pinned copy (all but cross)
   size_t ctr_bytes = 0, host_bytes = 0;
   BandMat* d_mats = nullptr;
@@ -620,9 +620,10 @@ struct BandRun {
 
   const BandCounters* counters() const { return (const BandCounters*)hctr; }
   const BandReach& h_reach(size_t m) const { return ((const BandReach*)(hctr + 64))[m]; }
-  int32_t* h_band() const { return (int32_t*)(hctr + 64 + 16 * mats.size()); }
-  unsigned long long* h_tot() const { return (unsigned long long*)(hctr + 64 + 24 * mats.size()); }
+  unsigned long long* h_tot() const { return (unsigned long long*)(hctr + 64 + 16 * mats.size()); }
+  int32_t* h_band() const { return (int32_t*)(hctr + 64 + 32 * mats.size()); }
   int32_t* h_nsuper() const { return (int32_t*)(hctr + 64 + 40 * mats.size()); }
+  int32_t h_entries(size_t m) const { return ((const int32_t*)(hctr + 64 + 44 * mats.size()))[m]; }
   void free_scratch() {
     pfree(ctr, st); pfree(d_mats, st); pfree(nL, st); pfree(nU, st); pfree(flags, st);
     pfree(part, st); pfree(bits, st);
@@ -668,7 +669,7 @@ int band_measure(BandRun& b, const gsofa_options& o) {
   a.rows = rows;
   a.groups = groups;
   const size_t cross_words = B == 1 ? (size_t)rows / 1024 + 2 : 0;
-  b.host_bytes = 64 + 44 * B;
+  b.host_bytes = 64 + 48 * B;
   b.ctr_bytes = ((b.host_bytes + 15) & ~(size_t)15) + 4 * cross_words;
   b.hctr = (unsigned char*)thread_pinned(b.host_bytes, 1);
   if (!b.hctr) return GSOFA_E_NOMEM;
@@ -688,18 +689,19 @@ int band_measure(BandRun& b, const gsofa_options& o) {
   }
   a.ctr = (BandCounters*)b.ctr;
   a.reach = (BandReach*)(b.ctr + 64);
-  a.band = (int32_t*)(b.ctr + 64 + 16 * B);
-  a.mat_tot = B > 1 ? (unsigned long long*)(b.ctr + 64 + 24 * B) : nullptr;
+  a.mat_tot = B > 1 ? (unsigned long long*)(b.ctr + 64 + 16 * B) : nullptr;
+  a.band = (int32_t*)(b.ctr + 64 + 32 * B);
   a.mat_nsuper = (int32_t*)(b.ctr + 64 + 40 * B);
+  a.entries = B > 1 ? (int32_t*)(b.ctr + 64 + 44 * B) : nullptr;
   a.cross = cross_words ? (uint32_t*)(b.ctr + ((b.host_bytes + 15) & ~(size_t)15)) : nullptr;
   a.fill = b.fill;
   if (launch_band_scan(a, st) != cudaSuccess) return GSOFA_E_CUDA;
   b.launches++;
-  if (B == 1 && reach_at_once(b.mats[0].n, false)) {
+  if (B == 1 && b.mats[0].n >= REACH_AT_ONCE) {
     const int rc = launch_reach(b, 1, b.mats[0].n);
     if (rc) return rc;
   }
-  if (cudaMemcpyAsync(b.hctr, b.ctr, 64 + 24 * B, cudaMemcpyDeviceToHost, st) != cudaSuccess) return GSOFA_E_CUDA;
+  if (cudaMemcpyAsync(b.hctr, b.ctr, b.host_bytes, cudaMemcpyDeviceToHost, st) != cudaSuccess) return GSOFA_E_CUDA;
   return wait_stream(st);
 }
 
@@ -1242,7 +1244,8 @@ int run_band_single(Ctx* c, int32_t n, const int32_t* rp, const int32_t* ci, con
         words = -1;
       blocks = n >= (near ? FRONT_NEAR_ORDER : FRONT_MIN_ORDER);
       const float band = words >= 0 ? band_us(n, (n + 31) / 32, m.LB, m.UB, false) : 0.f;
-      if (b.a.sampled == 0 && (words >= 0 || (blocks && !surely_blocks(n, h, near))) && reach_limit_us(n, band, false) > 0.f)
+      if (b.a.sampled == 0 && (words >= 0 || (blocks && !surely_blocks(n, h, near))) &&
+          reach_limit_us(n, h.nnz, band, false) > 0.f)
         rc = band_reach(b, 1, n);
       if (rc == GSOFA_OK && b.h_reach(0).levels) {
         const float traverse = traverse_us(n, b.h_reach(0), b.a.reach_rows, false);
@@ -1366,20 +1369,38 @@ int run_band_batch(Ctx* c, const std::vector<int32_t>& idx, const int32_t* n, co
         chain[m] = band_us(n[order[m]], (n[order[m]] + 31) / 32, LB, UB, false);
         all += chain[m] * (float)size[m];
       }
-      // bands that outlast the others: those that the traversal would have done sooner go there
+      // Bands that outlast the others and that the traversal would have done sooner go there, if
+      // the call gains by it: the longest chain left and the traversals come one after the other.
+      auto entries = [&](size_t m) {
+        return order.size() > 1 ? (unsigned long long)b.h_entries(m) : b.counters()->nnz;
+      };
       auto longest = [&](size_t m) {
         return pass == 0 && size[m] && chain[m] > 2.f * all / (float)c->sms &&
-               reach_limit_us(n[order[m]], chain[m], false) > 0.f;
+               reach_limit_us(n[order[m]], entries(m), chain[m], false) > 0.f;
       };
       int32_t sampled = 0;
       for (size_t m = 0; m < order.size(); m++)
         if (longest(m)) sampled = (int32_t)m + 1;
       if (sampled > 0 && b.a.sampled == 0) rc = band_reach(b, sampled, n[order[0]]);
-      if (rc == GSOFA_OK)
-        for (int32_t m = 0; m < sampled && m < b.a.sampled; m++)
-          if (longest(m) && b.h_reach(m).levels &&
-              ROUTE_MARGIN * traverse_us(n[order[m]], b.h_reach(m), b.a.reach_rows, false) < chain[m])
-            size[m] = 0;
+      if (rc == GSOFA_OK && sampled > 0) {
+        std::vector<char> move(order.size(), 0);
+        float before = 0.f, left = 0.f, traverse = 0.f;
+        bool alone = true;  // no other member is traversed
+        for (size_t m = 0; m < order.size(); m++) {
+          if (!size[m]) { alone = false; continue; }
+          before = std::max(before, chain[m]);
+          if ((int32_t)m < b.a.sampled && longest(m) && b.h_reach(m).levels) {
+            const float t = traverse_us(n[order[m]], b.h_reach(m), b.a.reach_rows, false);
+            move[m] = ROUTE_MARGIN * t < chain[m];
+            if (move[m]) traverse += t - traverse_base_us(0, false);
+          }
+          if (!move[m]) left = std::max(left, chain[m]);
+        }
+        if (alone) traverse += traverse_base_us(0, false);
+        if (ROUTE_MARGIN * (left + traverse) < before)
+          for (size_t m = 0; m < order.size(); m++)
+            if (move[m]) size[m] = 0;
+      }
       for (size_t m = 0; m < order.size(); m++) {
         if (size[m] == 0) rest->push_back(order[m]);
         if (size[m] == 0 || (m && size[m] < size[m - 1])) sorted = false;

@@ -159,6 +159,7 @@ __global__ void __launch_bounds__(256) band_scan_kernel(BandArgs a) {
       }
     }
     if (r < a.rows) {
+      if (a.entries && i == n - 1) a.entries[m] = re;
       a.fill[r] = (re - rb) + ((has >> lane) & 1u ? 0 : 1);
       nnz += (unsigned)(stop - rb);
       if (bad) {
@@ -223,10 +224,10 @@ __global__ void __launch_bounds__(256) band_scan_kernel(BandArgs a) {
 // that does not repeat with its structure): breadth-first search from s over vertices below
 // s, level by level, a thread (or eight) per vertex, vertices found marked in a bitmap.
 // Cut off after what the choice of the route can still use.  Bound by the latency of a
-// level: row pointers, columns, bitmap, a barrier, 1.3 us or more.  Calls that stay with the
-// elimination take 40 us more on a band of 211 (1,274 before), 100 on 317 x 293 (7,325); 32^3 and
-// dissections differ by less than their runs do.  The last CTA finds the longest stretch of
-// one matrix.
+// level: row pointers, columns, bitmap, a barrier, 1.3 us or more.  A call that stays with the
+// elimination after a search takes 100 us more on 317 x 293 (7,360), 40 for sizes alone on 27 x 25
+// x 29 (2,360); where there is none (route.cuh) nothing to be seen.  The last CTA finds the
+// longest stretch of one matrix.
 namespace {
 constexpr int REACH_THREADS = 256;
 constexpr int REACH_QUEUE = 256;    // vertices of a level: wider searches are long (a band of 211: 20 us against 45 with 1,024)
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(REACH_THREADS) band_reach_kernel(BandArgs a, b
     chain = min(panels, 4 * (panels / s_stretches + 1));
   }
   const float band = fits ? band_us(n, chain, LB, UB, counts) : 0.f;
-  const float limit = reach_limit_us(n, band, counts);
+  const float limit = reach_limit_us(n, (unsigned long long)nnz, band, counts);
   if (limit <= 0.f) return;
   const TraverseCost cost = traverse_cost(n, counts);
   const float row_ns = 1e3f * limit / (float)n;

@@ -55,6 +55,7 @@ struct BandArgs {
   int32_t group_rows;   // rows per group: a multiple of chunk
   BandCounters* ctr;
   int32_t* band;        // per matrix: largest i - j, largest j - i
+  int32_t* entries;     // per matrix of a batch: entries of A (null: one matrix, in ctr)
   BandReach* reach;     // per matrix
   int32_t sampled;      // matrices whose rows are sampled: the first ones
   int32_t reach_rows;   // rows sampled of each

@@ -98,7 +98,7 @@ extern "C" int gsofa_row_counts_noalloc(int32_t n, const int32_t* d_rowptr, cons
     if (launch_band_scan(b, st) != cudaSuccess) return GSOFA_E_CUDA;
     b.reach_rows = reach_rows(1);
     b.most_rows = n;
-    b.sampled = reach_at_once(n, true) ? 1 : 0;
+    b.sampled = n >= REACH_AT_ONCE ? 1 : 0;
     if (launch_band_reach(b, true, st) != cudaSuccess) return GSOFA_E_CUDA;
     struct { BandCounters c; unsigned char pad[64 - sizeof(BandCounters)]; BandReach reach; int32_t band[2]; } m;
     if (cudaMemcpyAsync(&m, p, sizeof(m), cudaMemcpyDeviceToHost, st) != cudaSuccess) return GSOFA_E_CUDA;
@@ -111,7 +111,8 @@ extern "C" int gsofa_row_counts_noalloc(int32_t n, const int32_t* d_rowptr, cons
     bool traverse = s.C == 0;
     if (!traverse && b.one.LB > COUNTS_WIDE_BAND)
       traverse = near_diagonal(m.c, m.band) ? n > NEAR_BAND_ORDER : n < WIDE_MIN_ORDER;
-    if (!traverse && !b.sampled && reach_limit_us(n, band_us(n, (n + 31) / 32, b.one.LB, b.one.UB, true), true) > 0.f) {
+    const float band = band_us(n, (n + 31) / 32, b.one.LB, b.one.UB, true);
+    if (!traverse && !b.sampled && reach_limit_us(n, m.c.nnz, band, true) > 0.f) {
       b.sampled = 1;
       if (launch_band_reach(b, true, st) != cudaSuccess) return GSOFA_E_CUDA;
       if (cudaMemcpyAsync(&m, p, sizeof(m), cudaMemcpyDeviceToHost, st) != cudaSuccess) return GSOFA_E_CUDA;

@@ -75,19 +75,19 @@ __host__ __device__ inline float fronts_limit_us(int n) { return ROUTE_MARGIN * 
 // us that the searches of all rows together have to stay below for a traversal to be chosen
 // instead of a band that takes `band` us (0: it does not fit) or of the search for blocks;
 // 0: not sampled.  A band is left alone where it takes less than 1.6 times what a traversal
-// takes at least: a 64 x 64 grid would pay 16 us of 340.
-__host__ __device__ inline float reach_limit_us(int n, float band, bool counts) {
+// takes at least, and below 3 ms where its rows have 3.25 entries or more (grids have 3.4 to
+// 6, chains 3): the search would take 30 us of 600 there, and 100 of 7,400 on a 317 x 293
+// grid.
+__host__ __device__ inline float reach_limit_us(int n, unsigned long long nnz, float band, bool counts) {
   const float base = traverse_base_us(n, counts);
   if (band == 0.f) return counts || n < FRONT_NEAR_ORDER ? 0.f : fronts_limit_us(n) - base;
+  if (band < 3000.f && (float)nnz >= 3.25f * (float)n) return 0.f;
   return band < 1.6f * ROUTE_MARGIN * base ? 0.f : band / ROUTE_MARGIN - base;
 }
 
-// Orders whose narrowest band is sampled (from 4,900 on, counts 800): the search is launched with
-// the scan.  Below, the scan is waited for first (25 us more, where the band is wide; 10 us
-// less where it is not sampled).
-inline bool reach_at_once(int n, bool counts) {
-  return reach_limit_us(n, band_us(n, (n + 31) / 32, 1, 0, counts), counts) > 0.f;
-}
+// Orders whose search is launched with the scan.  Below, the scan is waited for first: 25 us more
+// where there is a search, 10 less where there is none (3% of a band of order 5,000).
+constexpr int REACH_AT_ONCE = 16384;
 
 // A traversal, from the sums over `rows` sampled rows (r.levels is 0 where none were).
 inline float traverse_us(int n, const BandReach& r, int rows, bool counts) {

@@ -19,6 +19,7 @@
 // ---------------------------------------------------------------- what a scenario sets
 static int g_band_left = 0, g_band_right = 0;      // what the scan measures, for every matrix
 static long long g_reach = 1000000;                // entries that a sampled row reaches
+static int g_per_row = 3;                          // entries of a row
 static int g_blocks = 0;                           // a dissection: it falls into closed blocks
 static int g_fail_count = 0, g_fail_at = -1;       // the g_fail_at-th pool allocation from now on fails
 static std::map<void*, size_t> g_held;             // pool memory: bytes by block
@@ -163,8 +164,9 @@ cudaError_t launch_band_scan(const BandArgs& a, cudaStream_t) {
   for (int m = 0; m < a.nmats; m++) {
     a.band[2 * m] = g_band_left;
     a.band[2 * m + 1] = g_band_right;
+    if (a.entries) a.entries[m] = g_per_row * (a.mats ? a.mats[m] : a.one).n;
   }
-  a.ctr->nnz = 10 * (unsigned long long)a.rows;
+  a.ctr->nnz = (unsigned long long)g_per_row * (unsigned long long)a.rows;
   a.ctr->spread = a.ctr->nnz * (unsigned long long)(g_band_left > g_band_right ? g_band_left : g_band_right) / 2;
   return cudaSuccess;
 }
@@ -226,6 +228,7 @@ int main(int argc, char** argv) {
   g_fail_at = (int)get("fail_at", -1);
   g_blocks = (int)get("blocks", 0);
   g_reach = get("reach", 1000000);
+  g_per_row = (int)get("per_row", 3);
   gsofa_options o;
   gsofa_default_options(&o);
   o.max_ctas = (int32_t)get("max_ctas", 0);

@@ -73,7 +73,7 @@ def test_orders_near_the_largest_index(decide, below):
 def test_cap_on_ctas(decide, cap, reach, count):
     """No launch of the elimination has more CTAs than max_ctas; every matrix is eliminated once
     or traversed."""
-    lines = decide(n=9000, left=reach, right=reach, count=count, max_ctas=cap)
+    lines = decide(n=9000, left=reach, right=reach, count=count, max_ctas=cap, per_row=10)
     assert "rc 0" in lines
     got = _elim(lines)
     assert all(k * c <= cap for k, c, _, _ in got), lines
@@ -133,9 +133,9 @@ def test_no_search_for_blocks_of_short_traversals(decide):
     assert "front_blocks" in decide(n=20000, left=15000, right=15000, blocks=1, reach=20000)
 
 
-@pytest.mark.parametrize("count,traversed", [(2, 2), (20, 20), (120, 0)])
+@pytest.mark.parametrize("count,traversed", [(2, 2), (5, 5), (20, 0), (120, 0)])
 def test_batch_route_by_reach(decide, count, traversed):
-    """In a batch only bands that outlast the others are traversed."""
+    """In a batch only bands that outlast the others are traversed, where the call gains by it."""
     lines = decide(n=30000, left=200, right=200, reach=20, count=count)
     assert "rc 0" in lines and sum(k for k, _, _, _ in _elim(lines)) == count - traversed, lines
 
@@ -146,3 +146,9 @@ def test_buffers_of_abandoned_work_are_left_alone(decide, kw):
     of the first may still be under way."""
     lines = decide(n=20000, right=kw["left"], stuck=1, **kw)
     assert "first rc -5" in lines and "rc 0" in lines and "in flight" not in lines, lines
+
+
+@pytest.mark.parametrize("left,per_row,traversed", [(100, 3, True), (100, 4, False), (1500, 4, True)])
+def test_bands_of_many_entries_are_searched_where_they_take_long(decide, left, per_row, traversed):
+    lines = decide(n=15000, left=left, right=left, reach=20, per_row=per_row)
+    assert bool(_elim(lines)) == (not traversed), lines
